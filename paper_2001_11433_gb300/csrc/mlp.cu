@@ -9,8 +9,8 @@
 //
 //   k_features    per-vertex features (warp per vertex)
 //   k_mlp_fwd     inference, FP32 or BF16 weights/activations (FP32 accumulate)
-//   k_mlp_grad    forward + backward of the MSE loss over a tile of rows;
-//                 weight gradients reduced over the tile in shared memory
+//   k_mlp_grad    forward + backward of the MSE loss over tiles of rows as
+//                 register-tiled products; weight gradients summed in registers
 //   k_adam        Adam update
 #include <cuda_bf16.h>
 #include <string.h>
@@ -36,7 +36,6 @@ namespace {
 
 constexpr int kFeat = 8;
 constexpr int kMaxH = 64;
-constexpr int kRowsPerBlock = 128;
 
 struct Off {
     int64_t W1, b1, W2, b2, w3, b3, n;
@@ -221,99 +220,326 @@ __global__ void k_mlp_fwd(const float *__restrict__ wts, int H_rt, const float *
     }
 }
 
-// Forward + backward over rows idx[r0 .. r0 + cnt) (or r0.. when idx is null),
-// loss = (1/N) sum (y - t)^2.  One thread per row, kRowsPerBlock rows per block.
-__global__ void __launch_bounds__(kRowsPerBlock) k_mlp_grad(const float *__restrict__ wts, int H,
-                                                            const float *__restrict__ feat,
-                                                            const float *__restrict__ label,
-                                                            const int32_t *__restrict__ idx, int64_t r0, int64_t cnt,
-                                                            float inv_n, float *grad, float *loss) {
-    extern __shared__ float sm[];
-    const Off o = offsets(H);
-    float *sw = sm;                                // weights
-    float *sx = sw + ((o.n + 3) & ~3LL);           // x   [rows][8]
-    float *sh1 = sx + kRowsPerBlock * kFeat;       // h1  [rows][H]
-    float *sd2 = sh1 + kRowsPerBlock * H;          // dh2 [rows][H]
-    float *sd1 = sd2 + kRowsPerBlock * H;          // dh1 [rows][H]
-    for (int64_t i = threadIdx.x; i < o.n; i += blockDim.x) sw[i] = wts[i];
-    const int t = threadIdx.x;
-    const int64_t rr = (int64_t)blockIdx.x * kRowsPerBlock + t;
-    const bool valid = rr < cnt;
-    const int64_t row = valid ? (idx ? idx[r0 + rr] : r0 + rr) : 0;
-    for (int k = 0; k < kFeat; ++k) sx[t * kFeat + k] = valid ? feat[row * kFeat + k] : 0.f;
-    __syncthreads();
-    // forward
-    for (int j = 0; j < H; ++j) {
-        float a = sw[o.b1 + j];
-        for (int k = 0; k < kFeat; ++k) a = fmaf(sw[o.W1 + j * kFeat + k], sx[t * kFeat + k], a);
-        sh1[t * H + j] = fmaxf(a, 0.f);
-    }
-    float y = sw[o.b3];
-    for (int j = 0; j < H; ++j) {
-        float a = sw[o.b2 + j];
-        for (int i = 0; i < H; ++i) a = fmaf(sw[o.W2 + (int64_t)j * H + i], sh1[t * H + i], a);
-        const float h2 = fmaxf(a, 0.f);
-        sd2[t * H + j] = h2;   // h2 for now; replaced by dh2 below
-        y = fmaf(sw[o.w3 + j], h2, y);
-    }
-    const float err = valid ? (y - label[row]) : 0.f;
-    const float dy = 2.f * err * inv_n;
-    // loss
-    {
-        float l = err * err * inv_n;
-        for (int of = 16; of; of >>= 1) l += __shfl_xor_sync(0xffffffffu, l, of);
-        if ((t & 31) == 0 && l != 0.f) atomicAdd(loss, l);
-    }
-    // dh2 (and w3/b3 gradients need h2: accumulate per thread into shared later)
-    __syncthreads();
-    // dw3[j] = sum_r dy_r h2_r[j]; each thread j < H sums over rows
-    __shared__ float sdy[kRowsPerBlock];
-    sdy[t] = dy;
-    __syncthreads();
-    for (int j = t; j < H; j += blockDim.x) {
-        float a = 0.f;
-        for (int r = 0; r < kRowsPerBlock; ++r) a = fmaf(sdy[r], sd2[r * H + j], a);
-        atomicAdd(&grad[o.w3 + j], a);
-    }
-    if (t == 0) {
-        float a = 0.f;
-        for (int r = 0; r < kRowsPerBlock; ++r) a += sdy[r];
-        atomicAdd(&grad[o.b3], a);
-    }
-    __syncthreads();
-    for (int j = 0; j < H; ++j) {
-        const float h2 = sd2[t * H + j];
-        sd2[t * H + j] = h2 > 0.f ? dy * sw[o.w3 + j] : 0.f;
-    }
-    // dh1[i] = sum_j W2[j][i] dh2[j], masked by h1 > 0
-    for (int i = 0; i < H; ++i) {
-        float a = 0.f;
-        for (int j = 0; j < H; ++j) a = fmaf(sw[o.W2 + (int64_t)j * H + i], sd2[t * H + j], a);
-        sd1[t * H + i] = sh1[t * H + i] > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    // dW2[j][i] = sum_r dh2[r][j] h1[r][i]; db2[j] = sum_r dh2[r][j]
-    for (int64_t e = t; e < (int64_t)H * H; e += blockDim.x) {
-        const int j = (int)(e / H), i = (int)(e % H);
-        float a = 0.f;
-        for (int r = 0; r < kRowsPerBlock; ++r) a = fmaf(sd2[r * H + j], sh1[r * H + i], a);
-        atomicAdd(&grad[o.W2 + e], a);
-    }
-    // dW1[i][k] = sum_r dh1[r][i] x[r][k]; db1, db2
-    for (int64_t e = t; e < (int64_t)H * kFeat; e += blockDim.x) {
-        const int i = (int)(e / kFeat), k = (int)(e % kFeat);
-        float a = 0.f;
-        for (int r = 0; r < kRowsPerBlock; ++r) a = fmaf(sd1[r * H + i], sx[r * kFeat + k], a);
-        atomicAdd(&grad[o.W1 + e], a);
-    }
-    for (int j = t; j < H; j += blockDim.x) {
-        float a = 0.f, b = 0.f;
-        for (int r = 0; r < kRowsPerBlock; ++r) {
-            a += sd1[r * H + j];
-            b += sd2[r * H + j];
+// Two FP32 multiply-adds in one instruction (each rounded as fmaf).
+using f32x2 = unsigned long long;
+
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    return (f32x2)__float_as_uint(lo) | ((f32x2)__float_as_uint(hi) << 32);
+}
+
+__device__ __forceinline__ float lo2(f32x2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(f32x2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+
+// Gradient tile: kGradRows rows on kGradRows threads.  Matrices of the tile
+// are stored column by column (element [c][row]) with kRowStride floats a
+// column: 16-byte aligned columns that start 4 banks apart, so that eight
+// lanes reading 16 bytes of eight neighbouring columns hit all banks once.
+constexpr int kGradRows = 256;
+constexpr int kRowStride = kGradRows + 4;
+
+// Shared memory of k_mlp_grad (floats).  Weights are held as pairs (w, w),
+// ready for fma2 against two rows.
+template <int HP> struct GradSmem {
+    static constexpr int W1d = 0;                               // [8][2 HP]   (w, w) of W1[c][k] at [k][2c]
+    static constexpr int W2Td = W1d + kFeat * 2 * HP;           // [HP][2 HP]  W2[c][k] at [k][2c]
+    static constexpr int W2d = W2Td + HP * 2 * HP;              // [HP][2 HP]  W2[k][c] at [k][2c]
+    static constexpr int b1 = W2d + HP * 2 * HP;
+    static constexpr int b2 = b1 + HP;
+    static constexpr int w3 = b2 + HP;
+    static constexpr int xT = w3 + HP;                          // [8][rows]
+    static constexpr int h1T = xT + kFeat * kRowStride;         // [HP][rows]: h1, later dh1
+    static constexpr int dT = h1T + HP * kRowStride;            // [HP][rows]: dh2
+    static constexpr int part = dT + HP * kRowStride;           // [2][rows]: halves of y
+    static constexpr int dy = part + 2 * kGradRows;             // [rows]
+    static constexpr int n = dy + kGradRows;
+};
+
+// acc (8 rows as 4 pairs, NC columns) += A^T B over k < K: A[k][row] from
+// `a` (this thread's rows), B[k][2c] as (b, b) pairs from `b` (its columns).
+template <int NC, int V, int HP>
+__device__ __forceinline__ void grad_mm(f32x2 (&acc)[4][NC], const float *a, const float *b, int K) {
+#pragma unroll 4
+    for (int k = 0; k < K; ++k) {
+        f32x2 ar[4], br[NC];
+        const ulonglong2 a0 = *reinterpret_cast<const ulonglong2 *>(a + k * kRowStride);
+        const ulonglong2 a1 = *reinterpret_cast<const ulonglong2 *>(a + k * kRowStride + kGradRows / 2);
+        ar[0] = a0.x;
+        ar[1] = a0.y;
+        ar[2] = a1.x;
+        ar[3] = a1.y;
+#pragma unroll
+        for (int c = 0; c < NC; c += 2) {
+            const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(b + k * 2 * HP + 2 * ((c / V) * 8 * V + c % V));
+            br[c] = t.x;
+            br[c + 1] = t.y;
         }
-        atomicAdd(&grad[o.b1 + j], a);
-        atomicAdd(&grad[o.b2 + j], b);
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int p = 0; p < 4; ++p) acc[p][c] = fma2(ar[p], br[c], acc[p][c]);
+    }
+}
+
+// this thread's 8 rows of column c of a tile matrix
+__device__ __forceinline__ void grad_put(float *col, const f32x2 (&v)[4]) {
+    *reinterpret_cast<ulonglong2 *>(col) = make_ulonglong2(v[0], v[1]);
+    *reinterpret_cast<ulonglong2 *>(col + kGradRows / 2) = make_ulonglong2(v[2], v[3]);
+}
+
+// Forward + backward over rows idx[r0 .. r0 + cnt) (or r0.. when idx is null),
+// loss = (1/N) sum (y - t)^2, hidden width H padded with zero weights to HP.
+// Bound: FP32 multiply-adds (28,000 flops a row).  Persistent blocks, one an
+// SM, take tiles of 256 rows; each layer, forward and backward, is a register-
+// tiled product (8 rows x HP/8 columns a thread, 32 packed multiply-adds for
+// six 16-byte shared-memory loads at HP = 64), and every weight gradient is
+// summed over the block's rows in registers and added to memory once.  One
+// thread per row with serial dot products (columns of one row in one bank)
+// took 6.47 ms for 200,000 rows at H = 64; a call with this kernel takes
+// 0.20 ms, 28 TFLOP/s.
+template <int HP>
+__global__ void __launch_bounds__(kGradRows, 1) k_mlp_grad(const float *__restrict__ wts, int H,
+                                                           const float *__restrict__ feat,
+                                                           const float *__restrict__ label,
+                                                           const int32_t *__restrict__ idx, int64_t r0, int64_t cnt,
+                                                           float inv_n, float *grad, float *loss) {
+    using S = GradSmem<HP>;
+    constexpr int NC = HP / 8;             // columns a thread
+    constexpr int V = NC < 4 ? NC : 4;     // consecutive ones among them
+    constexpr int NJ = HP / 16;            // W2 gradient: NJ x NJ entries a thread
+    constexpr int KT = HP / 32 > 0 ? HP / 32 : 1;   // W1 gradient: entries a thread
+    extern __shared__ __align__(16) float sm[];
+    const Off o = offsets(H);
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (int i = t; i < HP * HP; i += kGradRows) {
+        const int j = i / HP, k = i % HP;
+        const float w = j < H && k < H ? wts[o.W2 + (int64_t)j * H + k] : 0.f;
+        *reinterpret_cast<float2 *>(sm + S::W2Td + k * 2 * HP + 2 * j) = make_float2(w, w);
+        *reinterpret_cast<float2 *>(sm + S::W2d + j * 2 * HP + 2 * k) = make_float2(w, w);
+    }
+    for (int i = t; i < HP * kFeat; i += kGradRows) {
+        const int j = i / kFeat, k = i % kFeat;
+        const float w = j < H ? wts[o.W1 + i] : 0.f;
+        *reinterpret_cast<float2 *>(sm + S::W1d + k * 2 * HP + 2 * j) = make_float2(w, w);
+    }
+    for (int i = t; i < HP; i += kGradRows) {
+        sm[S::b1 + i] = i < H ? wts[o.b1 + i] : 0.f;
+        sm[S::b2 + i] = i < H ? wts[o.b2 + i] : 0.f;
+        sm[S::w3 + i] = i < H ? wts[o.w3 + i] : 0.f;
+    }
+    const float b3 = wts[o.b3];
+    // rows 4 tr .. 4 tr + 3 and the same of the tile's second half; columns
+    // (c / V) * 8 V + tc V + c % V
+    const int tr = (warp & 3) * 8 + (lane & 7), tc = (warp >> 2) * 4 + (lane >> 3);
+    auto column = [&](int c) { return (c / V) * 8 * V + tc * V + c % V; };
+    // W2 gradient entries (tj + 16 a, ti + 16 b)
+    const int tj = (warp & 1) * 8 + (lane & 7), ti = (warp >> 1) * 4 + (lane >> 3);
+    f32x2 gW2[NJ][NJ], gW1[KT];
+    float gb1[NC], gb2[NC], gw3[NC], gb3 = 0.f, gl = 0.f;
+#pragma unroll
+    for (int a = 0; a < NJ; ++a)
+#pragma unroll
+        for (int b = 0; b < NJ; ++b) gW2[a][b] = 0ULL;
+#pragma unroll
+    for (int a = 0; a < KT; ++a) gW1[a] = 0ULL;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) gb1[c] = gb2[c] = gw3[c] = 0.f;
+    const int64_t tiles = (cnt + kGradRows - 1) / kGradRows;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t rr = tile * kGradRows + t;
+        const bool valid = rr < cnt;
+        const int64_t row = valid ? (idx ? idx[r0 + rr] : r0 + rr) : 0;
+#pragma unroll
+        for (int k = 0; k < kFeat; ++k) sm[S::xT + k * kRowStride + t] = valid ? feat[row * kFeat + k] : 0.f;
+        __syncthreads();
+        f32x2 acc[4][NC];
+        // ---- h1 = relu(W1 x + b1)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const float b = sm[S::b1 + column(c)];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) acc[p][c] = pack2(b, b);
+        }
+        grad_mm<NC, V, HP>(acc, sm + S::xT + tr * 4, sm + S::W1d + 2 * V * tc, kFeat);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            f32x2 v[4];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) v[p] = pack2(fmaxf(lo2(acc[p][c]), 0.f), fmaxf(hi2(acc[p][c]), 0.f));
+            grad_put(sm + S::h1T + column(c) * kRowStride + tr * 4, v);
+        }
+        __syncthreads();
+        // ---- h2 = relu(W2 h1 + b2), kept in registers; y = w3 h2 + b3
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const float b = sm[S::b2 + column(c)];
+#pragma unroll
+            for (int p = 0; p < 4; ++p) acc[p][c] = pack2(b, b);
+        }
+        grad_mm<NC, V, HP>(acc, sm + S::h1T + tr * 4, sm + S::W2Td + 2 * V * tc, HP);
+        {
+            float y[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) y[q] = 0.f;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const float w = sm[S::w3 + column(c)];
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const float a = fmaxf(lo2(acc[p][c]), 0.f), b = fmaxf(hi2(acc[p][c]), 0.f);
+                    acc[p][c] = pack2(a, b);
+                    y[2 * p] = fmaf(w, a, y[2 * p]);
+                    y[2 * p + 1] = fmaf(w, b, y[2 * p + 1]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                y[q] += __shfl_xor_sync(0xffffffffu, y[q], 8);
+                y[q] += __shfl_xor_sync(0xffffffffu, y[q], 16);
+            }
+            if (lane < 8) {
+                float *half = sm + S::part + (warp >> 2) * kGradRows + tr * 4;
+                *reinterpret_cast<float4 *>(half) = make_float4(y[0], y[1], y[2], y[3]);
+                *reinterpret_cast<float4 *>(half + kGradRows / 2) = make_float4(y[4], y[5], y[6], y[7]);
+            }
+        }
+        __syncthreads();
+        {
+            const float y = sm[S::part + t] + sm[S::part + kGradRows + t] + b3;
+            const float err = valid ? y - label[row] : 0.f;
+            const float d = 2.f * err * inv_n;
+            gl += err * err * inv_n;
+            gb3 += d;
+            sm[S::dy + t] = d;
+        }
+        __syncthreads();
+        // ---- dh2 = dy w3 where h2 > 0; gradients of w3 and b2
+        {
+            const float4 d0 = *reinterpret_cast<const float4 *>(sm + S::dy + tr * 4);
+            const float4 d1 = *reinterpret_cast<const float4 *>(sm + S::dy + tr * 4 + kGradRows / 2);
+            const float d[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const float w = sm[S::w3 + column(c)];
+                f32x2 v[4];
+                float sw = 0.f, sb = 0.f;
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const float a = lo2(acc[p][c]), b = hi2(acc[p][c]);
+                    sw = fmaf(d[2 * p], a, sw);
+                    sw = fmaf(d[2 * p + 1], b, sw);
+                    const float da = a > 0.f ? d[2 * p] * w : 0.f, db = b > 0.f ? d[2 * p + 1] * w : 0.f;
+                    sb += da;
+                    sb += db;
+                    v[p] = pack2(da, db);
+                }
+                gw3[c] += sw;
+                gb2[c] += sb;
+                grad_put(sm + S::dT + column(c) * kRowStride + tr * 4, v);
+            }
+        }
+        __syncthreads();
+        // ---- dh1 = W2^T dh2 where h1 > 0 (kept in registers); gradient of b1
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int p = 0; p < 4; ++p) acc[p][c] = 0ULL;
+        grad_mm<NC, V, HP>(acc, sm + S::dT + tr * 4, sm + S::W2d + 2 * V * tc, HP);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const float *h = sm + S::h1T + column(c) * kRowStride + tr * 4;
+            const float4 h0 = *reinterpret_cast<const float4 *>(h);
+            const float4 h1 = *reinterpret_cast<const float4 *>(h + kGradRows / 2);
+            const float hv[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+            float sb = 0.f;
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const float a = hv[2 * p] > 0.f ? lo2(acc[p][c]) : 0.f;
+                const float b = hv[2 * p + 1] > 0.f ? hi2(acc[p][c]) : 0.f;
+                sb += a;
+                sb += b;
+                acc[p][c] = pack2(a, b);
+            }
+            gb1[c] += sb;
+        }
+        // ---- gradient of W2: sum over rows of dh2[j] h1[i], even and odd rows apart
+#pragma unroll 2
+        for (int r = 0; r < kGradRows; r += 4) {
+            ulonglong2 dj[NJ], hi[NJ];
+#pragma unroll
+            for (int a = 0; a < NJ; ++a) {
+                dj[a] = *reinterpret_cast<const ulonglong2 *>(sm + S::dT + (tj + 16 * a) * kRowStride + r);
+                hi[a] = *reinterpret_cast<const ulonglong2 *>(sm + S::h1T + (ti + 16 * a) * kRowStride + r);
+            }
+#pragma unroll
+            for (int a = 0; a < NJ; ++a)
+#pragma unroll
+                for (int b = 0; b < NJ; ++b) {
+                    gW2[a][b] = fma2(dj[a].x, hi[b].x, gW2[a][b]);
+                    gW2[a][b] = fma2(dj[a].y, hi[b].y, gW2[a][b]);
+                }
+        }
+        __syncthreads();   // h1 is read by now: dh1 takes its place
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const f32x2 v[4] = {acc[0][c], acc[1][c], acc[2][c], acc[3][c]};
+            grad_put(sm + S::h1T + column(c) * kRowStride + tr * 4, v);
+        }
+        __syncthreads();
+        // ---- gradient of W1: sum over rows of dh1[i] x[k]
+        if (t / HP * KT < kFeat) {
+            const float *d = sm + S::h1T + (t % HP) * kRowStride, *x = sm + S::xT + (t / HP) * KT * kRowStride;
+#pragma unroll 4
+            for (int r = 0; r < kGradRows; r += 4) {
+                const ulonglong2 dv = *reinterpret_cast<const ulonglong2 *>(d + r);
+#pragma unroll
+                for (int a = 0; a < KT; ++a) {
+                    const ulonglong2 xv = *reinterpret_cast<const ulonglong2 *>(x + a * kRowStride + r);
+                    gW1[a] = fma2(dv.x, xv.x, gW1[a]);
+                    gW1[a] = fma2(dv.y, xv.y, gW1[a]);
+                }
+            }
+        }
+        __syncthreads();   // x and dh1 are read: the next tile may overwrite them
+    }
+    // ---- the block's sums to memory
+#pragma unroll
+    for (int a = 0; a < NJ; ++a)
+#pragma unroll
+        for (int b = 0; b < NJ; ++b) {
+            const int j = tj + 16 * a, i = ti + 16 * b;
+            if (j < H && i < H) atomicAdd(&grad[o.W2 + (int64_t)j * H + i], lo2(gW2[a][b]) + hi2(gW2[a][b]));
+        }
+    if (t / HP * KT < kFeat && t % HP < H)
+#pragma unroll
+        for (int a = 0; a < KT; ++a)
+            atomicAdd(&grad[o.W1 + (int64_t)(t % HP) * kFeat + t / HP * KT + a], lo2(gW1[a]) + hi2(gW1[a]));
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+#pragma unroll
+        for (int of = 1; of < 8; of <<= 1) {
+            gb1[c] += __shfl_xor_sync(0xffffffffu, gb1[c], of);
+            gb2[c] += __shfl_xor_sync(0xffffffffu, gb2[c], of);
+            gw3[c] += __shfl_xor_sync(0xffffffffu, gw3[c], of);
+        }
+        if ((lane & 7) == 0 && column(c) < H) {
+            atomicAdd(&grad[o.b1 + column(c)], gb1[c]);
+            atomicAdd(&grad[o.b2 + column(c)], gb2[c]);
+            atomicAdd(&grad[o.w3 + column(c)], gw3[c]);
+        }
+    }
+    for (int of = 16; of; of >>= 1) {
+        gl += __shfl_xor_sync(0xffffffffu, gl, of);
+        gb3 += __shfl_xor_sync(0xffffffffu, gb3, of);
+    }
+    if (lane == 0) {
+        if (gl != 0.f) atomicAdd(loss, gl);
+        atomicAdd(&grad[o.b3], gb3);
     }
 }
 
@@ -339,11 +565,6 @@ __global__ void k_keys_to_idx(const uint64_t *keys, int32_t n, int32_t idb, int3
     const uint64_t mask = (1ULL << idb) - 1;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         idx[i] = (int32_t)(keys[i] & mask);
-}
-
-size_t grad_smem(int H) {
-    const Off o = offsets(H);
-    return (size_t)(((o.n + 3) & ~3LL) + kRowsPerBlock * kFeat + 3 * kRowsPerBlock * H) * 4;
 }
 
 }  // namespace
@@ -386,13 +607,22 @@ mce_status model_predict(const mce_model *m, const float *feat, int32_t rows, in
     return MCE_OK;
 }
 
+template <int HP>
+static mce_status grad_launch_hp(const mce_model *m, const float *feat, const float *label, const int32_t *idx,
+                                 int64_t r0, int64_t cnt, float inv_n, float *loss, cudaStream_t s) {
+    const size_t smem = (size_t)GradSmem<HP>::n * 4;
+    MCE_CUDA(cudaFuncSetAttribute(k_mlp_grad<HP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int64_t tiles = (cnt + kGradRows - 1) / kGradRows;
+    const unsigned blocks = (unsigned)(tiles < num_sms() ? tiles : num_sms());
+    MCE_LAUNCH(k_mlp_grad<HP>, blocks, kGradRows, smem, s, m->w, m->H, feat, label, idx, r0, cnt, inv_n, m->g, loss);
+    return MCE_OK;
+}
+
 static mce_status grad_launch(const mce_model *m, const float *feat, const float *label, const int32_t *idx,
                               int64_t r0, int64_t cnt, float inv_n, float *loss, cudaStream_t s) {
-    const size_t smem = grad_smem(m->H);
-    MCE_CUDA(cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const unsigned blocks = (unsigned)((cnt + kRowsPerBlock - 1) / kRowsPerBlock);
-    MCE_LAUNCH(k_mlp_grad, blocks, kRowsPerBlock, smem, s, m->w, m->H, feat, label, idx, r0, cnt, inv_n, m->g, loss);
-    return MCE_OK;
+    if (m->H <= 16) return grad_launch_hp<16>(m, feat, label, idx, r0, cnt, inv_n, loss, s);
+    if (m->H <= 32) return grad_launch_hp<32>(m, feat, label, idx, r0, cnt, inv_n, loss, s);
+    return grad_launch_hp<kMaxH>(m, feat, label, idx, r0, cnt, inv_n, loss, s);
 }
 
 }  // namespace mce

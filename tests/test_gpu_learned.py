@@ -75,6 +75,22 @@ def test_loss_and_gradient_match_reference(gpu_lib):
     assert np.abs(grad_g - grad_r).max() <= 1e-4 * scale
 
 
+@pytest.mark.parametrize("hidden", [1, 5, 16, 17, 32, 33, 64])
+@pytest.mark.parametrize("rows", [1, 255, 256, 257, 256 * 152 + 13])
+def test_gradient_tiles_and_widths(gpu_lib, hidden, rows):
+    """Row tiles of 256 on 152 blocks, widths padded to 16, 32 and 64.  Sums of
+    `rows` FP32 terms: error below 1e-5 of the largest component."""
+    mce = gpu_lib
+    rng = np.random.default_rng(rows + hidden)
+    X = (rng.random((rows, 8)) * 4).astype(np.float32)
+    t = rng.normal(2.0, 1.0, rows).astype(np.float32)
+    m = mce.Model(hidden, seed=hidden)
+    loss_g, grad_g = m.loss_grad(_f(X), _f(t))
+    loss_r, grad_r = mlp.loss_grad(m.get().astype(np.float64), X.astype(np.float64), t.astype(np.float64), hidden)
+    assert loss_g == pytest.approx(loss_r, rel=1e-5)
+    assert np.abs(grad_g - grad_r).max() <= 1e-5 * max(np.abs(grad_r).max(), 1e-3)
+
+
 def test_prediction_fp32_and_bf16(gpu_lib):
     """BF16 inference: 8 significant bits per weight and activation; two
     64-term layers keep the error within a few percent of the output scale."""
