@@ -106,6 +106,30 @@ def test_prediction_fp32_and_bf16(gpu_lib):
     assert np.abs(y16 - ref).max() <= 0.03 * scale
 
 
+@pytest.mark.parametrize("hidden", [1, 16, 17, 33, 64])
+@pytest.mark.parametrize("rows", [1, 15, 17, 64 * 456 + 9])
+def test_bf16_prediction_tiles_and_widths(gpu_lib, hidden, rows):
+    """Tiles of 16 rows a warp, widths padded to 16, 32 and 64, against the same
+    roundings in float64.  Sums of at most 64 FP32 terms move a rounded value by
+    one step of 2^-8 at most where it lies next to a boundary."""
+    mce = gpu_lib
+    import torch
+    bf = lambda a: torch.from_numpy(a).float().bfloat16().double().numpy()  # noqa: E731
+    X = (np.random.default_rng(rows + hidden).random((rows, 8)) * 4 - 1).astype(np.float32)
+    m = mce.Model(hidden, seed=hidden)
+    p = bf(m.get().astype(np.float64))
+    cut = np.cumsum([hidden * 8, hidden, hidden * hidden, hidden, hidden, 1])
+    W1, b1, W2, b2, w3, b3 = (p[a:b] for a, b in zip([0, *cut[:-1]], cut))
+    W1, W2 = W1.reshape(hidden, 8), W2.reshape(hidden, hidden)
+    h1 = bf(np.maximum(bf(X.astype(np.float64)) @ W1.T + b1, 0))
+    h2 = bf(np.maximum(h1 @ W2.T + b2, 0))
+    ref = h2 @ w3 + b3
+    y = m.predict(_f(X), bf16=True).cpu().numpy()
+    scale = np.abs(h2 * w3).sum(1) + np.abs(b3) + 1e-3
+    assert (np.abs(y - ref) <= 2 ** -7 * scale).all()
+    assert np.linalg.norm(y - ref) <= 1e-3 * max(np.linalg.norm(ref), 1e-3)
+
+
 def test_training_on_recorded_node_counts(gpu_lib):
     """Train on log(1 + tree nodes) recorded by the search (degeneracy rank).
     Gain over the method without the network: on held-out vertices the network
