@@ -242,8 +242,7 @@ mce_status mce_batched_create(const mce_graph *g, const int32_t *graph_ptr, int3
     // rank, Γ+ lists, trivial subproblems, order
     MCE_TRY(b->rank.alloc(((size_t)n + 1) * 4, s));
     MCE_TRY(compute_rank(g, opts, s, b->rank.as<int32_t>()));
-    int64_t up_nnz = 0;
-    MCE_TRY(build_up_lists(g, b->rank.as<int32_t>(), s, b->up_ptr, b->up_col, &up_nnz));
+    MCE_TRY(build_up_lists(g, b->rank.as<int32_t>(), s, b->up_ptr, b->up_col));
     for (DevBuf *d : {&b->out0, &b->out}) MCE_TRY(d->alloc(OUT_WORDS * 8, s));
     for (DevBuf *d : {&b->gcount0, &b->ghash0, &b->gcount, &b->ghash, &b->gnodes}) MCE_TRY(d->alloc((size_t)k * 8, s));
     MCE_TRY(b->status.alloc((size_t)k * 4, s));

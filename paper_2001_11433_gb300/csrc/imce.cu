@@ -1297,8 +1297,7 @@ mce_status batch_cliques(imce_state *S, const mce_graph *gp, Batch &bt, DevBuf &
     MCE_TRY(drank.alloc((size_t)n * 4, s));
     MCE_TRY(vertex_key(gp, MCE_RANK_DEGREE, s, dkey.as<int64_t>()));
     MCE_TRY(rank_from_key_i64(dkey.as<int64_t>(), n, gp->id_bits, s, drank.as<int32_t>()));
-    int64_t up_nnz = 0;
-    MCE_TRY(build_up_lists(gp, drank.as<int32_t>(), s, up_ptr, up_col, &up_nnz));
+    MCE_TRY(build_up_lists(gp, drank.as<int32_t>(), s, up_ptr, up_col));
     DevBuf okeys, otmp, order, reqb, nout;
     MCE_TRY(okeys.alloc((size_t)rho * 8, s));
     MCE_TRY(otmp.alloc((size_t)rho * 8, s));

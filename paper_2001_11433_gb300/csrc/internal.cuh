@@ -128,9 +128,8 @@ mce_status vertex_key(const mce_graph *g, int32_t kind, cudaStream_t s, int64_t 
 mce_status rank_from_key_i64(const int64_t *key, int32_t n, int32_t id_bits, cudaStream_t s, int32_t *rank);
 // Same for float keys (higher float = higher rank; NaN not allowed).
 mce_status rank_from_key_f32(const float *key, int32_t n, int32_t id_bits, cudaStream_t s, int32_t *rank);
-// Higher-ranked neighbour lists: up_ptr int32[n+1], up_col int32[...] (sorted by id).
-mce_status build_up_lists(const mce_graph *g, const int32_t *rank, cudaStream_t s, DevBuf &up_ptr, DevBuf &up_col,
-                          int64_t *up_nnz);
+// Higher-ranked neighbour lists: up_ptr int32[n+1], up_col int32[nnz / 2 + 4] (sorted by id).
+mce_status build_up_lists(const mce_graph *g, const int32_t *rank, cudaStream_t s, DevBuf &up_ptr, DevBuf &up_col);
 // Features (mce_features).
 mce_status features(const mce_graph *g, int32_t kind, cudaStream_t s, float *feat);
 int32_t model_feature_kind(const mce_model *m);

@@ -407,8 +407,7 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
         MCE_TRY(compute_rank(g, o, s, rank.as<int32_t>()));
     }
     MCE_CUDA(cudaEventRecord(e1, s));
-    int64_t up_nnz = 0;
-    MCE_TRY(build_up_lists(g, rank.as<int32_t>(), s, up_ptr, up_col, &up_nnz));
+    MCE_TRY(build_up_lists(g, rank.as<int32_t>(), s, up_ptr, up_col));
     const float *costp = nullptr;
     const mce_model *cost_model = o->split_model ? o->split_model : (o->order_by_model ? o->model : nullptr);
     DevBuf heavy;

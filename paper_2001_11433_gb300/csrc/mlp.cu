@@ -684,8 +684,7 @@ mce_status features(const mce_graph *g, int32_t kind, cudaStream_t s, float *fea
     MCE_TRY(vertex_key(g, MCE_RANK_TRIANGLE, s, tri.as<int64_t>()));
     MCE_TRY(vertex_key(g, MCE_RANK_DEGREE, s, deg.as<int64_t>()));
     MCE_TRY(rank_from_key_i64(deg.as<int64_t>(), n, g->id_bits, s, drank.as<int32_t>()));
-    int64_t nnz = 0;
-    MCE_TRY(build_up_lists(g, drank.as<int32_t>(), s, up_ptr, up_col, &nnz));
+    MCE_TRY(build_up_lists(g, drank.as<int32_t>(), s, up_ptr, up_col));
     MCE_LAUNCH(k_features, grid_for((int64_t)n * 32, 256), 256, 0, s, g->row_ptr, g->col, core.as<int64_t>(),
                tri.as<int64_t>(), up_ptr.as<int32_t>(), n, feat);
     return MCE_OK;

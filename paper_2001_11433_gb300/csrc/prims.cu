@@ -73,16 +73,54 @@ __global__ void k_scan_apply(const T *in, T *out, int64_t n, const T *block_offs
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1) out[n] = run;
 }
 
+// Scans of up to this many items run in one launch of one block: three
+// launches of the tiled scan cost more than the one block takes.
+constexpr int64_t kScanOne = 16384;
+constexpr int kScanOneThreads = 1024;
+
+template <class T>
+__global__ void __launch_bounds__(kScanOneThreads) k_scan_one(const T *in, T *out, int32_t n) {
+    __shared__ T ws[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (n + kScanOneThreads - 1) / kScanOneThreads;
+    const int i0 = threadIdx.x * per, i1 = i0 + per < n ? i0 + per : n;
+    T s = 0;
+    for (int i = i0; i < i1; ++i) s += in[i];
+    T incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) ws[warp] = incl;
+    __syncthreads();
+    const T w = ws[lane];
+    T wi = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const T y = __shfl_up_sync(0xffffffffu, wi, o);
+        if (lane >= o) wi += y;
+    }
+    T run = __shfl_sync(0xffffffffu, wi - w, warp) + incl - s;
+    const T total = __shfl_sync(0xffffffffu, wi, 31);
+    for (int i = i0; i < i1; ++i) {
+        const T x = in[i];
+        out[i] = run;
+        run += x;
+    }
+    if (threadIdx.x == 0) out[n] = total;
+}
+
 template <class T>
 mce_status exclusive_scan(const T *in, T *out, int64_t n, cudaStream_t s) {
     if (n <= 0) {
         return cuda_status(cudaMemsetAsync(out, 0, sizeof(T), s), "scan memset");
     }
-    const int64_t tiles = (n + kScanTile - 1) / kScanTile;
-    if (tiles == 1) {
-        MCE_LAUNCH(k_scan_apply<T>, 1, kScanThreads, 0, s, in, out, n, (const T *)nullptr);
+    if (n <= kScanOne) {
+        MCE_LAUNCH(k_scan_one<T>, 1, kScanOneThreads, 0, s, in, out, (int32_t)n);
         return MCE_OK;
     }
+    const int64_t tiles = (n + kScanTile - 1) / kScanTile;
     DevBuf sums;
     MCE_TRY(sums.alloc((size_t)(tiles + 1) * sizeof(T), s));
     MCE_LAUNCH(k_scan_reduce<T>, (unsigned)tiles, kScanThreads, 0, s, in, n, sums.as<T>());

@@ -197,6 +197,50 @@ def test_rmat13_per_vertex_exact(gpu_lib, kind, split):
     assert np.array_equal(u64(pv[2]), o.per_vertex["nodes"])
 
 
+def awkward_graph(shape):
+    """Row layouts at the edges of the entry-balanced kernels: long runs of empty
+    rows (before, between, after), one row far longer than a segment, entry
+    counts at and next to segment boundaries."""
+    rng = np.random.default_rng(sum(map(ord, shape)))
+    if shape == "gaps":                       # 400 vertices 300 ids apart
+        u, v = graphgen.er(400, 0.05, 3)
+        return 400 * 300, u * 300 + 7, v * 300 + 7
+    if shape == "tail":
+        u, v = graphgen.er(100, 0.3, 4)
+        return 9000, u, v
+    if shape == "lead":
+        u, v = graphgen.er(100, 0.3, 5)
+        return 9000, u + 8900, v + 8900
+    if shape == "hub":                        # one row of 6,000 entries, sparse edges below it
+        a, b = rng.integers(1, 6001, 4000), rng.integers(1, 6001, 4000)
+        return 6001, np.concatenate([np.zeros(6000, np.int64), a]), np.concatenate([np.arange(1, 6001), b])
+    if shape == "pairs64":                    # 128 entries: exactly one segment of 128
+        return 128, np.arange(0, 128, 2), np.arange(1, 128, 2)
+    if shape == "pairs65":
+        return 200, np.arange(0, 130, 2), np.arange(1, 130, 2)
+    return 3, np.array([0]), np.array([2])    # "one": a single edge around an empty row
+
+
+AWKWARD = ["gaps", "tail", "lead", "hub", "pairs64", "pairs65", "one"]
+
+
+@pytest.mark.parametrize("kind", ["degree", "degen", "triangle"])
+@pytest.mark.parametrize("shape", AWKWARD)
+def test_awkward_rows_per_vertex_exact(gpu_lib, kind, shape):
+    mce = gpu_lib
+    n, u, v = awkward_graph(shape)
+    og = O.Graph(n, u.astype(np.int32), v.astype(np.int32))
+    rk = O.rank(og, kind)
+    o = O.parmce(og, rk, per_vertex=True)
+    g = gpu_graph(mce, n, u, v)
+    assert np.array_equal(mce.rank(g, rank=kind).cpu().numpy(), rk)
+    pv = per_vertex_bufs(n)
+    r = mce.enumerate_cliques(g, rank=kind, per_vertex=pv)
+    assert_same_summary(r, o)
+    for k, name in enumerate(("count", "hash", "nodes")):
+        assert np.array_equal(u64(pv[k]), o.per_vertex[name])
+
+
 @pytest.mark.parametrize("shape", [(2, 16), (3, 64), (4, 256)])
 def test_handover_stress_keeps_every_subproblem(gpu_lib, shape):
     """Hand-overs every few nodes (ParTTT prefix rule, Algorithm 3) from wide
