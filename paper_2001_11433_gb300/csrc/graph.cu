@@ -238,14 +238,6 @@ __global__ void k_scatter_rank(const uint64_t *sorted, int32_t n, int32_t idb, i
         rank[sorted[i] & mask] = (int32_t)i;
 }
 
-__global__ void k_max_i64(const int64_t *a, int32_t n, unsigned long long *mx) {
-    unsigned long long m = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned long long)max(a[v], (int64_t)0));
-    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(mx, m);
-}
-
 // ------------------------------------------------------------------ Γ+ lists
 
 // The CSR entries are cut into segments of `len` entries (a multiple of 32),
@@ -442,7 +434,7 @@ mce_status build_csr(const int32_t *u, const int32_t *v, int64_t m, int32_t n, c
         g_last_error = "mce_graph_create: vertex id outside [0, n)";
         return MCE_EINVAL;
     }
-    MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), k, 2 * B, s));
+    MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), k, 0, 2 * B, s));
     const uint64_t sentinel = (B >= 32) ? ~0ULL : ((1ULL << (2 * B)) - 1);
     MCE_LAUNCH(k_flag_unique, grid_for(k, 256), 256, 0, s, keys.as<uint64_t>(), k, sentinel, flag.as<int32_t>());
     MCE_TRY(exclusive_scan_i32(flag.as<int32_t>(), flag.as<int32_t>(), k, s));
@@ -501,7 +493,8 @@ static mce_status triangle_counts(const mce_graph *g, cudaStream_t s, int64_t *k
     MCE_TRY(deg.alloc((size_t)n * sizeof(int64_t), s));
     MCE_TRY(rank.alloc((size_t)n * sizeof(int32_t), s));
     MCE_LAUNCH(k_degree_key, grid_for(n, 256), 256, 0, s, g->row_ptr, n, deg.as<int64_t>());
-    MCE_TRY(rank_from_key_i64(deg.as<int64_t>(), n, g->id_bits, s, rank.as<int32_t>()));
+    MCE_TRY(rank_from_key_i64(deg.as<int64_t>(), n, g->id_bits, vertex_key_bits(g, MCE_RANK_DEGREE), s,
+                              rank.as<int32_t>()));
     MCE_TRY(build_up_lists(g, rank.as<int32_t>(), s, up_ptr, up_col));
     MCE_CUDA(cudaMemsetAsync(key, 0, (size_t)n * sizeof(int64_t), s));
     MCE_LAUNCH(k_triangles, grid_for((int64_t)n * 32, 256), 256, 0, s, up_ptr.as<int32_t>(), up_col.as<int32_t>(), n,
@@ -525,24 +518,30 @@ mce_status vertex_key(const mce_graph *g, int32_t kind, cudaStream_t s, int64_t 
     }
 }
 
-mce_status rank_from_key_i64(const int64_t *key, int32_t n, int32_t id_bits, cudaStream_t s, int32_t *rank) {
+int32_t vertex_key_bits(const mce_graph *g, int32_t kind) {
+    const uint64_t m = (uint64_t)(g->nnz / 2);
+    if (kind == MCE_RANK_DEGEN) {   // a k-core has at least k (k + 1) / 2 edges
+        int32_t b = 1;
+        while (b < 31 && ((1ULL << b) * (1ULL << b)) <= 2 * m) ++b;
+        return b;
+    }
+    if (kind == MCE_RANK_TRIANGLE) return bits_for(m);   // each triangle at v has its own edge opposite v
+    const uint64_t d = g->n > 0 ? (uint64_t)(g->n - 1) : 0;
+    return bits_for(d < m ? d : m);
+}
+
+mce_status rank_from_key_i64(const int64_t *key, int32_t n, int32_t id_bits, int32_t key_bits, cudaStream_t s,
+                             int32_t *rank) {
     if (n == 0) return MCE_OK;
-    DevBuf keys, tmp, mx;
+    DevBuf keys, tmp;
     MCE_TRY(keys.alloc((size_t)n * sizeof(uint64_t), s));
     MCE_TRY(tmp.alloc((size_t)n * sizeof(uint64_t), s));
-    MCE_TRY(mx.alloc(sizeof(unsigned long long), s));
-    MCE_CUDA(cudaMemsetAsync(mx.p, 0, sizeof(unsigned long long), s));
-    MCE_LAUNCH(k_max_i64, grid_for(n, 256), 256, 0, s, key, n, mx.as<unsigned long long>());
-    unsigned long long hmx = 0;
-    MCE_CUDA(cudaMemcpyAsync(&hmx, mx.p, sizeof(hmx), cudaMemcpyDeviceToHost, s));
-    MCE_CUDA(cudaStreamSynchronize(s));
-    const int32_t bits = bits_for(hmx) + id_bits;
-    if (bits > 64) {
+    if (key_bits + id_bits > 64) {
         g_last_error = "rank_from_key: key too large";
         return MCE_EINVAL;
     }
     MCE_LAUNCH(k_rank_keys_i64, grid_for(n, 256), 256, 0, s, key, n, id_bits, keys.as<uint64_t>());
-    MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), n, bits, s));
+    MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), n, id_bits, id_bits + key_bits, s));
     MCE_LAUNCH(k_scatter_rank, grid_for(n, 256), 256, 0, s, keys.as<uint64_t>(), n, id_bits, rank);
     return MCE_OK;
 }
@@ -553,7 +552,7 @@ mce_status rank_from_key_f32(const float *key, int32_t n, int32_t id_bits, cudaS
     MCE_TRY(keys.alloc((size_t)n * sizeof(uint64_t), s));
     MCE_TRY(tmp.alloc((size_t)n * sizeof(uint64_t), s));
     MCE_LAUNCH(k_rank_keys_f32, grid_for(n, 256), 256, 0, s, key, n, id_bits, keys.as<uint64_t>());
-    MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), n, 32 + id_bits, s));
+    MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), n, id_bits, 32 + id_bits, s));
     MCE_LAUNCH(k_scatter_rank, grid_for(n, 256), 256, 0, s, keys.as<uint64_t>(), n, id_bits, rank);
     return MCE_OK;
 }

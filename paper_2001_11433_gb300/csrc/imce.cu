@@ -167,7 +167,7 @@ __global__ void k_edge_order_keys(const int32_t *row_ptr2, const int32_t *eu, co
         const int32_t c = min(du, dv);
         r = max(r, (unsigned long long)bk_ws_words(c, c, BK_IMCE));
         cm = max(cm, (unsigned long long)c);
-        keys[i] = ((uint64_t)((1u << 30) - 1 - (uint32_t)c) << IB) | (uint64_t)i;
+        keys[i] = ((uint64_t)heavy_first_key((uint64_t)(uint32_t)c) << IB) | (uint64_t)i;
     }
     for (int o = 16; o; o >>= 1) {
         r = max(r, __shfl_xor_sync(FULL, r, o));
@@ -1212,7 +1212,7 @@ mce_status canonical_batch(imce_state *S, const int32_t *u, const int32_t *v, in
     if (k > 0) {
         MCE_LAUNCH(k_batch_keys, grid_for(k, 256), 256, 0, s, u, v, k, n, g->row_ptr, g->col, B, IB,
                    (int32_t)deletion, keys.as<uint64_t>(), bad.as<int32_t>());
-        MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), k, 64, s));
+        MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), k, IB, IB + 2 * B, s));
         MCE_LAUNCH(k_first_arrival, grid_for(k, 256), 256, 0, s, keys.as<uint64_t>(), k, IB, keep.as<int32_t>());
         MCE_TRY(exclusive_scan_i32(keep.as<int32_t>(), keep.as<int32_t>(), k, s));
         int32_t hb = 0;
@@ -1241,7 +1241,7 @@ mce_status canonical_batch(imce_state *S, const int32_t *u, const int32_t *v, in
     MCE_CUDA(cudaMemsetAsync(bt.hdeg.p, 0, ((size_t)n + 1) * 4, s));
     MCE_LAUNCH(k_h_keys, grid_for(rho, 256), 256, 0, s, bt.eu.as<int32_t>(), bt.ev.as<int32_t>(), rho, B, IBr,
                hkeys.as<uint64_t>(), bt.hdeg.as<int32_t>());
-    MCE_TRY(radix_sort_u64(hkeys.as<uint64_t>(), htmp.as<uint64_t>(), 2 * (int64_t)rho, 2 * B + IBr, s));
+    MCE_TRY(radix_sort_u64(hkeys.as<uint64_t>(), htmp.as<uint64_t>(), 2 * (int64_t)rho, IBr, IBr + 2 * B, s));
     MCE_LAUNCH(k_h_fill, grid_for(2 * (int64_t)rho, 256), 256, 0, s, hkeys.as<uint64_t>(), 2 * (int64_t)rho, B, IBr,
                bt.h_adj.as<int32_t>(), bt.h_idx.as<int32_t>());
     MCE_TRY(exclusive_scan_i32(bt.hdeg.as<int32_t>(), bt.h_ptr.as<int32_t>(), n, s));
@@ -1296,7 +1296,8 @@ mce_status batch_cliques(imce_state *S, const mce_graph *gp, Batch &bt, DevBuf &
     MCE_TRY(dkey.alloc((size_t)n * 8, s));
     MCE_TRY(drank.alloc((size_t)n * 4, s));
     MCE_TRY(vertex_key(gp, MCE_RANK_DEGREE, s, dkey.as<int64_t>()));
-    MCE_TRY(rank_from_key_i64(dkey.as<int64_t>(), n, gp->id_bits, s, drank.as<int32_t>()));
+    MCE_TRY(rank_from_key_i64(dkey.as<int64_t>(), n, gp->id_bits, vertex_key_bits(gp, MCE_RANK_DEGREE), s,
+                              drank.as<int32_t>()));
     MCE_TRY(build_up_lists(gp, drank.as<int32_t>(), s, up_ptr, up_col));
     DevBuf okeys, otmp, order, reqb, nout;
     MCE_TRY(okeys.alloc((size_t)rho * 8, s));
@@ -1306,7 +1307,7 @@ mce_status batch_cliques(imce_state *S, const mce_graph *gp, Batch &bt, DevBuf &
     MCE_CUDA(cudaMemsetAsync(reqb.p, 0, 16, s));
     MCE_LAUNCH(k_edge_order_keys, grid_for(rho, 256), 256, 0, s, gp->row_ptr, bt.eu.as<int32_t>(), bt.ev.as<int32_t>(),
                rho, IBr, okeys.as<uint64_t>(), reqb.as<unsigned long long>());
-    MCE_TRY(radix_sort_u64(okeys.as<uint64_t>(), otmp.as<uint64_t>(), rho, 30 + IBr, s));
+    MCE_TRY(radix_sort_u64(okeys.as<uint64_t>(), otmp.as<uint64_t>(), rho, IBr, IBr + 16, s));
     MCE_LAUNCH(k_keys_low, grid_for(rho, 256), 256, 0, s, okeys.as<uint64_t>(), rho, IBr, order.as<int32_t>());
     unsigned long long reqc[2] = {0, 0};
     MCE_CUDA(cudaMemcpyAsync(reqc, reqb.p, 16, cudaMemcpyDeviceToHost, s));

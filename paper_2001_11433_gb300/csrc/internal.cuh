@@ -114,9 +114,11 @@ inline unsigned grid_for(int64_t work, int32_t per_block) {
 // (in == out) is allowed.
 mce_status exclusive_scan_i32(const int32_t *in, int32_t *out, int64_t n, cudaStream_t s);
 mce_status exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, cudaStream_t s);
-// Ascending LSD radix sort of uint64 keys on their low `bits` bits (higher
-// bits must be zero).  keys is sorted in place; tmp has n entries.
-mce_status radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int32_t bits, cudaStream_t s);
+// Stable ascending LSD radix sort of uint64 keys by their bits [lo, hi).  A
+// payload in the low bits that ascends with the position needs no pass: keys
+// (value << lo) | index sort by value, then index.  keys is sorted in place;
+// tmp has n entries.
+mce_status radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int32_t lo, int32_t hi, cudaStream_t s);
 
 // ------------------------------------------------------------------ graph kernels (graph.cu)
 
@@ -124,8 +126,11 @@ mce_status radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int32_t bits
 mce_status build_csr(const int32_t *u, const int32_t *v, int64_t m, int32_t n, cudaStream_t s, mce_graph *g);
 // Per-vertex keys (int64[n]).
 mce_status vertex_key(const mce_graph *g, int32_t kind, cudaStream_t s, int64_t *key);
-// rank[v] = position of (key[v], v); key values < 2^(64 - id_bits).
-mce_status rank_from_key_i64(const int64_t *key, int32_t n, int32_t id_bits, cudaStream_t s, int32_t *rank);
+// rank[v] = position of (key[v], v); 0 <= key values < 2^key_bits.
+mce_status rank_from_key_i64(const int64_t *key, int32_t n, int32_t id_bits, int32_t key_bits, cudaStream_t s,
+                             int32_t *rank);
+// bits of the largest value that vertex_key can give for this graph
+int32_t vertex_key_bits(const mce_graph *g, int32_t kind);
 // Same for float keys (higher float = higher rank; NaN not allowed).
 mce_status rank_from_key_f32(const float *key, int32_t n, int32_t id_bits, cudaStream_t s, int32_t *rank);
 // Higher-ranked neighbour lists: up_ptr int32[n+1], up_col int32[nnz / 2 + 4] (sorted by id).
@@ -152,6 +157,14 @@ __device__ __forceinline__ uint64_t vertex_hash(int32_t v, uint64_t seed) {
 // H(K) from sum_{v in K} h(v) and |K|
 __device__ __forceinline__ uint64_t clique_hash_from_sum(uint64_t hsum, uint32_t size) {
     return fmix64(hsum + (uint64_t)size * kGolden);
+}
+
+// Order keys of subproblems, heaviest first, in kOrderBits bits: the sign-free
+// exponent and 8 mantissa bits of the estimate, inverted.  Estimates within
+// 0.4 % of each other keep the order of their ids; the sort takes two passes.
+constexpr int32_t kOrderBits = 16;
+__device__ __forceinline__ uint32_t heavy_first_key(uint64_t est) {
+    return 0xffffu - (__float_as_uint((float)est) >> 15);
 }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {

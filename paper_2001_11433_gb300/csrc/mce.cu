@@ -67,13 +67,12 @@ __global__ void k_mce_prepass(const int32_t *__restrict__ row_ptr, const int32_t
                 // descending predicted cost: invert the order-preserving float map
                 uint32_t b = __float_as_uint(cost[v]);
                 b ^= (b >> 31) ? 0xffffffffu : 0x80000000u;
-                k = ((uint64_t)(~b) << idb) | (uint64_t)v;
+                k = ((uint64_t)((~b) >> 16) << idb) | (uint64_t)v;
             } else {
                 // expected cost: the search grows with c^2 at least, the build
                 // with the neighbourhood (each of the w local vertices is scanned)
                 const uint64_t est = (uint64_t)c * (uint64_t)c + 64ULL * (uint64_t)w;
-                const uint64_t cap = (1ULL << (63 - idb)) - 1;
-                k = ((cap - (est < cap ? est : cap)) << idb) | (uint64_t)v;
+                k = ((uint64_t)heavy_first_key(est) << idb) | (uint64_t)v;
             }
             keys[v] = k;
             req = max(req, (unsigned long long)bk_ws_words(w, c, BK_MCE));
@@ -201,7 +200,7 @@ mce_status launch_order(const int32_t *flag_scan, const uint64_t *keys, int32_t 
                         uint64_t *tmp2, int32_t *order, cudaStream_t s) {
     uint64_t *act = tmp2, *act_tmp = tmp2 + n_act;
     MCE_LAUNCH(k_gather_active, grid_for(n, 256), 256, 0, s, flag_scan, keys, n, act);
-    MCE_TRY(radix_sort_u64(act, act_tmp, n_act, 64, s));
+    MCE_TRY(radix_sort_u64(act, act_tmp, n_act, idb, idb + kOrderBits, s));
     MCE_LAUNCH(k_order_from_keys, grid_for(n_act, 256), 256, 0, s, act, n_act, idb, order);
     return MCE_OK;
 }
@@ -317,7 +316,7 @@ mce_status compute_rank(const mce_graph *g, const mce_opts *o, cudaStream_t s, i
             DevBuf key;
             MCE_TRY(key.alloc((size_t)n * 8, s));
             MCE_TRY(vertex_key(g, o->rank_kind, s, key.as<int64_t>()));
-            return rank_from_key_i64(key.as<int64_t>(), n, g->id_bits, s, rank);
+            return rank_from_key_i64(key.as<int64_t>(), n, g->id_bits, vertex_key_bits(g, o->rank_kind), s, rank);
         }
         default:
             g_last_error = "unknown rank kind";
@@ -401,7 +400,7 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
             MCE_LAUNCH(k_whole_init, grid_for(n, 256), 256, 0, s, n, wkey.as<int64_t>(), wmask.as<uint8_t>());
             MCE_LAUNCH(k_whole_mark, 64, 256, 0, s, g->row_ptr, g->col, best.as<unsigned long long>(),
                        wkey.as<int64_t>(), wmask.as<uint8_t>());
-            MCE_TRY(rank_from_key_i64(wkey.as<int64_t>(), n, g->id_bits, s, rank.as<int32_t>()));
+            MCE_TRY(rank_from_key_i64(wkey.as<int64_t>(), n, g->id_bits, 1, s, rank.as<int32_t>()));
         }
     } else {
         MCE_TRY(compute_rank(g, o, s, rank.as<int32_t>()));
@@ -484,7 +483,7 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
         MCE_TRY(order.alloc((size_t)n_act * 4, s));
         uint64_t *act = tmp.as<uint64_t>(), *act_tmp = act + n_act;
         MCE_LAUNCH(k_gather_active, grid_for(n, 256), 256, 0, s, flag.as<int32_t>(), keys.as<uint64_t>(), n, act);
-        MCE_TRY(radix_sort_u64(act, act_tmp, n_act, 64, s));
+        MCE_TRY(radix_sort_u64(act, act_tmp, n_act, idb, idb + kOrderBits, s));
         MCE_LAUNCH(k_order_from_keys, grid_for(n_act, 256), 256, 0, s, act, n_act, idb, order.as<int32_t>());
         BkParams P{};
         P.mode = BK_MCE;

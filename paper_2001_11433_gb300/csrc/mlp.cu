@@ -683,7 +683,8 @@ mce_status features(const mce_graph *g, int32_t kind, cudaStream_t s, float *fea
     MCE_TRY(vertex_key(g, MCE_RANK_DEGEN, s, core.as<int64_t>()));
     MCE_TRY(vertex_key(g, MCE_RANK_TRIANGLE, s, tri.as<int64_t>()));
     MCE_TRY(vertex_key(g, MCE_RANK_DEGREE, s, deg.as<int64_t>()));
-    MCE_TRY(rank_from_key_i64(deg.as<int64_t>(), n, g->id_bits, s, drank.as<int32_t>()));
+    MCE_TRY(rank_from_key_i64(deg.as<int64_t>(), n, g->id_bits, vertex_key_bits(g, MCE_RANK_DEGREE), s,
+                              drank.as<int32_t>()));
     MCE_TRY(build_up_lists(g, drank.as<int32_t>(), s, up_ptr, up_col));
     MCE_LAUNCH(k_features, grid_for((int64_t)n * 32, 256), 256, 0, s, g->row_ptr, g->col, core.as<int64_t>(),
                tri.as<int64_t>(), up_ptr.as<int32_t>(), n, feat);
@@ -855,7 +856,7 @@ mce_status mce_model_train(mce_model *m, const float *feat, const float *label, 
     for (int32_t ep = 0; ep < epochs; ++ep) {
         MCE_LAUNCH(k_perm_keys, grid_for(rows, 256), 256, 0, s, rows, seed + (uint64_t)ep * 7919, idb,
                    keys.as<uint64_t>());
-        MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), rows, 64, s));
+        MCE_TRY(radix_sort_u64(keys.as<uint64_t>(), tmp.as<uint64_t>(), rows, idb, 64, s));
         MCE_LAUNCH(k_keys_to_idx, grid_for(rows, 256), 256, 0, s, keys.as<uint64_t>(), rows, idb, idx.as<int32_t>());
         for (int64_t r0 = 0; r0 < rows; r0 += batch) {
             const int64_t cnt = (r0 + batch <= rows) ? batch : rows - r0;

@@ -131,65 +131,229 @@ mce_status exclusive_scan(const T *in, T *out, int64_t n, cudaStream_t s) {
 
 // ------------------------------------------------------------------ radix sort
 
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;
-constexpr int kSortTile = kSortThreads * kSortItems;
 constexpr int kRadix = 256;
 
-// counts[d * tiles + t] = keys of tile t whose digit is d
-__global__ void k_radix_hist(const uint64_t *keys, int64_t n, int shift, int32_t *counts, int32_t tiles) {
-    __shared__ int32_t h[kRadix];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortTile;
-#pragma unroll 4
-    for (int r = 0; r < kSortItems; ++r) {
-        int64_t i = base + (int64_t)r * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & (kRadix - 1)], 1);
-    }
-    __syncthreads();
-    counts[(int64_t)threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];
+// Rank of this lane's key among the keys of its digit that its warp has seen
+// (earlier rounds, then earlier lanes of this round); digit = kRadix for a
+// lane without a key.  wcnt: the warp's digit counters.
+__device__ __forceinline__ int radix_rank(int32_t *wcnt, uint32_t digit) {
+    const uint32_t peers = __match_any_sync(0xffffffffu, digit);
+    const int before = __popc(peers & lanemask_lt());
+    const int seen = digit < kRadix ? wcnt[digit] : 0;
+    __syncwarp();
+    if (before == 0 && digit < kRadix) wcnt[digit] = seen + __popc(peers);
+    __syncwarp();
+    return seen + before;
 }
 
-// Stable scatter.  Items of a tile are visited in index order: round r covers
-// [r*256, r*256+256), and inside a round warps then lanes go in order.  A
-// digit's position = tile offset (from the scanned histogram) + items of the
-// same digit in earlier rounds + in earlier warps of this round + in earlier
-// lanes of this warp (match_any gives the lanes holding the same digit).
-__global__ void k_radix_scatter(const uint64_t *in, uint64_t *out, int64_t n, int shift, const int32_t *offsets,
-                                int32_t tiles) {
-    constexpr int W = kSortThreads / 32;
-    __shared__ int32_t base[kRadix];
-    __shared__ int32_t wcnt[W][kRadix];
-    const int tid = threadIdx.x, warp = tid >> 5;
-    base[tid] = offsets[(int64_t)tid * tiles + blockIdx.x];
-    const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
-    for (int r = 0; r < kSortItems; ++r) {
+// Exclusive scan over the first 256 threads of a block (one value a digit).
+__device__ __forceinline__ int32_t digit_scan(int32_t x, int32_t *ws) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t incl = x;
 #pragma unroll
-        for (int j = 0; j < W; ++j) wcnt[j][tid] = 0;
-        __syncthreads();
-        const int64_t i = tile0 + (int64_t)r * kSortThreads + tid;
-        const bool valid = i < n;
-        const uint64_t key = valid ? in[i] : 0;
-        const uint32_t digit = valid ? (uint32_t)((key >> shift) & (kRadix - 1)) : kRadix;
-        const uint32_t peers = __match_any_sync(0xffffffffu, digit);
-        const int rank = __popc(peers & lanemask_lt());
-        if (valid && rank == 0) wcnt[warp][digit] = __popc(peers);
-        __syncthreads();
-        {
-            int32_t run = base[tid];
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (warp < kRadix / 32 && lane == 31) ws[warp] = incl;
+    __syncthreads();
+    int32_t r = incl - x;
+    for (int w = 0; w < warp && w < kRadix / 32; ++w) r += ws[w];
+    __syncthreads();
+    return r;
+}
+
+// All passes of a small sort in one block, the keys in registers and, between
+// passes, in shared memory.  Three launches a pass cost more than the work
+// below a few thousand keys.
+constexpr int kOneThreads = 1024;
+constexpr int kOneItems = 8;
+constexpr int64_t kOneKeys = kOneThreads * kOneItems;
+constexpr int kOneWarps = kOneThreads / 32;
+constexpr size_t kOneSmem = kOneKeys * 8 + (size_t)kOneWarps * kRadix * 4 + kRadix * 4 + 64;
+
+__global__ void __launch_bounds__(kOneThreads) k_radix_one(uint64_t *keys, int32_t n, int lo, int hi, int width) {
+    extern __shared__ __align__(16) unsigned char smem_one[];
+    uint64_t *sk = reinterpret_cast<uint64_t *>(smem_one);
+    int32_t *cnt = reinterpret_cast<int32_t *>(sk + kOneKeys);   // [warp][digit]
+    int32_t *start = cnt + kOneWarps * kRadix;
+    int32_t *ws = start + kRadix;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int rounds = (n + kOneThreads - 1) / kOneThreads;   // a warp holds 32 * rounds consecutive keys
+    uint64_t key[kOneItems];
+    int rank[kOneItems];
+    const int w0 = warp * 32 * rounds;
 #pragma unroll
-            for (int j = 0; j < W; ++j) {
-                int32_t c = wcnt[j][tid];
-                wcnt[j][tid] = run;
+    for (int r = 0; r < kOneItems; ++r) {
+        const int i = w0 + r * 32 + lane;
+        key[r] = r < rounds && i < n ? keys[i] : 0ULL;
+    }
+    for (int shift = lo; shift < hi; shift += width) {
+        const uint32_t mask = (1u << (hi - shift < width ? hi - shift : width)) - 1u;
+        for (int i = t; i < kOneWarps * kRadix; i += kOneThreads) cnt[i] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kOneItems; ++r)
+            if (r < rounds) {
+                const bool valid = w0 + r * 32 + lane < n;
+                rank[r] = radix_rank(cnt + warp * kRadix, valid ? (uint32_t)(key[r] >> shift) & mask : kRadix);
+            }
+        __syncthreads();
+        int32_t run = 0;
+        if (t < kRadix)
+            for (int w = 0; w < kOneWarps; ++w) {
+                const int32_t c = cnt[w * kRadix + t];
+                cnt[w * kRadix + t] = run;
                 run += c;
             }
-            base[tid] = run;
+        const int32_t base = digit_scan(run, ws);
+        if (t < kRadix) start[t] = base;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kOneItems; ++r)
+            if (r < rounds && w0 + r * 32 + lane < n) {
+                const uint32_t d = (uint32_t)(key[r] >> shift) & mask;
+                sk[start[d] + cnt[warp * kRadix + d] + rank[r]] = key[r];
+            }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kOneItems; ++r) {
+            const int i = w0 + r * 32 + lane;
+            if (r < rounds && i < n) key[r] = sk[i];
         }
         __syncthreads();
-        if (valid) out[wcnt[warp][digit] + rank] = key;
+    }
+#pragma unroll
+    for (int r = 0; r < kOneItems; ++r) {
+        const int i = w0 + r * 32 + lane;
+        if (r < rounds && i < n) keys[i] = key[r];
+    }
+}
+
+// Larger sorts: per pass the digit counts of every tile, their scan along each
+// digit's row, and a stable scatter.  Bound: HBM (24 B a key and pass).
+constexpr int kSortThreads = 256;
+constexpr int kSortWarps = kSortThreads / 32;
+
+// counts[d * tiles + t] = keys of tile t whose digit is d
+template <int ITEMS>
+__global__ void __launch_bounds__(kSortThreads) k_radix_hist(const uint64_t *__restrict__ keys, int64_t n, int shift,
+                                                             uint32_t mask, int32_t *counts, int32_t tiles) {
+    __shared__ int32_t h[kSortWarps][kRadix];   // per warp: a frequent digit would serialise one counter
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) h[w][t] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * (kSortThreads * ITEMS);
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int64_t i = base + (int64_t)r * kSortThreads + t;
+        if (i < n) atomicAdd(&h[t >> 5][(uint32_t)(keys[i] >> shift) & mask], 1);
+    }
+    __syncthreads();
+    int32_t s = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) s += h[w][t];
+    counts[(int64_t)t * tiles + blockIdx.x] = s;
+}
+
+// row d of the counts: exclusive scan over the tiles in place, total[d] = its sum
+__global__ void __launch_bounds__(kSortThreads) k_radix_rows(int32_t *counts, int32_t tiles, int32_t *total) {
+    __shared__ int32_t ws[kRadix / 32];
+    __shared__ int32_t last;
+    int32_t *row = counts + (int64_t)blockIdx.x * tiles;
+    int32_t carry = 0;
+    for (int32_t i0 = 0; i0 < tiles; i0 += kSortThreads) {
+        const int32_t i = i0 + threadIdx.x;
+        const int32_t x = i < tiles ? row[i] : 0;
+        const int32_t r = digit_scan(x, ws);
+        if (i < tiles) row[i] = carry + r;
+        if (threadIdx.x == kSortThreads - 1) last = r + x;
+        __syncthreads();
+        carry += last;
         __syncthreads();
     }
+    if (threadIdx.x == 0) total[blockIdx.x] = carry;
+}
+
+// Stable scatter: a warp ranks its consecutive keys, the block adds the
+// counters of the warps before it, and the tile is put in digit order in
+// shared memory first, so that a digit's keys leave as one run.
+template <int ITEMS>
+__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const uint64_t *__restrict__ in,
+                                                                uint64_t *__restrict__ out, int64_t n, int shift,
+                                                                uint32_t mask, const int32_t *__restrict__ rows,
+                                                                int32_t tiles, const int32_t *__restrict__ total) {
+    constexpr int TILE = kSortThreads * ITEMS;
+    __shared__ uint64_t sk[TILE];
+    __shared__ int32_t cnt[kSortWarps][kRadix];
+    __shared__ int32_t start[kRadix], dst[kRadix], ws[kRadix / 32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t base = (int64_t)blockIdx.x * TILE;
+    const int have = (int)(n - base < TILE ? n - base : TILE);
+    uint64_t key[ITEMS];
+    int rank[ITEMS];
+    const int w0 = warp * 32 * ITEMS;
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int i = w0 + r * 32 + lane;
+        key[r] = i < have ? in[base + i] : 0ULL;
+    }
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) cnt[w][t] = 0;
+    const int32_t digit0 = digit_scan(total[t], ws);   // keys with a smaller digit
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r)
+        rank[r] = radix_rank(cnt[warp], w0 + r * 32 + lane < have ? (uint32_t)(key[r] >> shift) & mask : kRadix);
+    __syncthreads();
+    int32_t run = 0;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; ++w) {
+        const int32_t c = cnt[w][t];
+        cnt[w][t] = run;
+        run += c;
+    }
+    const int32_t s0 = digit_scan(run, ws);
+    start[t] = s0;
+    dst[t] = digit0 + rows[(int64_t)t * tiles + blockIdx.x] - s0;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r)
+        if (w0 + r * 32 + lane < have) {
+            const uint32_t d = (uint32_t)(key[r] >> shift) & mask;
+            sk[start[d] + cnt[warp][d] + rank[r]] = key[r];
+        }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int j = r * kSortThreads + t;
+        if (j < have) {
+            const uint64_t k = sk[j];
+            out[dst[(uint32_t)(k >> shift) & mask] + j] = k;
+        }
+    }
+}
+
+template <int ITEMS>
+mce_status radix_passes(uint64_t *keys, uint64_t *tmp, int64_t n, int lo, int hi, int width, cudaStream_t s) {
+    constexpr int TILE = kSortThreads * ITEMS;
+    const int32_t tiles = (int32_t)((n + TILE - 1) / TILE);
+    DevBuf counts;
+    MCE_TRY(counts.alloc(((size_t)kRadix * tiles + kRadix) * sizeof(int32_t), s));
+    int32_t *rows = counts.as<int32_t>(), *total = rows + (size_t)kRadix * tiles;
+    uint64_t *src = keys, *dst = tmp;
+    for (int shift = lo; shift < hi; shift += width) {
+        const uint32_t mask = (1u << (hi - shift < width ? hi - shift : width)) - 1u;
+        MCE_LAUNCH(k_radix_hist<ITEMS>, tiles, kSortThreads, 0, s, src, n, shift, mask, rows, tiles);
+        MCE_LAUNCH(k_radix_rows, kRadix, kSortThreads, 0, s, rows, tiles, total);
+        MCE_LAUNCH(k_radix_scatter<ITEMS>, tiles, kSortThreads, 0, s, src, dst, n, shift, mask, rows, tiles, total);
+        uint64_t *t = src;
+        src = dst;
+        dst = t;
+    }
+    if (src != keys) MCE_CUDA(cudaMemcpyAsync(keys, src, (size_t)n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
+    return MCE_OK;
 }
 
 }  // namespace
@@ -202,27 +366,22 @@ mce_status exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, cudaSt
     return exclusive_scan<int64_t>(in, out, n, s);
 }
 
-mce_status radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int32_t bits, cudaStream_t s) {
-    if (n <= 1) return MCE_OK;
+mce_status radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int32_t lo, int32_t hi, cudaStream_t s) {
+    if (n <= 1 || hi <= lo) return MCE_OK;
     if (n >= (int64_t)1 << 31) {
         g_last_error = "radix_sort_u64: too many keys";
         return MCE_EINVAL;
     }
-    const int32_t tiles = (int32_t)((n + kSortTile - 1) / kSortTile);
-    DevBuf counts;
-    MCE_TRY(counts.alloc((size_t)kRadix * tiles * sizeof(int32_t) + sizeof(int32_t), s));
-    uint64_t *src = keys, *dst = tmp;
-    int passes = 0;
-    for (int shift = 0; shift < bits; shift += 8, ++passes) {
-        MCE_LAUNCH(k_radix_hist, tiles, kSortThreads, 0, s, src, n, shift, counts.as<int32_t>(), tiles);
-        MCE_TRY(exclusive_scan_i32(counts.as<int32_t>(), counts.as<int32_t>(), (int64_t)kRadix * tiles, s));
-        MCE_LAUNCH(k_radix_scatter, tiles, kSortThreads, 0, s, src, dst, n, shift, counts.as<int32_t>(), tiles);
-        uint64_t *t = src;
-        src = dst;
-        dst = t;
+    const int passes = (hi - lo + 7) / 8;
+    const int width = (hi - lo + passes - 1) / passes;   // equal digits: shorter rows of counters
+    if (n <= kOneKeys) {
+        MCE_CUDA(cudaFuncSetAttribute(k_radix_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOneSmem));
+        MCE_LAUNCH(k_radix_one, 1, kOneThreads, kOneSmem, s, keys, (int32_t)n, lo, hi, width);
+        return MCE_OK;
     }
-    if (src != keys) MCE_CUDA(cudaMemcpyAsync(keys, src, (size_t)n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
-    return MCE_OK;
+    // tiles of 4,096 keys once they fill the GPU, else of 1,024
+    if (n >= (int64_t)num_sms() * kSortThreads * 16) return radix_passes<16>(keys, tmp, n, lo, hi, width, s);
+    return radix_passes<4>(keys, tmp, n, lo, hi, width, s);
 }
 
 }  // namespace mce

@@ -197,6 +197,27 @@ def test_rmat13_per_vertex_exact(gpu_lib, kind, split):
     assert np.array_equal(u64(pv[2]), o.per_vertex["nodes"])
 
 
+@pytest.mark.parametrize("n", [2, 31, 33, 1023, 1025, 2049, 8191, 8192, 8193, 12289, 152 * 4096 - 1, 152 * 4096 + 1])
+def test_rank_is_the_stable_order_of_the_keys(gpu_lib, n):
+    """One-block sort up to 8,192 keys, tiles of 1,024, then of 4,096 keys."""
+    mce = gpu_lib
+    rng = np.random.default_rng(n)
+    hub = np.zeros(n // 3, np.int64)                       # one frequent and one rare digit
+    u = np.concatenate([rng.integers(0, n, 2 * n), hub])
+    v = np.concatenate([rng.integers(0, n, 2 * n), rng.integers(0, n, len(hub))])
+    keep = u != v
+    key = np.unique(np.minimum(u, v)[keep] * n + np.maximum(u, v)[keep])
+    d = np.bincount(np.concatenate([key // n, key % n]), minlength=n)
+    expect = np.empty(n, np.int64)
+    expect[np.lexsort((np.arange(n), d))] = np.arange(n)
+    g = gpu_graph(mce, n, u, v)
+    row, col = g.csr()
+    assert np.array_equal(np.diff(row), d)
+    a, b = np.concatenate([key // n, key % n]), np.concatenate([key % n, key // n])
+    assert np.array_equal(col, b[np.lexsort((b, a))])
+    assert np.array_equal(mce.rank(g, rank="degree").cpu().numpy(), expect)
+
+
 def awkward_graph(shape):
     """Row layouts at the edges of the entry-balanced kernels: long runs of empty
     rows (before, between, after), one row far longer than a segment, entry
