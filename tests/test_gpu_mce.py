@@ -111,6 +111,39 @@ def test_vertex_keys_and_ranks(gpu_lib, case):
         assert np.array_equal(mce.rank(g, rank=kind).cpu().numpy(), O.rank(og, kind)), kind
 
 
+def core_graph(shape):
+    rng = np.random.default_rng(11)
+    if shape == "path":                       # one removal step after the other
+        return 3000, np.arange(2999), np.arange(1, 3000)
+    if shape == "tree":
+        return 4000, np.arange(1, 4000), rng.integers(0, np.arange(1, 4000))
+    if shape == "cliques":                    # K_2..K_70 chained by single edges: every value once
+        us, vs, base = [], [], 0
+        for k in range(2, 71):
+            i, j = np.triu_indices(k, 1)
+            us += [i + base, [base]]
+            vs += [j + base, [base - 1 if base else 1]]
+            base += k
+        return base, np.concatenate(us), np.concatenate(vs)
+    hubs = {"deg32": 32, "deg33": 33, "deg1024": 1024, "deg1025": 1025}[shape]
+    n = 3 * hubs + 50                         # three hubs of that degree over a sparse rest, two of them joined
+    leaves = np.arange(3, n)
+    u = np.concatenate([np.full(hubs, 0), np.full(hubs, 1), np.full(hubs, 2), rng.choice(leaves, 2 * n), [0]])
+    v = np.concatenate([rng.permutation(leaves)[:hubs], rng.permutation(leaves)[:hubs], leaves[:hubs],
+                        rng.choice(leaves, 2 * n), [1]])
+    return n, u, v
+
+
+@pytest.mark.parametrize("shape", ["path", "tree", "cliques", "deg32", "deg33", "deg1024", "deg1025"])
+def test_core_numbers_by_degree_class(gpu_lib, shape):
+    """Lanes, warps and blocks a vertex (degrees up to 32, up to 1024, above)."""
+    mce = gpu_lib
+    n, u, v = core_graph(shape)
+    og = O.Graph(n, np.asarray(u, np.int32), np.asarray(v, np.int32))
+    key = mce.vertex_key(gpu_graph(mce, n, u, v), "degen").cpu().numpy()
+    assert np.array_equal(key, O.core_numbers(og).astype(np.int64))
+
+
 # ---------------------------------------------------------------- enumeration: small exact cases
 
 def _check_lists(mce, n, pairs, expect, **kw):
