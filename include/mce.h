@@ -174,13 +174,14 @@ typedef struct {
     int32_t subproblems;          /* vertices with a non-trivial subproblem */
     float ms_rank;                /* ranking time (key + sort), device time */
     float ms_enum;                /* enumeration time, device time */
-    float ms_search;              /* device time of the search kernel alone */
+    float ms_search;              /* device time of the subproblem builds and the search */
     uint64_t word_ops;            /* algorithmic 32-bit word operations of the search: per
                                      tree node (|cand|+|fini|)*ceil(|cand|/32) AND+POPC for
                                      the pivot and 2*ceil((|cand|+|fini|)/32) per child
                                      searched, plus |K| per clique emitted */
     int64_t incomplete;           /* subproblems abandoned by subproblem_budget */
-    uint64_t stats[8];            /* search kernel, summed over warps: [0] ns building subproblems,
+    uint64_t stats[8];            /* search kernel, summed over warps: [0] ns building subproblems
+                                     beyond the build cache (the others are built before),
                                      [1] ns searching, [2] ns waiting for work, [3] builds,
                                      [4] handed-over pieces run, [5] largest busy ns of one
                                      warp, [6] warps, [7] ns from the last subproblem claim to

@@ -23,8 +23,10 @@ __global__ void k_check_disjoint(const int32_t *row_ptr, const int32_t *col, con
             if (graph_of[col[e]] != graph_of[x]) atomicOr(bad, 1);
 }
 
+// next_build (may be null): back to 0 for the plan's next run
 __global__ void k_graph_status(const unsigned long long *nodes, int32_t k, uint64_t budget, int32_t *status,
-                               int32_t *any) {
+                               int32_t *any, unsigned long long *next_build) {
+    if (next_build && blockIdx.x == 0 && threadIdx.x == 0) *next_build = 0ULL;
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < k; g += (int64_t)gridDim.x * blockDim.x) {
         const bool over = budget && nodes[g] > budget;
         status[g] = over ? MCE_EBUDGET : MCE_OK;
@@ -84,7 +86,7 @@ extern "C" mce_status mce_enumerate_batched(const mce_graph *g, const int32_t *g
     if (st != MCE_OK && st != MCE_EOVERFLOW) return st;
     MCE_CUDA(cudaMemsetAsync(bad.p, 0, 4, s));
     MCE_LAUNCH(k_graph_status, grid_for(k, 256), 256, 0, s, gnodes.as<unsigned long long>(), k, opts->node_budget,
-               status, bad.as<int32_t>());
+               status, bad.as<int32_t>(), (unsigned long long *)nullptr);
     MCE_CUDA(cudaMemcpyAsync(&hbad, bad.p, 4, cudaMemcpyDeviceToHost, s));
     MCE_CUDA(cudaStreamSynchronize(s));
     if (hbad) total->complete = 0;
@@ -99,18 +101,6 @@ extern "C" mce_status mce_enumerate_batched(const mce_graph *g, const int32_t *g
 // into a CUDA graph on its first call and replayed afterwards.  The tuner
 // times launch shapes (resident blocks per SM, hand-over interval) on runs
 // whose per-graph budget is cut, and keeps the fastest.
-
-namespace mce {
-namespace {
-
-__global__ void k_plan_reset(unsigned long long *seq, int64_t qcap, unsigned long long *ctl, unsigned long long pending) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < qcap; i += (int64_t)gridDim.x * blockDim.x)
-        seq[i] = (unsigned long long)i;
-    if (blockIdx.x == 0 && threadIdx.x < CTL_WORDS) ctl[threadIdx.x] = threadIdx.x == CTL_PENDING ? pending : 0ULL;
-}
-
-}  // namespace
-}  // namespace mce
 
 struct mce_batched {
     const mce_graph *g = nullptr;
@@ -170,21 +160,20 @@ mce_status plan_shape(mce_batched *b, cudaStream_t s) {
 // the stream work of one run (no host synchronisation, no allocation)
 mce_status plan_issue(mce_batched *b, cudaStream_t s) {
     BkParams &P = b->P;
-    const int32_t n = b->g->n, k = b->k;
+    const int32_t k = b->k;
     MCE_CUDA(cudaMemcpyAsync(b->out.p, b->out0.p, OUT_WORDS * 8, cudaMemcpyDeviceToDevice, s));
     MCE_CUDA(cudaMemcpyAsync(b->gcount.p, b->gcount0.p, (size_t)k * 8, cudaMemcpyDeviceToDevice, s));
     MCE_CUDA(cudaMemcpyAsync(b->ghash.p, b->ghash0.p, (size_t)k * 8, cudaMemcpyDeviceToDevice, s));
     MCE_CUDA(cudaMemsetAsync(b->gnodes.p, 0, (size_t)k * 8, s));
     MCE_CUDA(cudaMemsetAsync(b->any.p, 0, 4, s));
-    if (b->coff.p) MCE_CUDA(cudaMemsetAsync(b->coff.p, 0xff, (size_t)n * 8, s));
     if (P.n_sub > 0) {
-        MCE_LAUNCH(k_plan_reset, grid_for(P.qcap, 256), 256, 0, s, P.qseq, P.qcap, P.ctl, (unsigned long long)P.n_sub);
+        MCE_TRY(launch_build_rows(P, true, s));
         MCE_TRY(launch_bk(P, b->ls.warps_per_block, b->ls.blocks_per_sm, s));
     } else {
         MCE_CUDA(cudaMemsetAsync(P.ctl, 0, CTL_WORDS * 8, s));
     }
     MCE_LAUNCH(k_graph_status, grid_for(k, 256), 256, 0, s, b->gnodes.as<unsigned long long>(), k, P.graph_budget,
-               b->status.as<int32_t>(), b->any.as<int32_t>());
+               b->status.as<int32_t>(), b->any.as<int32_t>(), P.build_ctl ? P.build_ctl + BUILD_NEXT : nullptr);
     return MCE_OK;
 }
 
@@ -303,6 +292,13 @@ mce_status mce_batched_create(const mce_graph *g, const int32_t *graph_ptr, int3
         P.cache = reinterpret_cast<uint32_t *>(((uintptr_t)b->cache.p + 127) & ~(uintptr_t)127);
         P.cache_words = cw;
         P.cache_off = b->coff.as<long long>();
+        MCE_TRY(b->bb.big.alloc((size_t)n_act * 4, s));
+        MCE_TRY(b->bb.build_ctl.alloc(BUILD_WORDS * 8, s));
+        MCE_CUDA(cudaMemsetAsync(b->bb.build_ctl.p, 0, BUILD_WORDS * 8, s));
+        P.build_big = b->bb.big.as<int32_t>();
+        P.build_ctl = b->bb.build_ctl.as<unsigned long long>();
+        MCE_TRY(build_prepare());
+        MCE_TRY(launch_build_layout(P, s));
     }
     {
         // With a per-graph budget the lane search would finish its buffered

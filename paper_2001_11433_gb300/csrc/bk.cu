@@ -2172,39 +2172,14 @@ __device__ bool run_task(const BkParams &P, Ws &s, const Task &T, Acc &acc, unsi
     const uint64_t tb = globaltimer_ns();
     bool ready = false;
     if (P.mode == BK_MCE && P.cache) {
-        const int64_t sw = bk_shared_words(w, c);
-        long long off = -1;
-        if (lane == 0) {
-            if (T.rec < 0) {
-                const unsigned long long o = atomicAdd(&P.ctl[CTL_CACHE_TOP], (unsigned long long)sw);
-                off = ((int64_t)o + sw <= P.cache_words) ? (long long)o : -1;
-            } else {
-                off = __ldcg(P.cache_off + root);
-            }
-        }
-        off = __shfl_sync(FULL, off, 0);
+        const long long off = P.cache_off[root];
         if (off >= 0) {
-            uint32_t *sh = P.cache + off;
-            ws_layout_split(s, sh, base, w, c);
-            if (T.rec < 0) {
-                // open the subproblem: build it into the cache and publish it
-                build_mce(P, s, root, lane);
-                if (lane == 0) {
-                    sh[0] = (uint32_t)s.W;
-                    sh[1] = (uint32_t)s.f;
-                }
-                __threadfence();
-                __syncwarp();
-                if (lane == 0) atomicExch(reinterpret_cast<unsigned long long *>(P.cache_off + root),
-                                          (unsigned long long)off);
-                if (lane == 0) {
-                    cold().builds++;
-                    cold().build_ns += globaltimer_ns() - tb;
-                }
-            } else {
-                s.W = (int32_t)__ldcg(sh);
-                s.f = (int32_t)__ldcg(sh + 1);
-            }
+            const uint32_t *sh = P.cache + off;
+            ws_layout_split(s, P.cache + off, base, w, c);
+            s.W = (int32_t)sh[0];
+            s.f = (int32_t)sh[1];
+            s.Wf0 = (s.f + 31) >> 5;
+            if (T.rec < 0 && lane == 0) cold().builds++;
             built = -1;   // the private region no longer holds a private build
             ready = true;
         }

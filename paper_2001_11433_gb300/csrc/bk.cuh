@@ -15,12 +15,19 @@ enum CtlWord {
     CTL_QHEAD = 2 * 16,      // ring tickets taken by poppers
     CTL_PENDING = 3 * 16,    // subproblems + queued tasks not finished
     CTL_HUNGRY = 4 * 16,     // warps waiting for work
-    CTL_CACHE_TOP = 5 * 16,  // words of the build cache in use
-    CTL_NODES = 6 * 16,      // tree nodes, for the budget
-    CTL_ABORT = 7 * 16,      // 1 = budget, 2 = timeout, 4 = workspace too small, 8 = bad task
-    CTL_T_LAST = 8 * 16,     // globaltimer when the last subproblem was claimed
-    CTL_T_END = 9 * 16,      // latest globaltimer at which a warp left the launch
-    CTL_WORDS = 10 * 16
+    CTL_NODES = 5 * 16,      // tree nodes, for the budget
+    CTL_ABORT = 6 * 16,      // 1 = budget, 2 = timeout, 4 = workspace too small, 8 = bad task
+    CTL_T_LAST = 7 * 16,     // globaltimer when the last subproblem was claimed
+    CTL_T_END = 8 * 16,      // latest globaltimer at which a warp left the launch
+    CTL_WORDS = 9 * 16
+};
+
+// Control words of the builds (uint64).
+enum BuildWord {
+    BUILD_TOP = 0,     // words of the build cache in use
+    BUILD_BIG = 1,     // subproblems built by a block
+    BUILD_NEXT = 2,    // next of them
+    BUILD_WORDS = 4
 };
 
 // Output block (uint64 words); the size histogram follows at OUT_HIST.
@@ -78,11 +85,14 @@ struct BkParams {
     unsigned long long *qseq;
     int64_t qcap;
     uint32_t *taskbuf;
-    // build cache: the warp that opens a subproblem builds its read-only part
-    // here and publishes the offset in cache_off[v]; pieces reuse it
+    // build cache: the read-only parts of the subproblems, built before the
+    // search (launch_build); cache_off[v] = offset, -1 = no room, the warps that
+    // take it build it for themselves
     uint32_t *cache;
     int64_t cache_words;
     long long *cache_off;
+    int32_t *build_big;       // n_sub entries: the subproblems built by a block
+    unsigned long long *build_ctl;   // BUILD_* words
     unsigned long long *ctl;
     // outputs
     unsigned long long *out;
@@ -110,7 +120,8 @@ struct BkParams {
 // Words of the read-only part of a built subproblem with w local vertices of
 // which c are candidates: a 32-word header (kept vertices W, kept fini f),
 // then local ids, bounds, bitset rows, the bound-sorted fini list F0, and one
-// bitset over F0 positions per candidate (its lower-ranked neighbours).
+// bitset over F0 positions per candidate (its lower-ranked neighbours; builds
+// in the cache keep every local vertex and use ⌈f/32⌉ words a bitset).
 // Rounded to 32 words so that every part starts on a 128-byte line.
 // Bitset rows are ⌈c/32⌉ words padded to a multiple of 4, so that every row
 // starts on a 16-byte boundary and is read as 16-byte vectors.
@@ -169,6 +180,15 @@ __host__ __device__ inline int64_t bk_ws_words(int64_t w, int64_t c, int32_t mod
     return bk_shared_words(w, c) + bk_private_words(w, c, mode);
 }
 
+// Builds of every scheduled subproblem into the cache (which P has), before
+// launch_bk on the same stream; build_prepare once outside any capture.
+// launch_build_layout fills cache_off and build_big from the order (build_ctl
+// zero before it); launch_build_rows builds (BUILD_NEXT zero before it).  With
+// `reset`, the latter also sets the task ring and the control block to their
+// start values.
+mce_status build_prepare();
+mce_status launch_build_layout(const BkParams &p, cudaStream_t s);
+mce_status launch_build_rows(const BkParams &p, bool reset, cudaStream_t s);
 mce_status bk_prepare(int32_t blocks_per_sm, int64_t smem_bytes);
 mce_status launch_bk(const BkParams &p, int32_t warps_per_block, int32_t blocks_per_sm, cudaStream_t s);
 mce_status init_queue_seq(unsigned long long *seq, int64_t n, cudaStream_t s);

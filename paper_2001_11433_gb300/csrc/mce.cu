@@ -284,6 +284,15 @@ mce_status run_bk(BkParams &P, const LaunchShape &ls, int64_t req_max, int64_t c
     MCE_LAUNCH(k_set_u64, 1, 1, 0, s, P.ctl + CTL_PENDING, (unsigned long long)P.n_sub);
     if (P.timeout_ns == 0) P.timeout_ns = 60ULL * 1000000000ULL;
     if (P.max_run_ns == 0) P.max_run_ns = 600ULL * 1000000000ULL;
+    if (P.cache) {
+        MCE_TRY(b.big.alloc((size_t)P.n_sub * 4, s));
+        MCE_TRY(b.build_ctl.alloc(BUILD_WORDS * 8, s));
+        MCE_CUDA(cudaMemsetAsync(b.build_ctl.p, 0, BUILD_WORDS * 8, s));
+        P.build_big = b.big.as<int32_t>();
+        P.build_ctl = b.build_ctl.as<unsigned long long>();
+        MCE_TRY(launch_build_layout(P, s));
+        MCE_TRY(launch_build_rows(P, false, s));
+    }
     return launch_bk(P, ls.warps_per_block, ls.blocks_per_sm, s);
 }
 
@@ -538,7 +547,6 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
         if (cw > 0) {
             MCE_TRY(cache.alloc((size_t)cw * 4 + 512, s));
             MCE_TRY(coff.alloc((size_t)n * 8, s));
-            MCE_CUDA(cudaMemsetAsync(coff.p, 0xff, (size_t)n * 8, s));
             // 128-byte aligned start
             P.cache = reinterpret_cast<uint32_t *>(((uintptr_t)cache.p + 127) & ~(uintptr_t)127);
             P.cache_words = cw;

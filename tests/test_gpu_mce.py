@@ -295,6 +295,21 @@ def test_awkward_rows_per_vertex_exact(gpu_lib, kind, shape):
         assert np.array_equal(u64(pv[k]), o.per_vertex[name])
 
 
+@pytest.mark.parametrize("n,p", [(33, 0.97), (129, 0.3), (256, 0.5), (300, 0.44)])
+def test_builds_by_warp_and_block_exact(gpu_lib, n, p):
+    """Subproblems on both sides of 32 and 128 local vertices."""
+    mce = gpu_lib
+    u, v = graphgen.er(n, p, n)
+    og = O.Graph(n, u, v)
+    rk = np.random.default_rng(n).permutation(n).astype(np.int32)
+    o = O.parmce(og, rk, per_vertex=True, threads=4)
+    pv = per_vertex_bufs(n)
+    r = mce.enumerate_cliques(gpu_graph(mce, n, u, v), rank="user", user_rank=_t(rk), per_vertex=pv)
+    assert_same_summary(r, o)
+    for k, name in enumerate(("count", "hash", "nodes")):
+        assert np.array_equal(u64(pv[k]), o.per_vertex[name])
+
+
 @pytest.mark.parametrize("shape", [(2, 16), (3, 64), (4, 256)])
 def test_handover_stress_keeps_every_subproblem(gpu_lib, shape):
     """Hand-overs every few nodes (ParTTT prefix rule, Algorithm 3) from wide
