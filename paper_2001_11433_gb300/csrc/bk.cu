@@ -514,6 +514,7 @@ struct AccCold {
     unsigned long long count, hash, nodes;   // whole launch
     unsigned long long t_rep;                // this task's nodes already credited to sub_nodes / graph_nodes
     unsigned long long t_split;              // this task's nodes at its last hand-over
+    unsigned long long t_split_ns;           // and when that was (or when the task began)
 };
 __shared__ AccCold g_cold[8];   // warps of one search block
 __device__ __forceinline__ AccCold &cold() { return g_cold[threadIdx.x >> 5]; }
@@ -653,6 +654,16 @@ struct Task {
     int64_t rec;         // arena offset of a handed-over frame, -1 for a whole subproblem
 };
 
+// A wide node's share of the interval between two polls: its pivot and its
+// children walk cand ∪ fini, so a node of thousands of members counts as many
+// (64 nodes of a hub's subproblem could keep waiting warps idle for 20 ms).
+__device__ __forceinline__ int node_weight(int cn, int fn) { return 1 + ((cn + fn) >> 7); }
+
+// Time after which a task may hand over again whatever its nodes.  Measured on
+// GB300: 50 us; the 1.7M-vertex graph under the degeneracy rank searched
+// in 36 ms instead of 51 ms (one subproblem alone kept its warp busy for 42 ms).
+constexpr uint64_t BK_SPLIT_NS = 50000;
+
 // Budget, abort and splitting checks, made every 64 nodes with the current
 // frame written back to memory.  Returns 0 = go on, 1 = stop the launch,
 // 2 = drop this task (its graph or subproblem is over budget).
@@ -664,7 +675,8 @@ __device__ int poll(const BkParams &P, Acc &acc, int lane, int32_t root, uint64_
     unsigned long long ab = 0, hungry = 0;
     int lph = 0;
     if (lane == 0) {
-        if (globaltimer_ns() - t_start > P.max_run_ns) atomicOr(&P.ctl[CTL_ABORT], 2ULL);
+        const uint64_t now = globaltimer_ns();
+        if (now - t_start > P.max_run_ns) atomicOr(&P.ctl[CTL_ABORT], 2ULL);
         ab = *(volatile unsigned long long *)&P.ctl[CTL_ABORT];
         if (P.node_budget) {
             const unsigned long long tot = atomicAdd(&P.ctl[CTL_NODES], 64ULL) + 64ULL;
@@ -700,9 +712,13 @@ __device__ int poll(const BkParams &P, Acc &acc, int lane, int32_t root, uint64_
             const bool heavy = P.heavy && P.heavy[P.mode == BK_MCE ? root : 0];
             const unsigned long long every = heavy ? P.heavy_split_nodes : P.split_nodes;
             // a task hands over again only after 2048 more nodes of its own
-            // (fewer for a heavy one): pieces cut too small cost their receivers
-            // more than they hold
-            if (acc.t_nodes - cold().t_split < (heavy && every < 2048ULL ? every : 2048ULL)) hungry = 0;
+            // (fewer for a heavy one) or BK_SPLIT_NS: pieces cut too small cost
+            // their receivers more than they hold (without the build cache a
+            // whole build each: there only the nodes count), but the nodes of a
+            // hub's subproblem can take a tenth of a millisecond each
+            if (acc.t_nodes - cold().t_split < (heavy && every < 2048ULL ? every : 2048ULL) &&
+                (!P.cache || now - cold().t_split_ns < BK_SPLIT_NS))
+                hungry = 0;
             // a long-running task spreads its subtree before anybody waits
             if (!hungry && every && acc.t_nodes - cold().t_split >= every &&
                 qlen < (unsigned long long)P.qcap / 2) hungry = 1;
@@ -725,7 +741,10 @@ __device__ int poll(const BkParams &P, Acc &acc, int lane, int32_t root, uint64_
     hungry_out = hungry;
     if (ab & 3ULL) return 1;
     if (ab & 16ULL) return 2;
-    if (hungry && lane == 0) cold().t_split = acc.t_nodes;
+    if (hungry && lane == 0) {
+        cold().t_split = acc.t_nodes;
+        cold().t_split_ns = globaltimer_ns();
+    }
     return 0;
 }
 
@@ -1902,7 +1921,8 @@ __device__ int search(const BkParams &P, Ws &s, const Task &T, Acc &acc, unsigne
                 count_node_wops(acc, lane, node_cn, node_fn, __reduce_add_sync(FULL, ne));
             }
             enter = false;
-            if (++node_tick >= acc.tick) {
+            node_tick += node_weight(node_cn, node_fn);
+            if (node_tick >= acc.tick) {
                 node_tick = 0;
                 frame_store<NR>(s, d, lane, rc, rf, re, rx, imce);
                 __syncwarp();
@@ -2081,11 +2101,12 @@ __device__ int search_mem(const BkParams &P, Ws &s, const Task &T, Acc &acc, uns
                 const uint32_t *prow = s.A + (int64_t)p * s.S;
                 for (int k = lane; k < wc; k += 32) ext[k] = cand[k] & ~prow[k];
                 __syncwarp();
-                count_node_wops(acc, lane, warp_popc(cand, wc, lane), warp_popc(finic, wc, lane) + flen,
-                                warp_popc(ext, wc, lane));
+                const int node_cn = warp_popc(cand, wc, lane), node_fn = warp_popc(finic, wc, lane) + flen;
+                count_node_wops(acc, lane, node_cn, node_fn, warp_popc(ext, wc, lane));
+                node_tick += node_weight(node_cn, node_fn);
             }
             enter = false;
-            if (++node_tick >= acc.tick) {
+            if (node_tick >= acc.tick) {
                 node_tick = 0;
                 const int act = periodic(P, s, T, acc, lane, d, root, t_start);
                 if (act) return act;
@@ -2299,7 +2320,7 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
     uint32_t *ws_glob = P.gws + gwarp * P.gws_words;
     uint32_t *taskbuf = P.taskbuf + gwarp * P.slot_words;
     Acc acc = {0, 0, 0, 0, 64, 4, 0};
-    if (lane == 0) cold() = AccCold{0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    if (lane == 0) cold() = AccCold{};
     Ws s;
     s.piv = smem + 512 + (int64_t)wib * BK_PIV_WORDS;
     s.lp = lp_smem;
@@ -2398,6 +2419,7 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
         acc.t_count = acc.t_hash = acc.t_nodes = 0;
         if (lane == 0) cold().t_rep = cold().t_split = 0;
         const uint64_t t0 = globaltimer_ns();
+        if (lane == 0) cold().t_split_ns = t0;
         const bool go_on = run_task(P, s, T, acc, shist, ws_smem, ws_glob, taskbuf, lane, built, node_tick, t_start);
         if (lane == 0) cold().max_busy += globaltimer_ns() - t0;
         if (lane == 0) {
