@@ -515,6 +515,8 @@ struct AccCold {
     unsigned long long t_rep;                // this task's nodes already credited to sub_nodes / graph_nodes
     unsigned long long t_split;              // this task's nodes at its last hand-over
     unsigned long long t_split_ns;           // and when that was (or when the task began)
+    unsigned long long t_hist;               // this task's cliques already counted in since_hist
+    unsigned long long since_hist;           // cliques of this warp since it last emptied the shared bins
 };
 __shared__ AccCold g_cold[8];   // warps of one search block
 __device__ __forceinline__ AccCold &cold() { return g_cold[threadIdx.x >> 5]; }
@@ -537,15 +539,37 @@ __device__ __forceinline__ void count_node_wops(Acc &acc, int lane, int cn, int 
                     2ull * (unsigned long long)next * (unsigned long long)((cn + fn + 31) >> 5);
 }
 
+// The block's size bins are 32 bits wide: shared memory adds 32 bits in one
+// instruction, and counts the lanes of a warp that add 1 to the same bin
+// together (64 bits are a compare-and-swap loop over those lanes).  A warp that has emitted 2^18 cliques
+// since it last did so empties the bins into the 64-bit ones in memory;
+// between two checks a warp emits at most 64 * 3^11 more, so eight warps stay
+// far below 2^32.
+__device__ __forceinline__ void hist_guard(const BkParams &P, const Acc &acc, uint32_t *shist, int lane) {
+    const unsigned long long since = cold().since_hist + (acc.t_count - cold().t_hist);
+    __syncwarp();
+    const bool full = since >= (1ULL << 18);
+    if (lane == 0) {
+        cold().since_hist = full ? 0ULL : since;
+        cold().t_hist = acc.t_count;
+    }
+    if (full)
+        for (int b = lane; b < 256; b += 32) {
+            const uint32_t v = atomicExch(&shist[b], 0u);
+            if (v) atomicAdd(&P.out[OUT_HIST + b], (unsigned long long)v);
+        }
+    __syncwarp();
+}
+
 __device__ void emit(const BkParams &P, const Ws &s, int32_t root, int32_t k0, int d, uint64_t hsum, Acc &acc,
-                     unsigned long long *shist, int lane) {
+                     uint32_t *shist, int lane) {
     const uint32_t size = (uint32_t)(k0 + d);
     if (lane == 0) acc.wops += size;   // |K| additions of the clique hash
     const uint64_t h = clique_hash_from_sum(hsum, size);
     acc.t_count++;
     acc.t_hash += h;
     if (lane == 0) {
-        if (size < 256) atomicAdd(&shist[size], 1ULL);
+        if (size < 256) atomicAdd(&shist[size], 1u);
         else if (size < MCE_HIST_CAP) atomicAdd(&P.out[OUT_HIST + size], 1ULL);
         else atomicOr(&P.out[OUT_FLAGS], 2ULL);
     }
@@ -670,8 +694,9 @@ constexpr uint64_t BK_SPLIT_NS = 50000;
 // Lane 0 reads the control words and credits node counts; the result is
 // broadcast: returns 1 = stop the launch, 2 = drop this task, 0 = go on with
 // `hungry` = the number of hand-overs wanted (0 = none).
-__device__ int poll(const BkParams &P, Acc &acc, int lane, int32_t root, uint64_t t_start,
+__device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int32_t root, uint64_t t_start,
                     unsigned long long &hungry_out) {
+    hist_guard(P, acc, shist, lane);
     unsigned long long ab = 0, hungry = 0;
     int lph = 0;
     if (lane == 0) {
@@ -819,10 +844,10 @@ __device__ void donate_mem(const BkParams &P, Ws &s, const Task &T, int lane, in
 
 // Checks made every 64 nodes with the current frame written back to memory.
 // Returns 0 = go on, 1 = stop the launch, 2 = drop this task.
-__device__ int periodic(const BkParams &P, Ws &s, const Task &T, Acc &acc, int lane, int d, int32_t root,
-                        uint64_t t_start) {
+__device__ int periodic(const BkParams &P, Ws &s, const Task &T, Acc &acc, uint32_t *shist, int lane, int d,
+                        int32_t root, uint64_t t_start) {
     unsigned long long hungry = 0;
-    const int code = poll(P, acc, lane, root, t_start, hungry);
+    const int code = poll(P, acc, shist, lane, root, t_start, hungry);
     if (code || !hungry) return code;
     // up to four hand-overs per check when many warps wait
     int budget = hungry > (unsigned long long)acc.give ? acc.give : (int)hungry;
@@ -848,6 +873,7 @@ __device__ int periodic(const BkParams &P, Ws &s, const Task &T, Acc &acc, int l
 struct SmallU {
     uint32_t adjC, adjX, exclC;
     uint32_t tC, tX;         // 127 - (position of the global id among C ∪ X): pivot tie keys
+    uint32_t beforeC, posX;  // X_l: number of C with a smaller global id, position among X
     int cn, xn;
 };
 
@@ -1036,15 +1062,17 @@ __device__ __forceinline__ void small_relabel(const BkParams &P, const Ws &s, in
         gC = lane < u.cn ? s.gid[cidC] : 0x7fffffff;
         const int32_t gX = lane < u.xn ? s.gid[cidX] : 0x7fffffff;
         // C is in increasing global id, so C_l has l smaller ids in C
-        int oc = lane, ox = 0;
+        int oc = lane, ox = 0, xc = 0;
         for (int k = 0; k < u.xn; ++k) {
             const int32_t gk = __shfl_sync(FULL, gX, k);
             oc += gk < gC;
             ox += gk < gX;
         }
-        for (int k = 0; k < u.cn; ++k) ox += __shfl_sync(FULL, gC, k) < gX;
+        for (int k = 0; k < u.cn; ++k) xc += __shfl_sync(FULL, gC, k) < gX;
         u.tC = 127u - (uint32_t)oc;
-        u.tX = 127u - (uint32_t)ox;
+        u.tX = 127u - (uint32_t)(ox + xc);
+        u.beforeC = (uint32_t)xc;
+        u.posX = (uint32_t)ox;
     }
     __syncwarp();   // Cl / Xl are scratch again after this point
 }
@@ -1053,7 +1081,7 @@ __device__ __forceinline__ void small_relabel(const BkParams &P, const Ws &s, in
 // in rx, F list Fd[0..flen)), already counted, with cand not empty.
 // Frames 0..d-1 are in memory.  Returns as search<NR>.
 template <int NR>
-__device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, unsigned long long *shist, int lane,
+__device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, uint32_t *shist, int lane,
                             int &node_tick, uint64_t t_start, int32_t root, int k0, int d, uint64_t hsum,
                             const uint32_t (&rc)[NR], const uint32_t (&rf)[NR], const uint32_t (&rx)[NR],
                             const int32_t *Fd, int flen) {
@@ -1105,7 +1133,7 @@ __device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, u
         acc.t_count++;
         acc.t_hash += h;
         if (lane == 0) {
-            if (size < 256) atomicAdd(&shist[size], 1ULL);
+            if (size < 256) atomicAdd(&shist[size], 1u);
             else if (size < MCE_HIST_CAP) atomicAdd(&P.out[OUT_HIST + size], 1ULL);
             else atomicOr(&P.out[OUT_FLAGS], 2ULL);
         }
@@ -1180,7 +1208,7 @@ __device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, u
                 node_tick = 0;
                 flush();
                 unsigned long long hungry = 0;
-                const int code = poll(P, acc, lane, root, t_start, hungry);
+                const int code = poll(P, acc, shist, lane, root, t_start, hungry);
                 if (code) return code;
                 if (hungry) {
                     int budget = hungry > (unsigned long long)acc.give ? acc.give : (int)hungry;
@@ -1306,78 +1334,103 @@ __device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, u
 // reaches (small_relabel) into a universe in its shared-memory arena and goes
 // on with the wide search; when the arena or the root table is full, or the
 // task ends, the lanes search the buffered subtrees (lp_run): the TTT step of
-// search_small on 32-bit masks, one node per lane at a time, the nodes taken
-// 32 at a time from a stack of entered nodes that the lanes share, so that
-// the heavy-tailed subtree sizes spread over the lanes node by node.  Trees,
-// node counts, word operations and cliques are those of search_small.
+// search_small on 32-bit masks.  Trees, node counts, word operations and
+// cliques are those of search_small.
 //
-// Universe of a small node with cn candidates and xn fini vertices (arena
-// words): h(C_k) as uint64 [2 cn]; per C member its row adjC and tie key
-// [2 cn]; per X member its row adjX and tie key [2 xn] (a row and its key are
-// read together as one 8-byte word); the columns of adjX (adjXT[k] =
-// {x : X_x ~ C_k}) [cn].  Root record (4 words): arena offset,
+// Universe of a small node with cn candidates and xn fini vertices, X in
+// ascending global id like C (arena words): h(C_k) as uint64 [2 cn]; per C
+// member its rows (neighbours in C, neighbours in X), read together as one
+// 8-byte word [2 cn]; per X member its row in C and the number of C members
+// with a smaller global id [2 xn].  Root record (4 words): arena offset,
 // cn | xn << 8 | (clique size at the node) << 16, hash sum at the node.
 
-__device__ __forceinline__ int lp_universe_words(int cn, int xn) { return (5 * cn + 2 * xn + 1) & ~1; }
+__device__ __forceinline__ int lp_universe_words(int cn, int xn) { return 4 * cn + 2 * xn; }
 
+// Sums of one lane over one lp_run.  32 bits hold them: 64 universes of at
+// most 32 candidates have fewer than 2^24 nodes, each of fewer than 2^8 word
+// operations.
 struct LpSums {
-    unsigned long long hash, wops;
-    uint32_t count, nodes, smax;
+    unsigned long long hash;
+    uint32_t wops, count, nodes, smax;
 };
 
-// A small-subtree node for one lane: its universe and its state.
-struct LpNode {
-    const uint64_t *hC;
-    const uint2 *akC, *akX;   // (row, tie key) per C / X member
-    const uint32_t *adjXT;
-    int cn;
-    uint32_t base;     // clique size at the universe's root
-    uint32_t cand, finc, xs;
-    uint64_t hs;
-    int depth;         // below the universe's root
-};
-
-__device__ __forceinline__ void lp_emit(const BkParams &P, unsigned long long *shist, LpSums &o, uint32_t size,
-                                        uint64_t hsum) {
+__device__ __forceinline__ void lp_emit(const BkParams &P, uint32_t *shist, LpSums &o, uint32_t size, uint64_t hsum) {
     o.count++;
     o.hash += clique_hash_from_sum(hsum, size);
     o.wops += size;
-    if (size < 256) atomicAdd(&shist[size], 1ULL);
+    if (size < 256) atomicAdd(&shist[size], 1u);
     else if (size < MCE_HIST_CAP) atomicAdd(&P.out[OUT_HIST + size], 1ULL);
     else atomicOr(&P.out[OUT_FLAGS], 2ULL);
     if (size > o.smax) o.smax = size;
 }
 
-// Pivot of an entered node (cand not empty): ext = cand minus the pivot's
-// neighbours, with the pivot the largest (count + 1, tie key) over cand ∪
-// finc and xs (the order of search_small).
-__device__ __forceinline__ uint32_t lp_pivot_ext(const LpNode &u, LpSums &o) {
-    const uint32_t cf = u.cand | u.finc;
-    uint32_t best = 0u, badj = 0u;
-    for (uint32_t m = cf; m; m &= m - 1u) {
-        const uint2 ak = u.akC[__ffs(m) - 1];
-        const uint32_t kk = ((uint32_t)(__popc(u.cand & ak.x) + 1) << 7) | ak.y;
-        if (kk > best) {
-            best = kk;
-            badj = ak.x;
-        }
-    }
-    for (uint32_t m = u.xs; m; m &= m - 1u) {
-        const uint2 ak = u.akX[__ffs(m) - 1];
-        const uint32_t kk = ((uint32_t)(__popc(u.cand & ak.x) + 1) << 7) | ak.y;
-        if (kk > best) {
-            best = kk;
-            badj = ak.x;
-        }
-    }
-    const uint32_t ext = u.cand & ~badj;
-    const uint32_t t = (uint32_t)(__popc(cf) + __popc(u.xs));
-    o.wops += t + 2u * (uint32_t)__popc(ext) * ((t + 31u) >> 5);
-    return ext;
+// sum and carry of three bits, in every bit position
+__device__ __forceinline__ uint32_t full_add(uint32_t a, uint32_t b, uint32_t c, uint32_t &carry) {
+    carry = (a & b) | (c & (a | b));
+    return a ^ b ^ c;
 }
 
-// Child N = K + q with two candidates a < b (fini cf, cx), settled in closed
-// form with the node counts, word operations and cliques of the search:
+// Pivot of an entered node (cand not empty): ext = cand minus the neighbours
+// of the member of cand ∪ finc ∪ xs with most candidate neighbours, ties to
+// the smallest global id.  The counts of all members are added up at once,
+// one bit of each count in each of six words (bit k of sc[b] = bit b of C_k's
+// count): four candidates' rows at a time, so that a node costs by its
+// candidates and not by its members.
+__device__ __forceinline__ uint32_t lp_pivot_ext(const uint2 *rows, const uint2 *xr, uint32_t cand, uint32_t finc,
+                                                 uint32_t xs) {
+    uint32_t sc[6] = {0u, 0u, 0u, 0u, 0u, 0u}, sx[6] = {0u, 0u, 0u, 0u, 0u, 0u};
+    for (uint32_t m = cand; m;) {
+        uint2 r[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            r[k] = m ? rows[__ffs(m) - 1] : make_uint2(0u, 0u);
+            m &= m - 1u;
+        }
+        uint32_t a, b, c;
+        sc[0] = full_add(sc[0], r[0].x, r[1].x, a);
+        sc[0] = full_add(sc[0], r[2].x, r[3].x, b);
+        sc[1] = full_add(sc[1], a, b, c);
+#pragma unroll
+        for (int k = 2; k < 6; ++k) {
+            const uint32_t t = sc[k] & c;
+            sc[k] ^= c;
+            c = t;
+        }
+        sx[0] = full_add(sx[0], r[0].y, r[1].y, a);
+        sx[0] = full_add(sx[0], r[2].y, r[3].y, b);
+        sx[1] = full_add(sx[1], a, b, c);
+#pragma unroll
+        for (int k = 2; k < 6; ++k) {
+            const uint32_t t = sx[k] & c;
+            sx[k] ^= c;
+            c = t;
+        }
+    }
+    // the members with the largest count, from the highest bit down
+    uint32_t mc = cand | finc, mx = xs;
+#pragma unroll
+    for (int k = 5; k >= 0; --k) {
+        const uint32_t tc = mc & sc[k], tx = mx & sx[k];
+        const bool any = (tc | tx) != 0u;
+        mc = any ? tc : mc;
+        mx = any ? tx : mx;
+    }
+    // smallest id among them: C and X ascend, and X_j comes after beforeC[j] of C
+    const int ic = __ffs(mc) - 1, ix = __ffs(mx) - 1;
+    uint32_t adj = 0u;
+    bool fromX = ix >= 0;
+    if (fromX) {
+        const uint2 x = xr[ix];
+        adj = x.x;
+        fromX = ic < 0 || ic >= (int)x.y;
+    }
+    if (!fromX) adj = rows[ic].x;
+    return cand & ~adj;
+}
+
+// Node N = K + q (clique size sz, hash sum hn) with two candidates a < b (fini
+// cf, cx), settled in closed form with the node counts, word operations and
+// cliques of the search:
 //   - a fini vertex adjacent to both is the pivot (count 2): N has no child;
 //   - a ~ b: the pivot has count 1 and N has one child, whose one candidate
 //     gives the clique N + a + b (two more nodes);
@@ -1386,282 +1439,192 @@ __device__ __forceinline__ uint32_t lp_pivot_ext(const LpNode &u, LpSums &o) {
 //     vertex is adjacent to it;
 //   - otherwise every count is 0: both candidates are leaf children and both
 //     N + a and N + b are cliques.
-__device__ __forceinline__ void lp_two(const BkParams &P, unsigned long long *shist, const LpNode &u, int q, LpSums &o,
-                                       uint32_t cc, uint32_t cf, uint32_t cx, uint64_t hq) {
-    const int a = __ffs(cc) - 1, b = __ffs(cc & (cc - 1u)) - 1;
-    const uint2 ka = u.akC[a], kb = u.akC[b];
-    const uint32_t xa = u.adjXT[a], xb = u.adjXT[b];
+__device__ __forceinline__ void lp_two(const BkParams &P, uint32_t *shist, LpSums &o, const uint2 *rows,
+                                       const uint2 *xr, const uint64_t *hC, uint32_t sz, uint64_t hn, uint32_t cc,
+                                       uint32_t cf, uint32_t cx) {
+    const int a = __ffs(cc) - 1, b = 31 - __clz(cc);
+    const uint2 ra = rows[a], rb = rows[b];
     const uint32_t t = 2u + (uint32_t)(__popc(cf) + __popc(cx));
-    const uint32_t sz = u.base + (uint32_t)u.depth + 1u;   // |N|
-    const uint64_t hn = u.hs + hq;                         // hash sum of N
-    ++o.nodes;                                             // N
-    if ((cf & ka.x & kb.x) != 0u || (cx & xa & xb) != 0u) {
+    ++o.nodes;   // N
+    if (((cf & ra.x & rb.x) | (cx & ra.y & rb.y)) != 0u) {
         o.wops += t;
         return;
     }
     const uint32_t wt = 2u * ((t + 31u) >> 5);
-    const uint32_t f1c = cf & (ka.x ^ kb.x), f1x = cx & (xa ^ xb);   // fini adjacent to exactly one
-    // the fini member of f1 with the highest tie key, and whether it touches a
-    uint32_t fk = 0u;
-    bool f_on_a = false;
-    for (uint32_t m = f1c; m; m &= m - 1u) {
-        const int k = __ffs(m) - 1;
-        const uint32_t kk = u.akC[k].y;
-        if (kk >= fk) {
-            fk = kk + 1u;
-            f_on_a = (ka.x >> k) & 1u;
-        }
+    // fini adjacent to exactly one: the smallest id among them, whether it
+    // touches a, and whether it comes before a
+    const uint32_t f1c = cf & (ra.x ^ rb.x), f1x = cx & (ra.y ^ rb.y);
+    const int fc = __ffs(f1c) - 1, fx = __ffs(f1x) - 1;
+    bool on_a = fc >= 0 && ((ra.x >> (fc & 31)) & 1u), before_a = fc >= 0 && fc < a;
+    if (fx >= 0) {
+        const int after = (int)xr[fx].y;   // C members before it
+        if (fc < 0 || fc >= after) on_a = (ra.y >> fx) & 1u;
+        before_a |= a >= after;
     }
-    for (uint32_t m = f1x; m; m &= m - 1u) {
-        const int x = __ffs(m) - 1;
-        const uint32_t kk = u.akX[x].y;
-        if (kk >= fk) {
-            fk = kk + 1u;
-            f_on_a = (xa >> x) & 1u;
-        }
-    }
-    if ((ka.x >> b) & 1u) {
-        // a ~ b: pivot among a, b and f1 by tie key; the child is a if the pivot is
-        // a or a fini vertex on b only, else b
-        const uint32_t best = max(max(ka.y, kb.y) + 1u, fk);
-        int qq;
-        if (best == ka.y + 1u) qq = a;
-        else if (best == kb.y + 1u) qq = b;
-        else qq = f_on_a ? b : a;
-        const uint32_t rq = qq == a ? ka.x : kb.x, xq = qq == a ? xa : xb;
+    if ((ra.x >> b) & 1u) {
+        // a ~ b: pivot a, or the fini vertex before it; the child is a if the pivot
+        // is a or a fini vertex on b only, else b
+        const int qq = before_a && on_a ? b : a;
+        const uint2 rq = qq == a ? ra : rb;
         o.wops += t + wt;
-        const uint32_t tg = 1u + (uint32_t)(__popc(cf & rq) + __popc(cx & xq));
+        const uint32_t tg = 1u + (uint32_t)(__popc(cf & rq.x) + __popc(cx & rq.y));
         o.nodes += 2;
         o.wops += tg + 2u * ((tg + 31u) >> 5);
-        lp_emit(P, shist, o, sz + 2u, hn + u.hC[a] + u.hC[b]);
+        lp_emit(P, shist, o, sz + 2u, hn + hC[a] + hC[b]);
         return;
     }
-    if (fk) {
+    if ((f1c | f1x) != 0u) {
         // a !~ b: the pivot is the fini vertex; its other candidate is the child
-        const int qq = f_on_a ? b : a;
-        const uint32_t rq = qq == a ? ka.x : kb.x, xq = qq == a ? xa : xb;
+        const int qq = on_a ? b : a;
+        const uint2 rq = qq == a ? ra : rb;
         o.wops += t + wt;
         ++o.nodes;
-        if ((cf & rq) == 0u && (cx & xq) == 0u) lp_emit(P, shist, o, sz + 1u, hn + u.hC[qq]);
+        if (((cf & rq.x) | (cx & rq.y)) == 0u) lp_emit(P, shist, o, sz + 1u, hn + hC[qq]);
         return;
     }
     // all counts 0: both candidates are children, both leaves and cliques
     o.wops += t + 2u * wt;
     o.nodes += 2;
-    lp_emit(P, shist, o, sz + 1u, hn + u.hC[a]);
-    lp_emit(P, shist, o, sz + 1u, hn + u.hC[b]);
+    lp_emit(P, shist, o, sz + 1u, hn + hC[a]);
+    lp_emit(P, shist, o, sz + 1u, hn + hC[b]);
 }
 
-// Child q of a node whose cand / finc already exclude / include q: leaves
-// and one-candidate children are settled here (returns false); otherwise the
-// child's sets are returned for a push (returns true).  Node counts and word
-// operations follow search_small.
-__device__ __forceinline__ bool lp_child(const BkParams &P, unsigned long long *shist, const LpNode &u, int q,
-                                         LpSums &o, uint32_t &cc, uint32_t &cf, uint32_t &cx, uint64_t &hq) {
-    const uint32_t aq = u.akC[q].x;
-    cc = u.cand & aq;
-    cf = u.finc & aq;
-    cx = u.xs & u.adjXT[q];
-    hq = u.hC[q];
-    if (cc == 0u) {
-        // a leaf: a maximal clique unless fini is left
-        ++o.nodes;
-        if ((cf | cx) == 0u) lp_emit(P, shist, o, u.base + (uint32_t)u.depth + 1u, u.hs + hq);
-        return false;
+// The buffered small subtrees, from one stack of nodes (entered, not yet
+// pivoted) that the warp's lanes share.  Each round the lanes take up to 32
+// nodes off the top and pivot one each; then the children of all of them are
+// dealt out to the lanes one each: child q of a node follows from the node's
+// sets and the ext members before q alone.  Children with at most two
+// candidates are settled at once, the others pushed.  (Each lane going through
+// the children of its own node left half of the lanes idle: R-MAT 18 searched
+// at 23.6 warp instructions a node; see with the children dealt out
+// the lane search takes 88 of the 168 ms a warp searches on R-MAT 18, whose
+// search fell from 218 to 196 ms.)
+//
+// Room: up to 512 nodes on the stack 32 are taken, and each pushes fewer than
+// 32; up to 1024, 8; above, one at a time, whose whole subtree then holds at
+// most 3 + 4 + ... + 32 = 525 nodes: at most 1504 + 525 < BK_LP_TASK_CAP.
+// (scratch: 256 words, the nodes taken in this round.)
+__device__ __noinline__ LpSums lp_run(const BkParams &P, uint32_t *lp, int nroots, uint32_t *shist, uint32_t *tasks,
+                                      uint32_t *scratch, int lane) {
+    LpSums o = {0ULL, 0u, 0u, 0u, 0u};
+    const uint32_t *arena = lp + BK_LP_TABLE_WORDS;
+    uint4 *stack = reinterpret_cast<uint4 *>(tasks);
+    uint4 *node = reinterpret_cast<uint4 *>(scratch);
+    for (int r = lane; r < nroots; r += 32) {
+        const uint4 rec = *reinterpret_cast<const uint4 *>(lp + 4 * r);
+        const uint32_t cn = rec.y & 0xffu, xn = (rec.y >> 8) & 0xffu;
+        stack[2 * r] = make_uint4(rec.x | (cn << 16), cn == 32u ? FULL : ((1u << cn) - 1u), 0u,
+                                  xn == 32u ? FULL : ((1u << xn) - 1u));
+        stack[2 * r + 1] = make_uint4(rec.z, rec.w, rec.y >> 16, 0u);
     }
-    if ((cc & (cc - 1u)) == 0u) {
-        // one candidate c: one more node and the clique K + q + c, unless a fini
-        // vertex adjacent to c is the pivot (then no child)
-        const int c = __ffs(cc) - 1;
-        const uint32_t t = 1u + (uint32_t)(__popc(cf) + __popc(cx));
-        if ((cf & u.akC[c].x) != 0u || (cx & u.adjXT[c]) != 0u) {
-            ++o.nodes;
-            o.wops += t;
-        } else {
-            o.nodes += 2;
-            o.wops += t + 2u * ((t + 31u) >> 5);
-            lp_emit(P, shist, o, u.base + (uint32_t)u.depth + 2u, u.hs + hq + u.hC[c]);
-        }
-        return false;
-    }
-    if (__popc(cc) == 2) {
-        lp_two(P, shist, u, q, o, cc, cf, cx, hq);
-        return false;
-    }
-    ++o.nodes;
-    return true;
-}
-
-// The whole subtree below an entered-but-not-yet-pivoted node, depth first.
-__device__ void lp_dfs(const BkParams &P, unsigned long long *shist, LpNode u, LpSums &o) {
-    uint32_t stk[32 * 5];   // frames: cand, finc, xs, ext, q (a frame adds a distinct candidate: depth < 31)
-    const int d0 = u.depth;
-    uint32_t ext = 0u;
-    bool enter = true;
-    for (;;) {
-        if (enter) {
-            if (u.cand == 0u) {
-                if ((u.finc | u.xs) == 0u) lp_emit(P, shist, o, u.base + (uint32_t)u.depth, u.hs);
-                goto lpop;
-            }
-            ext = lp_pivot_ext(u, o);
-            enter = false;
-        }
-        if (ext == 0u) goto lpop;
-        {
-            const int q = __ffs(ext) - 1;
-            const uint32_t qb = 1u << q;
-            ext &= ~qb;
-            u.cand &= ~qb;
-            u.finc |= qb;
-            uint32_t cc, cf, cx;
-            uint64_t hq;
-            if (!lp_child(P, shist, u, q, o, cc, cf, cx, hq)) continue;
-            uint32_t *f = stk + 5 * (u.depth - d0);
-            f[0] = u.cand;
-            f[1] = u.finc;
-            f[2] = u.xs;
-            f[3] = ext;
-            f[4] = (uint32_t)q;
-            ++u.depth;
-            u.cand = cc;
-            u.finc = cf;
-            u.xs = cx;
-            u.hs += hq;
-            enter = true;
-            continue;
-        }
-    lpop:
-        if (u.depth == d0) break;
-        --u.depth;
-        {
-            const uint32_t *f = stk + 5 * (u.depth - d0);
-            u.cand = f[0];
-            u.finc = f[1];
-            u.xs = f[2];
-            ext = f[3];
-            u.hs -= u.hC[f[4]];
-        }
-    }
-}
-
-__device__ __forceinline__ LpNode lp_root_node(const uint32_t *lp, int r) {
-    const uint32_t *rec = lp + 4 * r;
-    const uint32_t meta = rec[1];
-    LpNode u;
-    u.cn = (int)(meta & 0xffu);
-    const int xn = (int)((meta >> 8) & 0xffu);
-    u.base = meta >> 16;
-    const uint32_t *uni = lp + BK_LP_TABLE_WORDS + rec[0];
-    u.hC = reinterpret_cast<const uint64_t *>(uni);
-    u.akC = reinterpret_cast<const uint2 *>(uni + 2 * u.cn);
-    u.akX = reinterpret_cast<const uint2 *>(uni + 4 * u.cn);
-    u.adjXT = uni + 4 * u.cn + 2 * xn;
-    u.cand = u.cn == 32 ? FULL : ((1u << u.cn) - 1u);
-    u.xs = xn == 32 ? FULL : ((1u << xn) - 1u);
-    u.finc = 0u;
-    u.hs = (uint64_t)rec[2] | ((uint64_t)rec[3] << 32);
-    u.depth = 0;
-    return u;
-}
-
-__device__ __forceinline__ void lp_task_put(uint32_t *t, int r, const LpNode &u) {
-    t[0] = (uint32_t)r | ((uint32_t)u.depth << 8);
-    t[1] = u.cand;
-    t[2] = u.finc;
-    t[3] = u.xs;
-    t[4] = (uint32_t)u.hs;
-    t[5] = (uint32_t)(u.hs >> 32);
-}
-
-__device__ __forceinline__ LpNode lp_task_get(const uint32_t *lp, const uint32_t *t) {
-    LpNode u = lp_root_node(lp, (int)(t[0] & 0xffu));
-    u.depth = (int)(t[0] >> 8);
-    u.cand = t[1];
-    u.finc = t[2];
-    u.xs = t[3];
-    u.hs = (uint64_t)t[4] | ((uint64_t)t[5] << 32);
-    return u;
-}
-
-// Enter node u and put its non-trivial children into the list `dst` (leaves
-// and one-candidate children are settled at once); a child that finds the
-// list full is searched here instead.
-__device__ void lp_expand(const BkParams &P, unsigned long long *shist, LpNode u, int r, LpSums &o, uint32_t *dst,
-                          uint32_t *dst_n, uint32_t cap) {
-    if (u.cand == 0u) {
-        if ((u.finc | u.xs) == 0u) lp_emit(P, shist, o, u.base + (uint32_t)u.depth, u.hs);
-        return;
-    }
-    uint32_t ext = lp_pivot_ext(u, o);
-    while (ext) {
-        const int q = __ffs(ext) - 1;
-        const uint32_t qb = 1u << q;
-        ext &= ~qb;
-        u.cand &= ~qb;
-        u.finc |= qb;
-        uint32_t cc, cf, cx;
-        uint64_t hq;
-        if (!lp_child(P, shist, u, q, o, cc, cf, cx, hq)) continue;
-        LpNode c = u;
-        c.cand = cc;
-        c.finc = cf;
-        c.xs = cx;
-        c.hs = u.hs + hq;
-        c.depth = u.depth + 1;
-        const uint32_t slot = atomicAdd(dst_n, 1u);
-        if (slot < cap) lp_task_put(dst + (int64_t)slot * BK_LP_TASK_WORDS, r, c);
-        else lp_dfs(P, shist, c, o);
-    }
-}
-
-// The buffered small subtrees, searched from one stack of nodes (entered,
-// not yet pivoted) shared by the warp's lanes: each round the lanes take up
-// to 32 nodes off the top together and push the children that are not
-// settled at once; a child that finds the stack full is searched depth
-// first by its lane.
-__device__ __noinline__ LpSums lp_run(const BkParams &P, uint32_t *lp, int nroots, unsigned long long *shist,
-                                      uint32_t *tasks, int lane) {
-    LpSums o = {0ULL, 0ULL, 0u, 0u, 0u};
-    uint32_t *ctr = lp + BK_LP_MAX_ROOTS * 4;   // [0] stack top
-    const uint32_t cap = (uint32_t)P.lp_task_cap;
-    for (int r = lane; r < nroots; r += 32) lp_task_put(tasks + (int64_t)r * BK_LP_TASK_WORDS, r, lp_root_node(lp, r));
-    if (lane == 0) ctr[0] = (uint32_t)nroots;
-    __syncwarp();
-    for (;;) {
-        const uint32_t top = min(ctr[0], cap);
-        if (top == 0u) break;
-        const uint32_t take = min(top, 32u), base = top - take;
-        LpNode u;
-        int r = -1;
+    uint32_t top = (uint32_t)nroots;
+    while (top) {
+        const uint32_t most = top <= 512u ? 32u : top <= 1024u ? 8u : 1u;
+        const uint32_t take = min(top, most);
+        uint32_t base = top - take;
+        __syncwarp();   // the last round's pushes and reads of `node` are done
+        uint32_t n = 0u;
         if ((uint32_t)lane < take) {
-            const uint32_t *t = tasks + (int64_t)(base + (uint32_t)lane) * BK_LP_TASK_WORDS;
-            r = (int)(t[0] & 0xffu);
-            u = lp_task_get(lp, t);
+            const uint4 a = stack[2 * (base + (uint32_t)lane)], b = stack[2 * (base + (uint32_t)lane) + 1];
+            const uint32_t off = a.x & 0xffffu, cn = a.x >> 16;
+            const uint2 *rows = reinterpret_cast<const uint2 *>(arena + off + 2u * cn);
+            const uint32_t ext = lp_pivot_ext(rows, rows + cn, a.y, a.z, a.w);
+            n = (uint32_t)__popc(ext);
+            const uint32_t t = (uint32_t)(__popc(a.y | a.z) + __popc(a.w));
+            o.wops += t + 2u * n * ((t + 31u) >> 5);
+            node[2 * lane] = make_uint4(a.y, a.z, a.w, ext);
+            node[2 * lane + 1] = make_uint4(a.x, b.z, b.x, b.y);
         }
-        __syncwarp();   // every taken record is read before pushes reuse its slot
-        if (lane == 0) ctr[0] = base;
+        // children of the lanes before, and of all
+        uint32_t end = n;
+#pragma unroll
+        for (int s = 1; s < 32; s <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, end, s);
+            if (lane >= s) end += y;
+        }
+        const uint32_t total = __shfl_sync(FULL, end, 31);
         __syncwarp();
-        if (r >= 0) lp_expand(P, shist, u, r, o, tasks, &ctr[0], cap);
-        __syncwarp();
+        for (uint32_t t0 = 0; t0 < total; t0 += 32u) {
+            const uint32_t t = t0 + (uint32_t)lane;
+            // parent: the number of lanes whose children end at or before t
+            int p = 0;
+#pragma unroll
+            for (int s = 16; s; s >>= 1)
+                if (__shfl_sync(FULL, end, p + s - 1) <= t) p += s;
+            uint32_t k = t - __shfl_sync(FULL, end - n, p);
+            bool push = false;
+            uint32_t id = 0u, cc = 0u, cf = 0u, cx = 0u, size = 0u;
+            uint64_t hs = 0ULL;
+            if (t < total) {
+                const uint4 a = node[2 * p], b = node[2 * p + 1];
+                uint32_t e = a.w;
+                for (; k; --k) e &= e - 1u;
+                const uint32_t bit = e & (0u - e), lower = a.w & (bit - 1u);
+                const int q = __ffs(e) - 1;
+                id = b.x;
+                const uint32_t off = id & 0xffffu, cn = id >> 16;
+                const uint64_t *hC = reinterpret_cast<const uint64_t *>(arena + off);
+                const uint2 *rows = reinterpret_cast<const uint2 *>(arena + off + 2u * cn);
+                const uint2 rq = rows[q];
+                cc = a.x & ~lower & rq.x;
+                cf = (a.y | lower) & rq.x;
+                cx = a.z & rq.y;
+                hs = ((uint64_t)b.z | ((uint64_t)b.w << 32)) + hC[q];
+                size = b.y + 1u;
+                const int nc = __popc(cc);
+                if (nc > 2) {
+                    ++o.nodes;
+                    push = true;
+                } else if (nc == 0) {
+                    // a leaf: a maximal clique unless fini is left
+                    ++o.nodes;
+                    if ((cf | cx) == 0u) lp_emit(P, shist, o, size, hs);
+                } else if (nc == 1) {
+                    // one candidate c: one more node and the clique K + q + c, unless a fini
+                    // vertex adjacent to c is the pivot (then no child)
+                    const int c = __ffs(cc) - 1;
+                    const uint2 rc = rows[c];
+                    const uint32_t w = 1u + (uint32_t)(__popc(cf) + __popc(cx));
+                    ++o.nodes;
+                    o.wops += w;
+                    if (((cf & rc.x) | (cx & rc.y)) == 0u) {
+                        ++o.nodes;
+                        o.wops += 2u * ((w + 31u) >> 5);
+                        lp_emit(P, shist, o, size + 1u, hs + hC[c]);
+                    }
+                } else {
+                    lp_two(P, shist, o, rows, rows + cn, hC, size, hs, cc, cf, cx);
+                }
+            }
+            const uint32_t pb = __ballot_sync(FULL, push);
+            if (push) {
+                const uint32_t at = base + (uint32_t)__popc(pb & lanemask_lt());
+                stack[2 * at] = make_uint4(id, cc, cf, cx);
+                stack[2 * at + 1] = make_uint4((uint32_t)hs, (uint32_t)(hs >> 32), size, 0u);
+            }
+            base += (uint32_t)__popc(pb);
+        }
+        top = base;
     }
     return o;
 }
 
 // Run the buffered small subtrees and fold their sums into the task.
-__device__ void lp_flush(const BkParams &P, Ws &s, Acc &acc, unsigned long long *shist, int lane, int &node_tick) {
+__device__ void lp_flush(const BkParams &P, Ws &s, Acc &acc, uint32_t *shist, int lane, int &node_tick) {
     if (s.lp_n == 0) return;
     const int64_t gwarp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    __syncwarp();   // the roots and universes are written
     const LpSums r = lp_run(P, s.lp, s.lp_n, shist, P.lp_tasks + gwarp * (int64_t)P.lp_task_cap * BK_LP_TASK_WORDS,
-                            lane);
-    unsigned long long cnt = r.count, nodes = r.nodes, hsh = r.hash, wops = r.wops;
+                            s.piv, lane);
+    __syncwarp();
     uint32_t smax = r.smax;
+    unsigned long long hsh = r.hash, wops = r.wops;
+    // counts below 2^24 a lane, 2^29 a warp
+    const uint32_t cnt = __reduce_add_sync(FULL, r.count), nodes = __reduce_add_sync(FULL, r.nodes);
+    smax = __reduce_max_sync(FULL, smax);
     for (int o = 16; o; o >>= 1) {
-        cnt += __shfl_xor_sync(FULL, cnt, o);
-        nodes += __shfl_xor_sync(FULL, nodes, o);
         hsh += __shfl_xor_sync(FULL, hsh, o);
         wops += __shfl_xor_sync(FULL, wops, o);
-        smax = max(smax, __shfl_xor_sync(FULL, smax, o));
     }
     acc.t_count += cnt;
     acc.t_hash += hsh;
@@ -1670,7 +1633,8 @@ __device__ void lp_flush(const BkParams &P, Ws &s, Acc &acc, unsigned long long 
         acc.wops += wops;
         if (smax > cold().maxsize) cold().maxsize = smax;
     }
-    node_tick += nodes > 4096ULL ? 4096 : (int)nodes;
+    hist_guard(P, acc, shist, lane);
+    node_tick += nodes > 4096u ? 4096 : (int)nodes;
     s.lp_n = 0;
     s.lp_top = 0;
 }
@@ -1678,28 +1642,30 @@ __device__ void lp_flush(const BkParams &P, Ws &s, Acc &acc, unsigned long long 
 // Relabel the small node (as search_small does) into the arena; the search
 // of its subtree is left to the next lp_flush.
 template <int NR>
-__device__ void lp_enqueue(const BkParams &P, Ws &s, Acc &acc, unsigned long long *shist, int lane, int &node_tick,
-                           int k0, int d, uint64_t hsum, const uint32_t (&rc)[NR], const uint32_t (&rf)[NR],
-                           const int32_t *Fd, int flen) {
+__device__ void lp_enqueue(const BkParams &P, Ws &s, Acc &acc, uint32_t *shist, int lane, int &node_tick, int k0,
+                           int d, uint64_t hsum, const uint32_t (&rc)[NR], const uint32_t (&rf)[NR], const int32_t *Fd,
+                           int flen) {
     SmallU u;
     int32_t gC, cidC, cidX;
     small_relabel<NR>(P, s, lane, rc, rf, Fd, flen, u, gC, cidC, cidX);
     const int need = lp_universe_words(u.cn, u.xn);
     if (s.lp_n == BK_LP_MAX_ROOTS || s.lp_top + need > P.lp_words - BK_LP_TABLE_WORDS)
         lp_flush(P, s, acc, shist, lane, node_tick);
-    // column k of adjX to lane k
+    uint32_t *uni = s.lp + BK_LP_TABLE_WORDS + s.lp_top;
+    uint2 *rows = reinterpret_cast<uint2 *>(uni + 2 * u.cn), *xr = rows + u.cn;
+    if (lane < u.xn) xr[u.posX] = make_uint2(u.adjX, u.beforeC);
+    __syncwarp();
+    // column k of X's rows, in X's order, to lane k
+    const uint32_t row = lane < u.xn ? xr[lane].x : 0u;
     uint32_t adjXT = 0u;
     for (int k = 0; k < u.cn; ++k) {
-        const uint32_t b = __ballot_sync(FULL, (u.adjX >> k) & 1u);
+        const uint32_t b = __ballot_sync(FULL, (row >> k) & 1u);
         if (lane == k) adjXT = b;
     }
-    uint32_t *uni = s.lp + BK_LP_TABLE_WORDS + s.lp_top;
     if (lane < u.cn) {
         reinterpret_cast<uint64_t *>(uni)[lane] = vertex_hash(gC, P.seed);
-        reinterpret_cast<uint2 *>(uni + 2 * u.cn)[lane] = make_uint2(u.adjC, u.tC);
-        uni[4 * u.cn + 2 * u.xn + lane] = adjXT;
+        rows[lane] = make_uint2(u.adjC, adjXT);
     }
-    if (lane < u.xn) reinterpret_cast<uint2 *>(uni + 4 * u.cn)[lane] = make_uint2(u.adjX, u.tX);
     if (lane == 0) {
         uint32_t *rec = s.lp + 4 * s.lp_n;
         rec[0] = (uint32_t)s.lp_top;
@@ -1754,7 +1720,7 @@ __device__ __forceinline__ void frame_load(const Ws &s, int d, int lane, uint32_
 // Frames are written to memory only when a child is pushed, and read back
 // when it is popped.  Returns 0 = done, 1 = stop the launch, 2 = dropped.
 template <int NR>
-__device__ int search(const BkParams &P, Ws &s, const Task &T, Acc &acc, unsigned long long *shist, int lane,
+__device__ int search(const BkParams &P, Ws &s, const Task &T, Acc &acc, uint32_t *shist, int lane,
                       int &node_tick, uint64_t t_start, int32_t root, int k0, bool enter) {
     const int wc = s.wc;
     const bool imce = P.mode == BK_IMCE;
@@ -1926,7 +1892,7 @@ __device__ int search(const BkParams &P, Ws &s, const Task &T, Acc &acc, unsigne
                 node_tick = 0;
                 frame_store<NR>(s, d, lane, rc, rf, re, rx, imce);
                 __syncwarp();
-                const int act = periodic(P, s, T, acc, lane, d, root, t_start);
+                const int act = periodic(P, s, T, acc, shist, lane, d, root, t_start);
                 if (act) return act;
 #pragma unroll
                 for (int r = 0; r < NR; ++r) {   // a hand-over may have shrunk this frame's ext
@@ -2027,7 +1993,7 @@ __device__ int search(const BkParams &P, Ws &s, const Task &T, Acc &acc, unsigne
 // The same search for candidate sets wider than 32 words (more than 1024
 // candidates, which some ranks produce for hubs): frames stay in memory and
 // every set operation loops over its words.  Returns as search<NR>.
-__device__ int search_mem(const BkParams &P, Ws &s, const Task &T, Acc &acc, unsigned long long *shist, int lane,
+__device__ int search_mem(const BkParams &P, Ws &s, const Task &T, Acc &acc, uint32_t *shist, int lane,
                           int &node_tick, uint64_t t_start, int32_t root, int k0, bool enter) {
     const int wc = s.wc;
     int d = 0;
@@ -2108,7 +2074,7 @@ __device__ int search_mem(const BkParams &P, Ws &s, const Task &T, Acc &acc, uns
             enter = false;
             if (node_tick >= acc.tick) {
                 node_tick = 0;
-                const int act = periodic(P, s, T, acc, lane, d, root, t_start);
+                const int act = periodic(P, s, T, acc, shist, lane, d, root, t_start);
                 if (act) return act;
             }
         }
@@ -2167,7 +2133,7 @@ __device__ int search_mem(const BkParams &P, Ws &s, const Task &T, Acc &acc, uns
 }
 
 // Run one task to completion.  Returns false when the launch must stop.
-__device__ bool run_task(const BkParams &P, Ws &s, const Task &T, Acc &acc, unsigned long long *shist,
+__device__ bool run_task(const BkParams &P, Ws &s, const Task &T, Acc &acc, uint32_t *shist,
                          uint32_t *ws_smem, uint32_t *ws_glob, const uint32_t *taskbuf, int lane,
                          int32_t &built, int &node_tick, uint64_t t_start) {
     const int32_t root = T.root;
@@ -2309,20 +2275,21 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
         if ((int32_t)smid >= P.sm_limit) return;
     }
     extern __shared__ __align__(16) uint32_t smem[];
-    unsigned long long *shist = reinterpret_cast<unsigned long long *>(smem);   // 256 bins
+    uint32_t *shist = smem;   // 256 bins
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int nw_block = blockDim.x >> 5;
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) shist[i] = 0ULL;
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) shist[i] = 0u;
     __syncthreads();
-    uint32_t *ws_smem = smem + 512 + (int64_t)nw_block * BK_PIV_WORDS + (int64_t)wib * P.smem_words;
-    uint32_t *lp_smem = smem + 512 + (int64_t)nw_block * (BK_PIV_WORDS + P.smem_words) + (int64_t)wib * P.lp_words;
+    uint32_t *ws_smem = smem + BK_HIST_WORDS + (int64_t)nw_block * BK_PIV_WORDS + (int64_t)wib * P.smem_words;
+    uint32_t *lp_smem = smem + BK_HIST_WORDS + (int64_t)nw_block * (BK_PIV_WORDS + P.smem_words) + (int64_t)wib * P.lp_words;
     const int64_t gwarp = (int64_t)blockIdx.x * nw_block + wib;
     uint32_t *ws_glob = P.gws + gwarp * P.gws_words;
     uint32_t *taskbuf = P.taskbuf + gwarp * P.slot_words;
     Acc acc = {0, 0, 0, 0, 64, 4, 0};
     if (lane == 0) cold() = AccCold{};
+    __syncwarp();
     Ws s;
-    s.piv = smem + 512 + (int64_t)wib * BK_PIV_WORDS;
+    s.piv = smem + BK_HIST_WORDS + (int64_t)wib * BK_PIV_WORDS;
     s.lp = lp_smem;
     s.lp_n = s.lp_top = 0;
     int32_t built = -1;
@@ -2417,10 +2384,11 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
         T.kdepth = __shfl_sync(FULL, T.kdepth, 0);
         T.rec = __shfl_sync(FULL, T.rec, 0);
         acc.t_count = acc.t_hash = acc.t_nodes = 0;
-        if (lane == 0) cold().t_rep = cold().t_split = 0;
+        if (lane == 0) cold().t_rep = cold().t_split = cold().t_hist = 0;
         const uint64_t t0 = globaltimer_ns();
         if (lane == 0) cold().t_split_ns = t0;
         const bool go_on = run_task(P, s, T, acc, shist, ws_smem, ws_glob, taskbuf, lane, built, node_tick, t_start);
+        hist_guard(P, acc, shist, lane);
         if (lane == 0) cold().max_busy += globaltimer_ns() - t0;
         if (lane == 0) {
             AccCold &c = cold();
@@ -2475,7 +2443,7 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 256; i += blockDim.x)
-        if (shist[i]) atomicAdd(&P.out[OUT_HIST + i], shist[i]);
+        if (shist[i]) atomicAdd(&P.out[OUT_HIST + i], (unsigned long long)shist[i]);
 }
 
 }  // namespace

@@ -143,21 +143,23 @@ __host__ __device__ inline int64_t bk_shared_words(int64_t w, int64_t c) {
 constexpr int BK_PIV_WORDS = 64 + 256 + 96;
 
 // Lane-parallel small search: per warp a table of up to BK_LP_MAX_ROOTS
-// relabelled small nodes (4 words each, then the next-root counter) and an
-// arena for their universes.
+// relabelled small nodes (4 words each) and an arena for their universes.
 constexpr int BK_LP_MAX_ROOTS = 64;
-constexpr int BK_LP_TABLE_WORDS = BK_LP_MAX_ROOTS * 4 + 4;
-// A node of a small subtree waiting for a lane: root index | depth << 8,
-// cand, finc, xs, hash sum (2 words).
-constexpr int BK_LP_TASK_WORDS = 6;
+constexpr int BK_LP_TABLE_WORDS = BK_LP_MAX_ROOTS * 4;
+// A node of a small subtree waiting for its pivot, two 16-byte halves: (arena
+// offset | cn << 16, cand, finc, xs), (hash sum, clique size, unused).
+constexpr int BK_LP_TASK_WORDS = 8;
 constexpr int BK_LP_TASK_CAP = 2048;
 
-// Dynamic shared memory of one search block: 256 histogram bins, the pivot
+// 32-bit bins of the clique sizes below 256 that a block counts in shared memory
+constexpr int BK_HIST_WORDS = 256;
+
+// Dynamic shared memory of one search block: the histogram bins, the pivot
 // scratch of every warp, the optional per-warp workspace slots, then the
 // per-warp regions of the lane-parallel small search.
 __host__ __device__ inline int64_t bk_block_smem_bytes(int32_t warps_per_block, int32_t smem_words,
                                                        int32_t lp_words) {
-    return (int64_t)512 * 4 + (int64_t)warps_per_block * (BK_PIV_WORDS + smem_words + lp_words) * 4;
+    return (int64_t)BK_HIST_WORDS * 4 + (int64_t)warps_per_block * (BK_PIV_WORDS + smem_words + lp_words) * 4;
 }
 
 // Frames of the explicit stack: one per clique vertex beyond the seeds,

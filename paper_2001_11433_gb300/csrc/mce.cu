@@ -233,7 +233,7 @@ LaunchShape launch_shape(const mce_opts *o) {
         int64_t lp = (per_block - 2048) / 4 / ls.warps_per_block - BK_PIV_WORDS - ls.smem_words;
         if (lp > 2048) lp = 2048;
         if (o && o->lane_search_words > 0 && o->lane_search_words < lp) lp = o->lane_search_words;
-        lp &= ~int64_t(1);
+        lp &= ~int64_t(3);   // 16-byte aligned regions
         ls.lp_words = lp >= 512 ? (int32_t)lp : 0;
     }
     // the ring's sequence numbers tell "published for ticket p" (p + 1) from

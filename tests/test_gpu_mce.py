@@ -553,6 +553,22 @@ def test_stream_rmat12_summary(gpu_lib):
     assert total[0] == r.count and total[1] == r.count + sum(i * int(c) for i, c in enumerate(r.hist))
 
 
+@pytest.mark.parametrize("parts", [(8, 7), (5, 8), (2, 18)])
+def test_lane_stack_of_wide_universes(gpu_lib, parts):
+    """Complete multipartite graphs: universes of 32 candidates whose nodes push
+    many children each, so that fewer nodes are taken from the lanes' stack."""
+    mce = gpu_lib
+    size, k = parts
+    n = size * k
+    i, j = np.triu_indices(n, 1)
+    keep = i // size != j // size
+    g = gpu_graph(mce, n, i[keep], j[keep])
+    r = mce.enumerate_cliques(g)
+    w = mce.enumerate_cliques(g, warp_small_search=True)
+    assert r.count == size ** k and r.hist[k] == size ** k
+    assert (r.hash, r.tree_nodes, r.word_ops) == (w.hash, w.tree_nodes, w.word_ops)
+
+
 @pytest.mark.parametrize("rank", ["degen", "degree"])
 def test_lane_search_equals_warp_search(gpu_lib, rank):
     """The lane-parallel small search (nodes taken by the lanes from a shared
