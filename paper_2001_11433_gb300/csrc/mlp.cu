@@ -7,7 +7,7 @@
 // per-vertex features predicts log(1 + search-tree nodes) of the vertex's
 // subproblem, trained on node counts recorded by the search itself.
 //
-//   k_features    per-vertex features (warp per vertex)
+//   k_features    per-vertex features (eight lanes a vertex, a block a hub)
 //   k_mlp_fwd, k_mlp_fwd_bf16   inference, FP32 or BF16 weights and activations
 //                 (FP32 sums)
 //   k_mlp_grad    forward + backward of the MSE loss over tiles of rows as
@@ -56,87 +56,130 @@ __host__ __device__ inline Off offsets(int H) {
 
 // ------------------------------------------------------------------ features
 
-__global__ void k_features(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
-                           const int64_t *__restrict__ core, const int64_t *__restrict__ tri,
-                           const int32_t *__restrict__ up_ptr, int32_t n, float *feat) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = warp; v < n; v += nwarps) {
-        const int32_t e0 = row_ptr[v], e1 = row_ptr[v + 1], d = e1 - e0;
-        float s = 0.f, s2 = 0.f, mx = 0.f;
-        for (int32_t e = e0 + lane; e < e1; e += 32) {
-            const int32_t w = col[e];
-            const float x = log1pf((float)(row_ptr[w + 1] - row_ptr[w]));
-            s += x;
-            s2 += x * x;
-            mx = fmaxf(mx, x);
+// Degree statistics of a vertex's neighbours.  A neighbour w ranks higher than
+// v by degree when (d(w), w) > (d(v), v).
+struct NbrSums {
+    float s = 0.f, s2 = 0.f, mx = 0.f, mins = 0.f, dsum = 0.f;
+    int hi = 0;
+    template <bool LIGHT>
+    __device__ __forceinline__ void add(const int32_t *__restrict__ row_ptr, int32_t w, int32_t v, int32_t d) {
+        const int32_t dw = row_ptr[w + 1] - row_ptr[w];
+        const float x = log1pf((float)dw);
+        s += x;
+        s2 += x * x;
+        mx = fmaxf(mx, x);
+        if (LIGHT) {
+            mins += (float)min(dw, d);
+            dsum += (float)dw;
+            hi += (dw > d || (dw == d && w > v)) ? 1 : 0;
         }
-        for (int o = 16; o; o >>= 1) {
+    }
+    // sum over the lanes that differ in the bits of `from`, `from` / 2, ... 1
+    template <bool LIGHT> __device__ __forceinline__ void reduce(int from) {
+        for (int o = from; o; o >>= 1) {
             s += __shfl_xor_sync(0xffffffffu, s, o);
             s2 += __shfl_xor_sync(0xffffffffu, s2, o);
             mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+            if (LIGHT) {
+                mins += __shfl_xor_sync(0xffffffffu, mins, o);
+                dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
+                hi += __shfl_xor_sync(0xffffffffu, hi, o);
+            }
         }
-        if (lane == 0) {
-            float *f = feat + v * kFeat;
-            const float mean = d ? s / d : 0.f;
-            const float var = d ? fmaxf(s2 / d - mean * mean, 0.f) : 0.f;
-            f[0] = log1pf((float)d);
-            f[1] = (float)core[v];
-            f[2] = log1pf((float)tri[v]);
-            f[3] = mean;
-            f[4] = sqrtf(var);
-            f[5] = mx;
-            f[6] = log1pf((float)(up_ptr[v + 1] - up_ptr[v]));
-            f[7] = d >= 2 ? (float)(2.0 * (double)tri[v] / ((double)d * (d - 1))) : 0.f;
+    }
+};
+
+struct FeatParams {
+    const int32_t *row_ptr, *col;
+    const int64_t *core, *tri;   // MCE_FEATURES_FULL
+    const int32_t *up_ptr;       //
+    int32_t n;
+    int32_t *hubs, *n_hubs;
+    float *feat;
+};
+
+// feature k of vertex v from its reduced sums
+template <bool LIGHT>
+__device__ __forceinline__ float feature(const FeatParams &P, int64_t v, int32_t d, const NbrSums &a, int k) {
+    const float mean = d ? a.s / d : 0.f;
+    const float var = d ? fmaxf(a.s2 / d - mean * mean, 0.f) : 0.f;
+    if (LIGHT) {   // MCE_FEATURES_LIGHT: one pass, degrees only
+        switch (k) {
+            case 0: return log1pf((float)d);
+            case 1: return mean;
+            case 2: return sqrtf(var);
+            case 3: return a.mx;
+            case 4: return log1pf((float)a.hi);
+            case 5: return log1pf(a.mins * 0.5f);
+            case 6: return d ? (float)a.hi / (float)d : 0.f;
+            default: return log1pf(a.dsum);
         }
+    }
+    switch (k) {
+        case 0: return log1pf((float)d);
+        case 1: return (float)P.core[v];
+        case 2: return log1pf((float)P.tri[v]);
+        case 3: return mean;
+        case 4: return sqrtf(var);
+        case 5: return a.mx;
+        case 6: return log1pf((float)(P.up_ptr[v + 1] - P.up_ptr[v]));
+        default: return d >= 2 ? (float)(2.0 * (double)P.tri[v] / ((double)d * (d - 1))) : 0.f;
     }
 }
 
-// One-pass features (MCE_FEATURES_LIGHT): degrees of the vertex and its
-// neighbours only.  A neighbour w ranks higher than v by degree when
-// (d(w), w) > (d(v), v).
-__global__ void k_features_light(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, int32_t n,
-                                 float *feat) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t v = warp; v < n; v += nwarps) {
-        const int32_t e0 = row_ptr[v], e1 = row_ptr[v + 1], d = e1 - e0;
-        float s = 0.f, s2 = 0.f, mx = 0.f, mins = 0.f, dsum = 0.f;
-        int hi = 0;
-        for (int32_t e = e0 + lane; e < e1; e += 32) {
-            const int32_t w = col[e];
-            const int32_t dw = row_ptr[w + 1] - row_ptr[w];
-            const float x = log1pf((float)dw);
-            s += x;
-            s2 += x * x;
-            mx = fmaxf(mx, x);
-            mins += (float)min(dw, d);
-            dsum += (float)dw;
-            hi += (dw > d || (dw == d && w > (int32_t)v)) ? 1 : 0;
+// Eight lanes a vertex, one feature a lane at the end; vertices of more than
+// kFeatHub neighbours are left to k_features_hubs, a block each.  Bound: L2
+// (two gathers a neighbour).  A warp per vertex left most lanes of short rows
+// idle and took 0.99 ms on the 1.7M-vertex graph, waiting for the hubs; both
+// kernels together take 0.31 ms.
+constexpr int kFeatHub = 512;
+
+template <bool LIGHT> __global__ void k_features(FeatParams P) {
+    const int lane = threadIdx.x & 31, k = lane & 7;
+    const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
+    for (int64_t w0 = g0 - (lane >> 3); w0 < P.n; w0 += stride) {   // the same for the whole warp
+        const int64_t v = w0 + (lane >> 3);
+        int32_t e0 = 0, d = 0;
+        if (v < P.n) {
+            e0 = P.row_ptr[v];
+            d = P.row_ptr[v + 1] - e0;
         }
-        for (int o = 16; o; o >>= 1) {
-            s += __shfl_xor_sync(0xffffffffu, s, o);
-            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            mins += __shfl_xor_sync(0xffffffffu, mins, o);
-            dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-            hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        const bool hub = d > kFeatHub;
+        NbrSums a;
+        if (!hub) {
+#pragma unroll 4
+            for (int32_t e = k; e < d; e += 8) a.add<LIGHT>(P.row_ptr, P.col[e0 + e], (int32_t)v, d);
+        } else if (k == 0) {
+            P.hubs[atomicAdd(P.n_hubs, 1)] = (int32_t)v;
         }
-        if (lane == 0) {
-            float *f = feat + v * kFeat;
-            const float mean = d ? s / d : 0.f;
-            const float var = d ? fmaxf(s2 / d - mean * mean, 0.f) : 0.f;
-            f[0] = log1pf((float)d);
-            f[1] = mean;
-            f[2] = sqrtf(var);
-            f[3] = mx;
-            f[4] = log1pf((float)hi);
-            f[5] = log1pf(mins * 0.5f);
-            f[6] = d ? (float)hi / (float)d : 0.f;
-            f[7] = log1pf(dsum);
+        __syncwarp();
+        a.reduce<LIGHT>(4);
+        if (v < P.n && !hub) P.feat[v * kFeat + k] = feature<LIGHT>(P, v, d, a, k);
+    }
+}
+
+template <bool LIGHT> __global__ void __launch_bounds__(512) k_features_hubs(FeatParams P) {
+    __shared__ __align__(8) unsigned char raw[16 * sizeof(NbrSums)];
+    NbrSums *part = reinterpret_cast<NbrSums *>(raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int32_t n_hubs = *P.n_hubs;
+    for (int32_t i = blockIdx.x; i < n_hubs; i += gridDim.x) {
+        const int32_t v = P.hubs[i];
+        const int32_t e0 = P.row_ptr[v], d = P.row_ptr[v + 1] - e0;
+        NbrSums a;
+#pragma unroll 4
+        for (int32_t e = threadIdx.x; e < d; e += 512) a.add<LIGHT>(P.row_ptr, P.col[e0 + e], v, d);
+        __syncwarp();
+        a.reduce<LIGHT>(16);
+        if (lane == 0) part[warp] = a;
+        __syncthreads();
+        if (warp == 0) {
+            a = lane < 16 ? part[lane] : NbrSums();
+            a.reduce<LIGHT>(8);
+            if (lane < kFeat) P.feat[(int64_t)v * kFeat + lane] = feature<LIGHT>(P, v, d, a, lane);
         }
+        __syncthreads();
     }
 }
 
@@ -671,11 +714,23 @@ int32_t model_feature_kind(const mce_model *m) { return m ? m->feature_kind : 0;
 mce_status features(const mce_graph *g, int32_t kind, cudaStream_t s, float *feat) {
     const int32_t n = g->n;
     if (n == 0) return MCE_OK;
+    FeatParams P{};
+    P.row_ptr = g->row_ptr;
+    P.col = g->col;
+    P.n = n;
+    P.feat = feat;
+    const int64_t max_hubs = g->nnz / kFeatHub;
+    DevBuf hubs, core, tri, deg, drank, up_ptr, up_col;
+    MCE_TRY(hubs.alloc((size_t)(max_hubs + 1) * 4, s));
+    MCE_CUDA(cudaMemsetAsync(hubs.p, 0, 4, s));
+    P.n_hubs = hubs.as<int32_t>();
+    P.hubs = P.n_hubs + 1;
+    const unsigned hub_blocks = (unsigned)(max_hubs < 2 * num_sms() ? max_hubs : 2 * num_sms());
     if (kind == MCE_FEATURES_LIGHT) {
-        MCE_LAUNCH(k_features_light, grid_for((int64_t)n * 32, 256), 256, 0, s, g->row_ptr, g->col, n, feat);
+        MCE_LAUNCH(k_features<true>, grid_for((int64_t)n * 8, 256), 256, 0, s, P);
+        if (hub_blocks) MCE_LAUNCH(k_features_hubs<true>, hub_blocks, 512, 0, s, P);
         return MCE_OK;
     }
-    DevBuf core, tri, deg, drank, up_ptr, up_col;
     MCE_TRY(core.alloc((size_t)n * 8, s));
     MCE_TRY(tri.alloc((size_t)n * 8, s));
     MCE_TRY(deg.alloc((size_t)n * 8, s));
@@ -686,8 +741,11 @@ mce_status features(const mce_graph *g, int32_t kind, cudaStream_t s, float *fea
     MCE_TRY(rank_from_key_i64(deg.as<int64_t>(), n, g->id_bits, vertex_key_bits(g, MCE_RANK_DEGREE), s,
                               drank.as<int32_t>()));
     MCE_TRY(build_up_lists(g, drank.as<int32_t>(), s, up_ptr, up_col));
-    MCE_LAUNCH(k_features, grid_for((int64_t)n * 32, 256), 256, 0, s, g->row_ptr, g->col, core.as<int64_t>(),
-               tri.as<int64_t>(), up_ptr.as<int32_t>(), n, feat);
+    P.core = core.as<int64_t>();
+    P.tri = tri.as<int64_t>();
+    P.up_ptr = up_ptr.as<int32_t>();
+    MCE_LAUNCH(k_features<false>, grid_for((int64_t)n * 8, 256), 256, 0, s, P);
+    if (hub_blocks) MCE_LAUNCH(k_features_hubs<false>, hub_blocks, 512, 0, s, P);
     return MCE_OK;
 }
 
