@@ -224,8 +224,10 @@ struct HubShared {
     int32_t active[kHubThreads], n_active, red[kHubWarps], found, kept, at;
 };
 
+// (barrier.sync, not bar.sync: the lanes of a warp may arrive one after the other)
 __device__ __forceinline__ void hub_sync(int bar) {
-    asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(kHubThreads) : "memory");
+    __syncwarp();
+    asm volatile("barrier.sync %0, %1;" ::"r"(bar), "n"(kHubThreads) : "memory");
 }
 
 __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, int32_t i, int32_t round, int bar) {
