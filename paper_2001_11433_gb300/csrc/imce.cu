@@ -209,16 +209,57 @@ __device__ __forceinline__ uint64_t list_hash(const int32_t *vs, int32_t s, uint
     return clique_hash_from_sum(h, (uint32_t)s);
 }
 
-// append listed cliques to the pool (ids base_id..) and the table
-__global__ void k_index_insert(const int64_t *loff, const int32_t *lvtx, int64_t nc, int64_t base_id, int64_t pool_base,
-                               const int64_t *woff, int32_t *pool, int64_t *off, int32_t *alive,
-                               unsigned long long *tkey, int32_t *tid, int64_t tmask, uint64_t seed) {
+// Listed cliques that the index still holds as a dead entry (an update that
+// takes back an earlier one creates the same cliques again): back[c] = its id,
+// else -1; fresh[c] and words[c] = 1 and the words of a new entry, or 0.
+// Without this every such update left its cliques behind once more, and the
+// probes of equal keys ran over all of them.
+__global__ void k_index_match(const int64_t *loff, const int32_t *lvtx, int64_t nc, const int32_t *pool,
+                              const int64_t *off, const int32_t *alive, const unsigned long long *tkey,
+                              const int32_t *tid, int64_t tmask, uint64_t seed, int32_t *back, int64_t *fresh,
+                              int64_t *words) {
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t *src = lvtx + loff[c];
+        const int32_t s = src[0];
+        const uint64_t h = list_hash(src + 1, s, seed);
+        int32_t found = -1;
+        int64_t slot = (int64_t)(h & (uint64_t)tmask);
+        for (int64_t probe = 0; tid && probe <= tmask; ++probe) {
+            const int32_t id1 = tid[slot];
+            if (id1 == 0) break;
+            if (tkey[slot] == h && !alive[id1 - 1]) {
+                const int32_t *pl = pool + off[id1 - 1];
+                bool eq = pl[0] == s;
+                for (int i = 1; i <= s && eq; ++i) eq = pl[i] == src[i];
+                if (eq) {
+                    found = id1 - 1;
+                    break;
+                }
+            }
+            slot = (slot + 1) & tmask;
+        }
+        back[c] = found;
+        fresh[c] = found < 0;
+        words[c] = found < 0 ? (int64_t)s + 1 : 0;
+    }
+}
+
+// listed cliques into the index: dead entries come alive again, the others
+// are appended to the pool (ids base_id + their place among them) and the table
+__global__ void k_index_insert(const int64_t *loff, const int32_t *lvtx, int64_t nc, int64_t base_id, int64_t pool_base,
+                               const int32_t *back, const int64_t *place, const int64_t *woff, int32_t *pool,
+                               int64_t *off, int32_t *alive, unsigned long long *tkey, int32_t *tid, int64_t tmask,
+                               uint64_t seed) {
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x) {
+        if (back[c] >= 0) {
+            alive[back[c]] = 1;
+            continue;
+        }
         const int32_t *src = lvtx + loff[c];
         const int32_t s = src[0];
         const int64_t dst = pool_base + woff[c];
         for (int i = 0; i <= s; ++i) pool[dst + i] = src[i];
-        const int64_t id = base_id + c;
+        const int64_t id = base_id + place[c];
         off[id] = dst;
         alive[id] = 1;
         const uint64_t h = list_hash(src + 1, s, seed);
@@ -231,11 +272,6 @@ __global__ void k_index_insert(const int64_t *loff, const int32_t *lvtx, int64_t
             slot = (slot + 1) & tmask;
         }
     }
-}
-
-__global__ void k_list_sizes(const int64_t *loff, const int32_t *lvtx, int64_t nc, int64_t *words) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += (int64_t)gridDim.x * blockDim.x)
-        words[c] = lvtx[loff[c]] + 1;
 }
 
 // re-insert every id into a fresh table (after growing it)
@@ -1142,23 +1178,28 @@ mce_status index_reserve_table(CliqueIndex &I, int64_t n_ids_after, cudaStream_t
 mce_status index_append(CliqueIndex &I, const int64_t *loff, const int32_t *lvtx, int64_t nc, cudaStream_t s,
                         uint64_t seed) {
     if (nc == 0) return MCE_OK;
-    DevBuf words;
-    MCE_TRY(words.alloc((size_t)(nc + 1) * 8, s));
-    MCE_LAUNCH(k_list_sizes, grid_for(nc, 256), 256, 0, s, loff, lvtx, nc, words.as<int64_t>());
-    MCE_TRY(exclusive_scan_i64(words.as<int64_t>(), words.as<int64_t>(), nc, s));
-    int64_t tot = 0;
-    MCE_CUDA(cudaMemcpyAsync(&tot, words.as<int64_t>() + nc, 8, cudaMemcpyDeviceToHost, s));
+    DevBuf back, buf;
+    MCE_TRY(back.alloc((size_t)nc * 4, s));
+    MCE_TRY(buf.alloc((size_t)(nc + 1) * 16, s));
+    int64_t *words = buf.as<int64_t>(), *place = words + nc + 1;
+    MCE_LAUNCH(k_index_match, grid_for(nc, 256), 256, 0, s, loff, lvtx, nc, I.pool, I.off, I.alive, I.tkey, I.tid,
+               I.tcap - 1, seed, back.as<int32_t>(), place, words);
+    MCE_TRY(exclusive_scan_i64(words, words, nc, s));
+    MCE_TRY(exclusive_scan_i64(place, place, nc, s));
+    int64_t tot = 0, fresh = 0;
+    MCE_CUDA(cudaMemcpyAsync(&tot, words + nc, 8, cudaMemcpyDeviceToHost, s));
+    MCE_CUDA(cudaMemcpyAsync(&fresh, place + nc, 8, cudaMemcpyDeviceToHost, s));
     MCE_CUDA(cudaStreamSynchronize(s));
     MCE_TRY(grow(I.pool, I.pool_cap, I.pool_words + tot, I.pool_words, s));
     int64_t cap2 = I.ids_cap;
-    MCE_TRY(grow(I.off, cap2, I.n_ids + nc, I.n_ids, s));
+    MCE_TRY(grow(I.off, cap2, I.n_ids + fresh, I.n_ids, s));
     int64_t cap3 = I.ids_cap;
-    MCE_TRY(grow(I.alive, cap3, I.n_ids + nc, I.n_ids, s));
+    MCE_TRY(grow(I.alive, cap3, I.n_ids + fresh, I.n_ids, s));
     I.ids_cap = cap2;
-    MCE_TRY(index_reserve_table(I, I.n_ids + nc, s, seed));
+    MCE_TRY(index_reserve_table(I, I.n_ids + fresh, s, seed));
     MCE_LAUNCH(k_index_insert, grid_for(nc, 256), 256, 0, s, loff, lvtx, nc, I.n_ids, I.pool_words,
-               words.as<int64_t>(), I.pool, I.off, I.alive, I.tkey, I.tid, I.tcap - 1, seed);
-    I.n_ids += nc;
+               back.as<int32_t>(), place, words, I.pool, I.off, I.alive, I.tkey, I.tid, I.tcap - 1, seed);
+    I.n_ids += fresh;
     I.pool_words += tot;
     I.n_alive += nc;
     return MCE_OK;

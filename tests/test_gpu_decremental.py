@@ -261,3 +261,26 @@ def test_more_than_256_endpoints_in_one_clique_is_refused(gpu_lib):
     assert st.cliques(16, 1024) == before
     row1, col1 = st.graph().csr()
     assert np.array_equal(np.asarray(row0), np.asarray(row1)) and np.array_equal(np.asarray(col0), np.asarray(col1))
+
+
+@pytest.mark.parametrize("n,p", [(12, 0.9), (40, 0.4)])
+def test_edges_out_and_in_again(gpu_lib, n, p):
+    """Cliques that come back after their deletion are dead entries of the
+    index until then, some of them deleted through a different batch."""
+    mce, rng = gpu_lib, random.Random(n)
+    pairs = [e for e in itertools.combinations(range(n), 2) if rng.random() < p]
+    g, og = _pairs_graph(mce, n, pairs)
+    st = mce.Imce(g)
+    whole = st.cliques(1 << 16, 1 << 20)
+    assert whole == O.ttt_whole(og, want_list=True).cliques
+    for i in range(8):
+        cut = rng.sample(pairs, rng.randint(1, len(pairs) // 2))
+        a, b = (np.array(x, np.int32) for x in zip(*cut))
+        d = st.remove_edges(a, b)
+        left = _pairs_graph(mce, n, sorted(set(pairs) - set(cut)))[1]
+        want = O.ttt_whole(left, want_list=True)
+        assert st.cliques(1 << 16, 1 << 20) == want.cliques and d.alive == want.count
+        back = st.add_edges(a, b)
+        assert (back.new_count, back.new_hash, back.sub_count, back.sub_hash) == (d.sub_count, d.sub_hash, d.new_count,
+                                                                                  d.new_hash)
+        assert st.cliques(1 << 16, 1 << 20) == whole and back.alive == len(whole)
