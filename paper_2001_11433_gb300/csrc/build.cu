@@ -35,7 +35,7 @@ constexpr int kWarpSlots = 256;
 // Γ+ lists more than this many times longer than C (hubs) have the candidates
 // searched in them instead of their elements looked up in C
 constexpr int kReverse = 8;
-constexpr int kFlat = 4;
+constexpr int kFlat = 4;   // elements a lane looks up at a time
 
 struct WarpSmem {
     int32_t key[kWarpSlots];
@@ -97,36 +97,71 @@ __device__ __forceinline__ Parts parts_of(uint32_t *base, int32_t w, int32_t c) 
 
 __device__ __forceinline__ uint32_t slot_of(int32_t y, int shift) { return ((uint32_t)y * 0x9E3779B1u) >> shift; }
 
-// table of 2^(32 - shift) slots, at most half full: index of y, or -1
+// The loops below run until a vote of the whole warp ends them and have no
+// other exit: with a loop that each lane left by its own return, lanes with a
+// long chain of slots came out of it apart from their warp, and the shuffles
+// after it gave them wrong owners (a row of a subproblem in some 10^5 lost its
+// bits, in some runs).
+
+// table of 2^(32 - shift) slots, at most half full: j[u] = index of y[u], or
+// -1 (also for y[u] = -1); the whole warp
 template <class I>
-__device__ __forceinline__ int find(const int32_t *key, const I *idx, int shift, uint32_t mask, int32_t y) {
-    for (uint32_t s = slot_of(y, shift);; s = (s + 1) & mask) {
-        const int32_t k = key[s];
-        if (k == y) return idx[s];
-        if (k < 0) return -1;
+__device__ __forceinline__ void find(const int32_t *key, const I *idx, int shift, uint32_t mask,
+                                     const int32_t (&y)[kFlat], int (&j)[kFlat]) {
+    uint32_t s[kFlat];
+    bool open[kFlat], any = false;
+#pragma unroll
+    for (int u = 0; u < kFlat; ++u) {
+        s[u] = slot_of(y[u], shift);
+        j[u] = -1;
+        open[u] = y[u] >= 0;
+        any |= open[u];
+    }
+    while (__any_sync(FULL, any)) {
+        any = false;
+        int32_t k[kFlat];
+#pragma unroll
+        for (int u = 0; u < kFlat; ++u) k[u] = open[u] ? key[s[u]] : -1;
+#pragma unroll
+        for (int u = 0; u < kFlat; ++u) {
+            if (open[u] && k[u] == y[u]) j[u] = idx[s[u]];
+            open[u] = open[u] && k[u] >= 0 && k[u] != y[u];
+            any |= open[u];
+            s[u] = (s[u] + 1) & mask;
+        }
     }
 }
 
+// y (-1 = none) with index i into the table; the whole warp
 template <class I>
 __device__ __forceinline__ void insert(int32_t *key, I *idx, int shift, uint32_t mask, int32_t y, int i) {
     uint32_t s = slot_of(y, shift);
-    while (atomicCAS(&key[s], -1, y) != -1) s = (s + 1) & mask;
-    idx[s] = (I)i;
+    bool open = y >= 0;
+    while (__any_sync(FULL, open)) {
+        if (open && atomicCAS(&key[s], -1, y) == -1) {
+            idx[s] = (I)i;
+            open = false;
+        }
+        s = (s + 1) & mask;
+    }
 }
 
-// position of y in sorted g[0..n), or -1
+// position of y in sorted g[0..n), or -1 (n = 0 for a lane without a search);
+// the whole warp
 __device__ __forceinline__ int search(const int32_t *g, int n, int32_t y) {
     int lo = 0, hi = n;
-    while (lo < hi) {
+    while (__any_sync(FULL, lo < hi)) {
         const int mid = (lo + hi) >> 1;
-        if (g[mid] < y) lo = mid + 1; else hi = mid;
+        const bool less = lo < hi && g[mid] < y;
+        if (less) lo = mid + 1;
+        else if (lo < hi) hi = mid;
     }
     return lo < n && g[lo] == y ? lo : -1;
 }
 
 // For the 32 local vertices whose global ids the lanes hold (gx, -1 = none;
 // lane l has local id x0 + l): hit(x, j) for every candidate j in Γ+(x).
-// lookup(y) = candidate index of y or -1; cand(j) = global id of candidate j.
+// lookup(y, j): candidate indices of the y[u], or -1; cand(j) = global id of candidate j.
 template <class Lookup, class Cand, class Hit>
 __device__ __forceinline__ void flat_lists(const BuildParams &P, int32_t gx, int x0, int c, int lane, Lookup lookup,
                                            Cand cand, Hit hit) {
@@ -162,19 +197,17 @@ __device__ __forceinline__ void flat_lists(const BuildParams &P, int32_t gx, int
             at[u] = __shfl_sync(FULL, from, o) + t;
             y[u] = t < total && !((revs >> o) & 1u) ? P.up_col[at[u]] : -1;
         }
+        int j[kFlat];
+        lookup(y, j);
 #pragma unroll
         for (int u = 0; u < kFlat; ++u) {
             if (revs) {
                 const int32_t s0 = __shfl_sync(FULL, e0, own[u]), dd = __shfl_sync(FULL, d, own[u]);
-                if (t0 + 32 * u + lane < total && ((revs >> own[u]) & 1u)) {
-                    const int j = at[u] - s0;
-                    if (search(P.up_col + s0, dd, cand(j)) >= 0) hit(x0 + own[u], j);
-                }
+                const bool mine = t0 + 32 * u + lane < total && ((revs >> own[u]) & 1u);
+                const int q = mine ? at[u] - s0 : 0;
+                if (search(P.up_col + s0, mine ? dd : 0, cand(q)) >= 0) j[u] = q;
             }
-            if (y[u] >= 0) {
-                const int j = lookup(y[u]);
-                if (j >= 0) hit(x0 + own[u], j);
-            }
+            if (j[u] >= 0) hit(x0 + own[u], j[u]);
         }
     }
 }
@@ -222,28 +255,39 @@ __device__ void build_by_warp(const BuildParams &P, WarpSmem &m, const Parts &p,
     for (int s = lane; s <= (int)mask; s += 32) m.key[s] = -1;
     for (int k = lane; k < w; k += 32) *reinterpret_cast<uint4 *>(m.row + k * kWarpS) = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
-    for (int i = lane; i < c; i += 32) {
-        const int32_t y = P.up_col[u0 + i];
-        m.gid[i] = y;
+    for (int i0 = 0; i0 < c; i0 += 32) {
+        const int i = i0 + lane;
+        const int32_t y = i < c ? P.up_col[u0 + i] : -1;
+        if (i < c) m.gid[i] = y;
         insert(m.key, m.idx, shift, mask, y, i);
     }
     __syncwarp();
+    auto lookup = [&](const int32_t (&y)[kFlat], int (&j)[kFlat]) { find(m.key, m.idx, shift, mask, y, j); };
     // the other neighbours rank below v
     int out = c;
-    for (int b0 = 0; b0 < w; b0 += 32) {
-        const int32_t x = b0 + lane < w ? P.col[r0 + b0 + lane] : 0;
-        const bool low = b0 + lane < w && find(m.key, m.idx, shift, mask, x) < 0;
-        const uint32_t b = __ballot_sync(FULL, low);
-        if (low) m.gid[out + __popc(b & lanemask_lt())] = x;
-        out += __popc(b);
+    for (int b0 = 0; b0 < w; b0 += 32 * kFlat) {
+        int32_t x[kFlat];
+        int j[kFlat];
+#pragma unroll
+        for (int u = 0; u < kFlat; ++u) {
+            const int k = b0 + 32 * u + lane;
+            x[u] = k < w ? P.col[r0 + k] : -1;
+        }
+        lookup(x, j);
+#pragma unroll
+        for (int u = 0; u < kFlat; ++u) {
+            const bool low = x[u] >= 0 && j[u] < 0;
+            const uint32_t b = __ballot_sync(FULL, low);
+            if (low) m.gid[out + __popc(b & lanemask_lt())] = x[u];
+            out += __popc(b);
+        }
     }
     __syncwarp();
     for (int x0 = 0; x0 < w; x0 += 32) {
         const int32_t gx = x0 + lane < w ? m.gid[x0 + lane] : -1;
         if (gx >= 0) p.gid[x0 + lane] = gx;
         flat_lists(
-            P, gx, x0, c, lane, [&](int32_t y) { return find(m.key, m.idx, shift, mask, y); },
-            [&](int j) { return m.gid[j]; },
+            P, gx, x0, c, lane, lookup, [&](int j) { return m.gid[j]; },
             [&](int x, int j) {
                 atomicOr(&m.row[x * kWarpS + (j >> 5)], 1u << (j & 31));
                 if (x < c) atomicOr(&m.row[j * kWarpS + (x >> 5)], 1u << (x & 31));
@@ -306,20 +350,31 @@ __device__ void build_by_block(const BuildParams &P, BlockSmem &m, const Parts &
         for (int s = t; s <= (int)mask; s += kThreads) m.key[s] = -1;
     __syncthreads();
     const int32_t *cl = P.up_col + u0;
-    for (int i = t; i < c; i += kThreads) {
-        const int32_t y = cl[i];
-        p.gid[i] = y;
+    for (int i0 = warp * 32; i0 < c; i0 += kThreads) {
+        const int i = i0 + lane;
+        const int32_t y = i < c ? cl[i] : -1;
+        if (i < c) p.gid[i] = y;
         if (table) insert(m.key, m.idx, shift, mask, y, i);
     }
     uint4 *rows = reinterpret_cast<uint4 *>(p.A);
     for (int64_t k = t; k < (int64_t)w * (p.S >> 2); k += kThreads) rows[k] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    auto lookup = [&](int32_t y) { return table ? find(m.key, m.idx, shift, mask, y) : search(cl, c, y); };
+    auto lookup = [&](const int32_t (&y)[kFlat], int (&j)[kFlat]) {
+        if (table) {
+            find(m.key, m.idx, shift, mask, y, j);
+        } else {
+#pragma unroll
+            for (int u = 0; u < kFlat; ++u) j[u] = search(cl, y[u] >= 0 ? c : 0, y[u]);
+        }
+    };
     // lower-ranked neighbours, in order
     int out = c;
     for (int b0 = 0; b0 < w; b0 += kThreads) {
-        const int32_t x = b0 + t < w ? P.col[r0 + b0 + t] : 0;
-        const bool low = b0 + t < w && lookup(x) < 0;
+        const int32_t x = b0 + t < w ? P.col[r0 + b0 + t] : -1;
+        int32_t y[kFlat] = {x, -1, -1, -1};
+        int j[kFlat];
+        lookup(y, j);
+        const bool low = x >= 0 && j[0] < 0;
         const uint32_t b = __ballot_sync(FULL, low);
         if (lane == 0) red[warp] = __popc(b);
         __syncthreads();

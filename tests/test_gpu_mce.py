@@ -336,6 +336,20 @@ def test_handover_stress_keeps_every_subproblem(gpu_lib, shape):
     assert mce.decode_list(off, vtx, r2.list_cliques) == O.ttt_whole(og, want_list=True).cliques
 
 
+def test_builds_are_the_same_every_time(gpu_lib):
+    """Long chains in the hash tables of the candidates come and go with the
+    order of the inserts; no run may lose a row over one."""
+    import torch
+    mce = gpu_lib
+    n, u, v = rmat(12, seed=9)
+    perm = np.random.default_rng(4).permutation(n).astype(np.int32)
+    g, rank = gpu_graph(mce, n, u, v), _t(perm)
+    first, pv = (torch.empty((3, n), dtype=torch.int64, device="cuda") for _ in range(2))
+    for i in range(60):
+        mce.enumerate_cliques(g, rank="user", user_rank=rank, per_vertex=tuple(pv if i else first))
+        assert i == 0 or torch.equal(pv, first), i
+
+
 def test_user_rank_random_permutation(gpu_lib):
     mce = gpu_lib
     n, u, v = rmat(12, seed=9)
