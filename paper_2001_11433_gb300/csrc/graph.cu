@@ -132,20 +132,19 @@ __global__ void k_degree_key(const int32_t *row_ptr, int32_t n, int64_t *key) {
 // the latency of a round (one hub's visit and the barrier), of which graphs
 // whose hubs fall one step after the other take hundreds.  Peeling level by
 // level (three barriers per removal step, each removed hub's row walked by one
-// warp) took 42.1 ms on the 1.7M-vertex graph and 9.3 ms on R-MAT 18; this
-// kernel: 39 ms and 3.4 ms.
+// warp) took 42.1 ms on the 1.7M-vertex graph (750 rounds here) and 9.3 ms on
+// R-MAT 18; this kernel: 25 ms and 3.4 ms.
 //
 // stamp[v] = round in which v is to be visited.  Lists by degree: [0] 2..32
-// (8 lanes a vertex), [1] 33..1024 (a warp), [2] above (256 threads, with the
+// (8 lanes a vertex), [1] 33..1024 (a warp), [2] above (128 threads, with the
 // neighbours that can still matter kept apart once the hub has fallen); degrees
 // 0 and 1 are their own core numbers.  more[k][r % 3] = round r visits list k.
-constexpr int kCoreThreads = 1024;
+constexpr int kCoreThreads = 512;   // 128 registers: a warp holds a row of 1024 entries
 constexpr int kCoreWarps = kCoreThreads / 32;
 constexpr int kCoreSmall = 32, kCoreMid = 1024;
-constexpr int kHubThreads = 256, kHubWarps = kHubThreads / 32, kHubGroups = kCoreThreads / kHubThreads;
-constexpr int kHubBins = 4096;                       // a group's share of the warps' bins holds more
-constexpr size_t kCoreSmem = (size_t)kCoreWarps * kCoreMid * sizeof(int32_t);
-static_assert(kHubBins <= kHubWarps * kCoreMid, "hub bins");
+constexpr int kHubThreads = 128, kHubWarps = kHubThreads / 32, kHubGroups = kCoreThreads / kHubThreads;
+constexpr int kHubBins = 4096;
+constexpr size_t kCoreSmem = (size_t)kHubGroups * kHubBins * sizeof(int32_t);
 
 struct CoreParams {
     const int32_t *row_ptr, *col;
@@ -192,12 +191,13 @@ __global__ void k_core_init(CoreParams P) {
 // val[v] fell from `was` to `now`: neighbour w (value x) is visited in the
 // next round if v counted towards x and no longer does.  A neighbour that is
 // visited in this round may end anywhere up to x, so its bound is `now` alone.
-// Returns the bit of w's list, or 0.
+// Returns the bit of w's list (of both it can be in, if x tells only that), or 0.
 __device__ __forceinline__ uint32_t core_tell(const CoreParams &P, int32_t w, int32_t x, int32_t was, int32_t now,
                                               int32_t round) {
     if (x <= now) return 0u;
     if (x > was && __ldcg(P.stamp + w) != round) return 0u;
     P.stamp[w] = round + 1;
+    if (x > kCoreSmall) return 6u;   // its degree is at least x
     return 1u << core_class(P.row_ptr[w + 1] - P.row_ptr[w]);
 }
 
@@ -254,7 +254,7 @@ __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, in
         for (int32_t k = t; k < hi - lo; k += kHubThreads) bin[k] = 0;
         hub_sync(bar);
         int32_t cnt = 0;
-#pragma unroll 4
+#pragma unroll 8
         for (int32_t e = t; e < len; e += kHubThreads) {
             const int32_t x = __ldcg(P.val + (few ? __ldcg(row + e) : row[e]));
             if (x >= hi) ++cnt;
@@ -278,7 +278,7 @@ __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, in
     if (t == 0) P.val[v] = h;
     uint32_t told = 0u;
     if (from && h >= from) {   // neighbours above h are all among the kept ones
-#pragma unroll 4
+#pragma unroll 8
         for (int32_t e = t; e < n_kept; e += kHubThreads) {
             const int32_t w = __ldcg(kept + e);
             told |= core_tell(P, w, __ldcg(P.val + w), c, h, round);
@@ -316,16 +316,51 @@ __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, in
     return told;
 }
 
+// The visit of a vertex v with up to 32 EACH neighbours by a warp: its row is
+// read once, all of a lane's entries in flight, and held while the value is
+// searched and the neighbours are told.  (Dependent passes over the row with
+// bins in shared memory made this visit 14 to 30 us long, and in each round
+// all other warps waited for one: the rounds of the 1.7M-vertex graph took 34 ms
+// and now take 25.)  Returns the list bits told.
+template <int EACH>
+__device__ __forceinline__ uint32_t core_mid(const CoreParams &P, int32_t v, int32_t e0, int32_t d, int32_t c,
+                                             int32_t round, int lane) {
+    int32_t w[EACH], x[EACH];
+#pragma unroll
+    for (int q = 0; q < EACH; ++q) w[q] = q * 32 + lane < d ? P.col[e0 + q * 32 + lane] : -1;
+#pragma unroll
+    for (int q = 0; q < EACH; ++q) x[q] = w[q] >= 0 ? __ldcg(P.val + w[q]) : 0;
+    auto at_least = [&](int32_t h) {
+        int32_t k = 0;
+#pragma unroll
+        for (int q = 0; q < EACH; ++q) k += x[q] >= h;
+        return __reduce_add_sync(0xffffffffu, k);
+    };
+    const int32_t cnt = at_least(c);
+    if (cnt >= c) return 0u;
+    // cnt neighbours have val >= c > cnt, so the value is at least cnt
+    int32_t lo = cnt > 1 ? cnt : 1, hi = c - 1;
+    while (lo < hi) {   // the same for all lanes
+        const int32_t mid = (lo + hi + 1) >> 1;
+        if (at_least(mid) >= mid) lo = mid; else hi = mid - 1;
+    }
+    if (lane == 0) P.val[v] = lo;
+    uint32_t told = 0u;
+#pragma unroll
+    for (int q = 0; q < EACH; ++q)
+        if (w[q] >= 0) told |= core_tell(P, w[q], x[q], c, lo, round);
+    return told;
+}
+
 __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
     cg::grid_group grid = cg::this_grid();
-    extern __shared__ int32_t core_bins[];   // kCoreMid bins a warp; a group's together for its hub
+    extern __shared__ int32_t core_bins[];   // kHubBins a group
     __shared__ HubShared hub[kHubGroups];
     __shared__ uint32_t block_told;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nblk = gridDim.x;
     const int64_t gwarp = (int64_t)blockIdx.x * kCoreWarps + warp, nwarp = nblk * kCoreWarps;
     const int32_t n_small = P.ctl[0], n_mid = P.ctl[1], n_big = P.ctl[2];
-    int32_t *bin = core_bins + warp * kCoreMid;
     if (threadIdx.x == 0) block_told = 0u;
     uint32_t visit = 7u;   // lists with visits in this round
     for (int32_t round = 0;; ++round) {
@@ -344,12 +379,11 @@ __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
                 hub_sync(1 + g);
                 const int na = m.n_active;
                 for (int a = 0; a < na; ++a) {
-                    told |= core_hub(P, m, core_bins + g * kHubWarps * kCoreMid, m.active[a], round, 1 + g);
+                    told |= core_hub(P, m, core_bins + g * kHubBins, m.active[a], round, 1 + g);
                     hub_sync(1 + g);
                 }
             }
         }
-        __syncthreads();   // the bins are the warps' again
         // ---- degrees 33..1024: a warp each, items dealt out warp by warp
         if (visit & 2u)
             for (int64_t i0 = gwarp; i0 < n_mid; i0 += nwarp * 32) {
@@ -358,45 +392,10 @@ __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
                 uint32_t m = __ballot_sync(0xffffffffu, mine >= 0 && __ldcg(P.stamp + (mine < 0 ? 0 : mine)) == round);
                 for (; m; m &= m - 1u) {
                     const int32_t v = __shfl_sync(0xffffffffu, mine, __ffs(m) - 1);
-                    const int32_t e0 = P.row_ptr[v], e1 = P.row_ptr[v + 1];
-                    const int32_t c = __ldcg(P.val + v);
-                    int32_t cnt = 0;
-                    for (int32_t b0 = e0; b0 < e1 && cnt < c; b0 += 128) {
-                        int32_t k = 0;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int32_t e = b0 + q * 32 + lane;
-                            if (e < e1) k += __ldcg(P.val + P.col[e]) >= c;
-                        }
-                        cnt += __reduce_add_sync(0xffffffffu, k);
-                    }
-                    if (cnt >= c) continue;
-                    int32_t h = 0;   // windows of bins, as for the hubs
-                    for (int32_t hi = c;;) {
-                        const int32_t lo = hi >> 1 > 1 ? hi >> 1 : 1;
-                        for (int32_t k = lane; k < hi - lo; k += 32) bin[k] = 0;
-                        __syncwarp();
-                        int32_t top = 0;
-#pragma unroll 4
-                        for (int32_t e = e0 + lane; e < e1; e += 32) {
-                            const int32_t x = __ldcg(P.val + P.col[e]);
-                            if (x >= hi) ++top;
-                            else if (x >= lo) atomicAdd(&bin[x - lo], 1);
-                        }
-                        top = __reduce_add_sync(0xffffffffu, top);
-                        __syncwarp();
-                        h = core_from_bins(bin, lo, hi, top, lane);
-                        __syncwarp();
-                        if (h || lo == 1) break;
-                        hi = lo;
-                    }
-                    if (h < 1) h = 1;
-                    if (lane == 0) P.val[v] = h;
-#pragma unroll 4
-                    for (int32_t e = e0 + lane; e < e1; e += 32) {
-                        const int32_t w = P.col[e];
-                        told |= core_tell(P, w, __ldcg(P.val + w), c, h, round);
-                    }
+                    const int32_t e0 = P.row_ptr[v], d = P.row_ptr[v + 1] - e0, c = __ldcg(P.val + v);
+                    if (d <= 128) told |= core_mid<4>(P, v, e0, d, c, round, lane);
+                    else if (d <= 384) told |= core_mid<12>(P, v, e0, d, c, round, lane);
+                    else told |= core_mid<32>(P, v, e0, d, c, round, lane);
                 }
             }
         // ---- degrees 2..32: 8 lanes each, four vertices of a warp at a time

@@ -125,7 +125,13 @@ def core_graph(shape):
             vs += [j + base, [base - 1 if base else 1]]
             base += k
         return base, np.concatenate(us), np.concatenate(vs)
-    hubs = {"deg32": 32, "deg33": 33, "deg1024": 1024, "deg1025": 1025}[shape]
+    if shape == "core":                       # degrees 35..1999: values that fall for many rounds
+        n = 2000
+        i, j = np.triu_indices(n, 1)
+        w = 10.0 * (np.arange(n) + 1.0) ** -0.6
+        hit = rng.random(len(i)) < np.minimum(w[i] * w[j], 1.0)
+        return n, i[hit], j[hit]
+    hubs = int(shape[3:])
     n = 3 * hubs + 50                         # three hubs of that degree over a sparse rest, two of them joined
     leaves = np.arange(3, n)
     u = np.concatenate([np.full(hubs, 0), np.full(hubs, 1), np.full(hubs, 2), rng.choice(leaves, 2 * n), [0]])
@@ -134,7 +140,8 @@ def core_graph(shape):
     return n, u, v
 
 
-@pytest.mark.parametrize("shape", ["path", "tree", "cliques", "deg32", "deg33", "deg1024", "deg1025"])
+@pytest.mark.parametrize("shape", ["path", "tree", "cliques", "deg32", "deg33", "deg128", "deg129", "deg384", "deg385", "deg1024",
+                                   "deg1025", "core"])
 def test_core_numbers_by_degree_class(gpu_lib, shape):
     """Lanes, warps and blocks a vertex (degrees up to 32, up to 1024, above)."""
     mce = gpu_lib
