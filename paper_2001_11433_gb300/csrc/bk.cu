@@ -705,6 +705,12 @@ __device__ __forceinline__ int node_weight(int cn, int fn) { return 1 + ((cn + f
 // GB300: 50 us; the 1.7M-vertex graph under the degeneracy rank searched
 // in 36 ms instead of 51 ms (one subproblem alone kept its warp busy for 42 ms).
 constexpr uint64_t BK_SPLIT_NS = 50000;
+// Longest pause between two looks of a waiting warp at the ring and the
+// counters.  Each look is a handful of loads and an atomic of words that the
+// busy warps need for their hand-overs: with 2,000 warps looking every 16 us
+// the 1.7M-vertex graph took 50.8 ms under the degeneracy rank (builds and
+// search) and 29.3 under the degree rank, now 39.6 and 28.6 (R-MAT 18 equal).
+constexpr unsigned BK_WAIT_NS = 128000;
 
 // Budget, abort and splitting checks, made every 64 nodes with the current
 // frame written back to memory.  Returns 0 = go on, 1 = stop the launch,
@@ -2308,7 +2314,7 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
     int node_tick = 0;
     bool hungry = false;
     uint64_t idle_since = 0;
-    unsigned backoff = 500;   // ns between tries while waiting (doubles to 16 us)
+    unsigned backoff = 500;   // ns between tries while waiting (doubles to BK_WAIT_NS)
     const uint64_t t_start = globaltimer_ns();
     for (;;) {
         // ---- acquire work: queued pieces first, then the next subproblem
@@ -2380,7 +2386,7 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
                 break;
             }
             __nanosleep(backoff);
-            if (backoff < 16000u) backoff <<= 1;
+            if (backoff < BK_WAIT_NS) backoff <<= 1;
             continue;
         }
         backoff = 500;
