@@ -167,7 +167,7 @@ mce_status plan_issue(mce_batched *b, cudaStream_t s) {
     MCE_CUDA(cudaMemsetAsync(b->gnodes.p, 0, (size_t)k * 8, s));
     MCE_CUDA(cudaMemsetAsync(b->any.p, 0, 4, s));
     if (P.n_sub > 0) {
-        MCE_TRY(launch_build_rows(P, true, s));
+        MCE_TRY(launch_build_rows(P, s));
         MCE_TRY(launch_bk(P, b->ls.warps_per_block, b->ls.blocks_per_sm, s));
     } else {
         MCE_CUDA(cudaMemsetAsync(P.ctl, 0, CTL_WORDS * 8, s));
@@ -241,8 +241,8 @@ mce_status mce_batched_create(const mce_graph *g, const int32_t *graph_ptr, int3
     MCE_CUDA(cudaMemsetAsync(b->ghash0.p, 0, (size_t)k * 8, s));
     MCE_TRY(flag.alloc(((size_t)n + 1) * 4, s));
     MCE_TRY(keys.alloc(((size_t)n + 1) * 8, s));
-    MCE_TRY(reqb.alloc(32, s));
-    MCE_CUDA(cudaMemsetAsync(reqb.p, 0, 32, s));
+    MCE_TRY(reqb.alloc(PREPASS_WORDS * 8, s));
+    MCE_CUDA(cudaMemsetAsync(reqb.p, 0, PREPASS_WORDS * 8, s));
     MCE_TRY(launch_prepass(g, b->up_ptr.as<int32_t>(), opts->hash_seed, nullptr, b->out0.as<unsigned long long>(),
                            flag.as<int32_t>(), keys.as<uint64_t>(), reqb.as<unsigned long long>(),
                            b->graph_of.as<int32_t>(), b->gcount0.as<unsigned long long>(),

@@ -185,12 +185,11 @@ __host__ __device__ inline int64_t bk_ws_words(int64_t w, int64_t c, int32_t mod
 // Builds of every scheduled subproblem into the cache (which P has), before
 // launch_bk on the same stream; build_prepare once outside any capture.
 // launch_build_layout fills cache_off and build_big from the order (build_ctl
-// zero before it); launch_build_rows builds (BUILD_NEXT zero before it).  With
-// `reset`, the latter also sets the task ring and the control block to their
-// start values.
+// zero before it); launch_build_rows builds (BUILD_NEXT zero before it), and
+// sets the task ring and the control block to their start values.
 mce_status build_prepare();
 mce_status launch_build_layout(const BkParams &p, cudaStream_t s);
-mce_status launch_build_rows(const BkParams &p, bool reset, cudaStream_t s);
+mce_status launch_build_rows(const BkParams &p, cudaStream_t s);
 mce_status bk_prepare(int32_t blocks_per_sm, int64_t smem_bytes);
 mce_status launch_bk(const BkParams &p, int32_t warps_per_block, int32_t blocks_per_sm, cudaStream_t s);
 mce_status init_queue_seq(unsigned long long *seq, int64_t n, cudaStream_t s);

@@ -68,7 +68,7 @@ struct BuildParams {
     const int32_t *big;                 // vertices for block builds, heavy ones first
     const unsigned long long *n_big;
     unsigned long long *next;           // next entry of big
-    // a plan's run: ring and control block to their start values (null: not here)
+    // ring and control words of the search, set to their start values here
     unsigned long long *qseq, *ctl;
     int64_t qcap;
 };
@@ -449,11 +449,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_build_rows(BuildParams P) {
     __shared__ int32_t red[kWarps];
     __shared__ int32_t claim;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (P.qseq) {
-        const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-        for (int64_t i = tid; i < P.qcap; i += (int64_t)gridDim.x * kThreads) P.qseq[i] = (unsigned long long)i;
-        if (tid < CTL_WORDS) P.ctl[tid] = tid == CTL_PENDING ? (unsigned long long)P.n_sub : 0ULL;
-    }
+    const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    for (int64_t i = tid; i < P.qcap; i += (int64_t)gridDim.x * kThreads) P.qseq[i] = (unsigned long long)i;
+    if (tid < CTL_WORDS) P.ctl[tid] = tid == CTL_PENDING ? (unsigned long long)P.n_sub : 0ULL;
     const int32_t n_big = (int32_t)*P.n_big;
     for (;;) {
         if (threadIdx.x == 0) claim = (int32_t)atomicAdd(P.next, 1ULL);
@@ -540,7 +538,7 @@ mce_status launch_build_layout(const BkParams &P, cudaStream_t s) {
     return MCE_OK;
 }
 
-mce_status launch_build_rows(const BkParams &P, bool reset, cudaStream_t s) {
+mce_status launch_build_rows(const BkParams &P, cudaStream_t s) {
     MCE_TRY(build_prepare());
     BuildParams B{};
     B.row_ptr = P.row_ptr;
@@ -554,11 +552,9 @@ mce_status launch_build_rows(const BkParams &P, bool reset, cudaStream_t s) {
     B.big = P.build_big;
     B.n_big = P.build_ctl + BUILD_BIG;
     B.next = P.build_ctl + BUILD_NEXT;
-    if (reset) {
-        B.qseq = P.qseq;
-        B.qcap = P.qcap;
-        B.ctl = P.ctl;
-    }
+    B.qseq = P.qseq;
+    B.qcap = P.qcap;
+    B.ctl = P.ctl;
     const int64_t blocks = ((int64_t)P.n_sub + kWarps - 1) / kWarps, most = (int64_t)num_sms() * 2;
     MCE_LAUNCH(k_build_rows, (unsigned)(blocks < most ? blocks : most), kThreads, sizeof(BuildSmem), s, B);
     return MCE_OK;

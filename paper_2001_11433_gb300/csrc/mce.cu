@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
                               unsigned long long *req_max, const int32_t *graph_of, unsigned long long *g_count,
                               unsigned long long *g_hash, int64_t *list_off, int32_t *list_vtx,
                               int64_t list_max_cliques, int64_t list_max_words, const uint8_t *in_subset) {
-    unsigned long long cnt = 0, hsh = 0, nodes = 0, req = 0, cmax = 0, shw = 0, prv = 0;
+    unsigned long long cnt = 0, hsh = 0, nodes = 0, req = 0, cmax = 0, shw = 0, prv = 0, act = 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         if (in_subset && !in_subset[v]) {
             flag[v] = 0;
@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
             if (pv_count) pv_nodes[v] = 1;
         } else {
             f = 1;
+            ++act;
             uint64_t k;
             if (cost) {
                 // descending predicted cost: invert the order-preserving float map
@@ -99,8 +100,9 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
         cmax = max(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
         shw += __shfl_xor_sync(0xffffffffu, shw, o);
         prv = max(prv, __shfl_xor_sync(0xffffffffu, prv, o));
+        act += __shfl_xor_sync(0xffffffffu, act, o);
     }
-    __shared__ unsigned long long part[7][kPrepassThreads / 32];
+    __shared__ unsigned long long part[8][kPrepassThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) {
         part[0][warp] = cnt;
@@ -110,6 +112,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
         part[4][warp] = cmax;
         part[5][warp] = shw;
         part[6][warp] = prv;
+        part[7][warp] = act;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -121,6 +124,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
             cmax = max(cmax, part[4][k]);
             shw += part[5][k];
             prv = max(prv, part[6][k]);
+            act += part[7][k];
         }
         if (cnt) {
             atomicAdd(&out[OUT_COUNT], cnt);
@@ -133,6 +137,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
         if (cmax) atomicMax(req_max + 1, cmax);
         if (shw) atomicAdd(req_max + 2, shw);
         if (prv) atomicMax(req_max + 3, prv);
+        if (act) atomicAdd(req_max + 4, act);
     }
 }
 
@@ -304,14 +309,11 @@ mce_status run_bk(BkParams &P, const LaunchShape &ls, int64_t req_max, int64_t c
     MCE_TRY(b.arena.alloc((size_t)P.qcap * P.slot_words * 4, s));
     MCE_TRY(b.qseq.alloc((size_t)P.qcap * 8, s));
     MCE_TRY(b.taskbuf.alloc((size_t)nwarps * P.slot_words * 4, s));
-    MCE_TRY(init_queue_seq(b.qseq.as<unsigned long long>(), P.qcap, s));
     MCE_TRY(b.ctl.alloc(CTL_WORDS * sizeof(unsigned long long), s));
-    MCE_CUDA(cudaMemsetAsync(b.ctl.p, 0, CTL_WORDS * sizeof(unsigned long long), s));
     P.arena = b.arena.as<uint32_t>();
     P.qseq = b.qseq.as<unsigned long long>();
     P.taskbuf = b.taskbuf.as<uint32_t>();
     P.ctl = b.ctl.as<unsigned long long>();
-    MCE_LAUNCH(k_set_u64, 1, 1, 0, s, P.ctl + CTL_PENDING, (unsigned long long)P.n_sub);
     if (P.timeout_ns == 0) P.timeout_ns = 60ULL * 1000000000ULL;
     if (P.max_run_ns == 0) P.max_run_ns = 600ULL * 1000000000ULL;
     if (P.cache) {
@@ -321,7 +323,11 @@ mce_status run_bk(BkParams &P, const LaunchShape &ls, int64_t req_max, int64_t c
         P.build_big = b.big.as<int32_t>();
         P.build_ctl = b.build_ctl.as<unsigned long long>();
         MCE_TRY(launch_build_layout(P, s));
-        MCE_TRY(launch_build_rows(P, false, s));
+        MCE_TRY(launch_build_rows(P, s));   // and the ring and control words to their start
+    } else {
+        MCE_TRY(init_queue_seq(P.qseq, P.qcap, s));
+        MCE_CUDA(cudaMemsetAsync(P.ctl, 0, CTL_WORDS * sizeof(unsigned long long), s));
+        MCE_LAUNCH(k_set_u64, 1, 1, 0, s, P.ctl + CTL_PENDING, (unsigned long long)P.n_sub);
     }
     return launch_bk(P, ls.warps_per_block, ls.blocks_per_sm, s);
 }
@@ -462,13 +468,12 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
             MCE_LAUNCH(k_heavy_flags, grid_for(n, 256), 256, 0, s, cost.as<float>(), n, thr, heavy.as<uint8_t>());
         }
     }
-    MCE_TRY(out.alloc(OUT_WORDS * 8, s));
-    MCE_CUDA(cudaMemsetAsync(out.p, 0, OUT_WORDS * 8, s));
+    MCE_TRY(out.alloc((OUT_WORDS + PREPASS_WORDS) * 8, s));   // the run's totals, then the prepass'
+    MCE_CUDA(cudaMemsetAsync(out.p, 0, (OUT_WORDS + PREPASS_WORDS) * 8, s));
+    unsigned long long *req = out.as<unsigned long long>() + OUT_WORDS;
     MCE_TRY(flag.alloc((size_t)(n + 1) * 4, s));
     MCE_TRY(keys.alloc((size_t)(n + 1) * 8, s));
-    DevBuf reqb, mask;
-    MCE_TRY(reqb.alloc(32, s));
-    MCE_CUDA(cudaMemsetAsync(reqb.p, 0, 32, s));
+    DevBuf mask;
     const uint8_t *maskp = nullptr;
     DevBuf hsub;
     const int32_t *subp = o->subset;
@@ -506,17 +511,20 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
         MCE_LAUNCH(k_mce_prepass, prepass_grid(n), kPrepassThreads, 0, s, g->row_ptr, up_ptr.as<int32_t>(), n, idb, o->hash_seed,
                    costp, out.as<unsigned long long>(), (unsigned long long *)o->pv_count,
                    (unsigned long long *)o->pv_hash, (unsigned long long *)o->pv_nodes, flag.as<int32_t>(),
-                   keys.as<uint64_t>(), reqb.as<unsigned long long>(), graph_of, g_count, g_hash, o->list_off,
+                   keys.as<uint64_t>(), req, graph_of, g_count, g_hash, o->list_off,
                    o->list_vtx, o->list_max_cliques, o->list_max_words, maskp);
     MCE_TRY(exclusive_scan_i32(flag.as<int32_t>(), flag.as<int32_t>(), n, s));
-    int32_t n_act = 0;
-    unsigned long long reqc[4] = {0, 0, 0, 0};
-    MCE_CUDA(cudaMemcpyAsync(&n_act, flag.as<int32_t>() + n, 4, cudaMemcpyDeviceToHost, s));
-    MCE_CUDA(cudaMemcpyAsync(reqc, reqb.p, 32, cudaMemcpyDeviceToHost, s));
+    unsigned long long reqc[PREPASS_WORDS];
+    MCE_CUDA(cudaMemcpyAsync(reqc, req, sizeof(reqc), cudaMemcpyDeviceToHost, s));
     MCE_CUDA(cudaStreamSynchronize(s));
+    const int32_t n_act = (int32_t)reqc[4];
     res->subproblems = n_act;
     BkBuffers bb;
-    DevBuf subn;
+    DevBuf subn, cache, coff;
+    cudaEvent_t k0, k1;
+    MCE_CUDA(cudaEventCreate(&k0));
+    MCE_CUDA(cudaEventCreate(&k1));
+    EvPair kg{k0, k1};
     if (n_act > 0) {
         MCE_TRY(tmp.alloc((size_t)n_act * 8 * 2, s));
         MCE_TRY(order.alloc((size_t)n_act * 4, s));
@@ -568,7 +576,6 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
         P.max_run_ns = (uint64_t)o->time_limit_ms * 1000000ULL;
         // build cache for every subproblem (up to 2^30 words); when it holds them
         // all, a warp's own workspace only needs the private search state
-        DevBuf cache, coff;
         const int64_t cw = (int64_t)reqc[2] < ((int64_t)1 << 30) ? (int64_t)reqc[2] : ((int64_t)1 << 30);
         int64_t per_warp = (int64_t)reqc[0];
         if (cw == (int64_t)reqc[2]) per_warp = (int64_t)reqc[3];
@@ -583,17 +590,9 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
             P.cache_off = coff.as<long long>();
         }
         const LaunchShape ls = launch_shape(o);
-        cudaEvent_t k0, k1;
-        MCE_CUDA(cudaEventCreate(&k0));
-        MCE_CUDA(cudaEventCreate(&k1));
-        EvPair kg{k0, k1};
         MCE_CUDA(cudaEventRecord(k0, s));
         MCE_TRY(run_bk(P, ls, per_warp, (int64_t)reqc[1], s, bb));
         MCE_CUDA(cudaEventRecord(k1, s));
-        MCE_CUDA(cudaEventSynchronize(k1));
-        float ks = 0;
-        cudaEventElapsedTime(&ks, k0, k1);
-        res->ms_search = ks;
     }
     MCE_CUDA(cudaEventRecord(e2, s));
     if (subn.p) {
@@ -609,6 +608,7 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
     }
     mce_status st = read_result(out, bb.ctl, s, res);
     if (o->whole_graph && n > 0) res->tree_nodes += 1;   // the root node of the whole-graph tree
+    if (n_act > 0) cudaEventElapsedTime(&res->ms_search, k0, k1);
     float a = 0, b = 0;
     cudaEventElapsedTime(&a, e0, e1);
     cudaEventElapsedTime(&b, e1, e2);

@@ -19,6 +19,9 @@ struct BkBuffers {
 };
 // task lists of the lane-parallel small search (static MCE only)
 mce_status alloc_lp_tasks(BkParams &P, int64_t nwarps, cudaStream_t s, BkBuffers &b);
+// totals of the prepass: largest workspace, largest candidate count, build cache
+// words, largest private workspace, scheduled vertices
+constexpr int PREPASS_WORDS = 5;
 mce_status run_bk(BkParams &P, const LaunchShape &ls, int64_t req_max, int64_t cmax, cudaStream_t s, BkBuffers &b);
 mce_status compute_rank(const mce_graph *g, const mce_opts *o, cudaStream_t s, int32_t *rank);
 mce_status read_result(const DevBuf &out, const DevBuf &ctl, cudaStream_t s, mce_result *res);
