@@ -133,16 +133,18 @@ __global__ void k_degree_key(const int32_t *row_ptr, int32_t n, int64_t *key) {
 // whose hubs fall one step after the other take hundreds.  Peeling level by
 // level (three barriers per removal step, each removed hub's row walked by one
 // warp) took 42.1 ms on the 1.7M-vertex graph (750 rounds here) and 9.3 ms on
-// R-MAT 18; this kernel: 25 ms and 3.4 ms.
+// R-MAT 18; this kernel: 21 ms and 3.4 ms.
 //
 // stamp[v] = round in which v is to be visited.  Lists by degree: [0] 2..32
-// (8 lanes a vertex), [1] 33..1024 (a warp), [2] above (128 threads, with the
+// (8 lanes a vertex), [1] 33..1024 (a warp), [2] above (64 threads, with the
 // neighbours that can still matter kept apart once the hub has fallen); degrees
 // 0 and 1 are their own core numbers.  more[k][r % 3] = round r visits list k.
 constexpr int kCoreThreads = 512;   // 128 registers: a warp holds a row of 1024 entries
 constexpr int kCoreWarps = kCoreThreads / 32;
 constexpr int kCoreSmall = 32, kCoreMid = 1024;
-constexpr int kHubThreads = 128, kHubWarps = kHubThreads / 32, kHubGroups = kCoreThreads / kHubThreads;
+// (64: on the 1.7M-vertex graph nearly all of the 1,100 hubs are visited in every
+// round, one a group; with 128 threads two in turn, 25 ms for the 21.)
+constexpr int kHubThreads = 64, kHubWarps = kHubThreads / 32, kHubGroups = kCoreThreads / kHubThreads;
 constexpr int kHubBins = 4096;
 constexpr size_t kCoreSmem = (size_t)kHubGroups * kHubBins * sizeof(int32_t);
 
@@ -254,7 +256,7 @@ __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, in
         for (int32_t k = t; k < hi - lo; k += kHubThreads) bin[k] = 0;
         hub_sync(bar);
         int32_t cnt = 0;
-#pragma unroll 8
+#pragma unroll 16
         for (int32_t e = t; e < len; e += kHubThreads) {
             const int32_t x = __ldcg(P.val + (few ? __ldcg(row + e) : row[e]));
             if (x >= hi) ++cnt;
@@ -278,7 +280,7 @@ __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, in
     if (t == 0) P.val[v] = h;
     uint32_t told = 0u;
     if (from && h >= from) {   // neighbours above h are all among the kept ones
-#pragma unroll 8
+#pragma unroll 16
         for (int32_t e = t; e < n_kept; e += kHubThreads) {
             const int32_t w = __ldcg(kept + e);
             told |= core_tell(P, w, __ldcg(P.val + w), c, h, round);
