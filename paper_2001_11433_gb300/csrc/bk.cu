@@ -768,9 +768,14 @@ __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int3
             if (acc.t_nodes - cold().t_split < (heavy && every < 2048ULL ? every : 2048ULL) &&
                 (!P.cache || now - cold().t_split_ns < BK_SPLIT_NS))
                 hungry = 0;
-            // a long-running task spreads its subtree before anybody waits
+            // a long-running task spreads its subtree before anybody waits, while
+            // less than a piece a warp lies in the ring: pieces are taken before
+            // the next subproblems, and up to half a ring of them kept heavy
+            // subproblems waiting (R-MAT 18 192 ms; with this bound 182, Chung-Lu
+            // 1.7M equal)
+            const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
             if (!hungry && every && acc.t_nodes - cold().t_split >= every &&
-                qlen < (unsigned long long)P.qcap / 2) hungry = 1;
+                qlen < (warps < (unsigned long long)P.qcap / 2 ? warps : (unsigned long long)P.qcap / 2)) hungry = 1;
         }
     }
     // endgame: every subproblem has been taken and warps wait for pieces; the
