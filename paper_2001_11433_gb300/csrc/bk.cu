@@ -709,8 +709,10 @@ constexpr uint64_t BK_SPLIT_NS = 50000;
 // counters.  Each look is a handful of loads and an atomic of words that the
 // busy warps need for their hand-overs: with 2,000 warps looking every 16 us
 // the 1.7M-vertex graph took 50.8 ms under the degeneracy rank (builds and
-// search) and 29.3 under the degree rank, now 39.6 and 28.6 (R-MAT 18 equal).
-constexpr unsigned BK_WAIT_NS = 128000;
+// search) and 29.3 under the degree rank, with 128 us 39.6 and 28.6 (R-MAT 18
+// equal).  A warp pauses for a sixteenth of the time it has waited: 128 us
+// right away made searches of a millisecond up to 4 % slower.
+constexpr uint64_t BK_WAIT_NS = 128000;
 
 // Budget, abort and splitting checks, made every 64 nodes with the current
 // frame written back to memory.  Returns 0 = go on, 1 = stop the launch,
@@ -2319,7 +2321,6 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
     int node_tick = 0;
     bool hungry = false;
     uint64_t idle_since = 0;
-    unsigned backoff = 500;   // ns between tries while waiting (doubles to BK_WAIT_NS)
     const uint64_t t_start = globaltimer_ns();
     for (;;) {
         // ---- acquire work: queued pieces first, then the next subproblem
@@ -2390,11 +2391,10 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
                 if (lane == 0) atomicAdd(&P.ctl[CTL_HUNGRY], ~0ULL);
                 break;
             }
-            __nanosleep(backoff);
-            if (backoff < BK_WAIT_NS) backoff <<= 1;
+            const uint64_t pause = (now - idle_since) >> 4;
+            __nanosleep(pause < 500 ? 500u : (unsigned)(pause < BK_WAIT_NS ? pause : BK_WAIT_NS));
             continue;
         }
-        backoff = 500;
         if (hungry) {
             hungry = false;
             if (lane == 0) {
