@@ -1526,10 +1526,9 @@ __device__ __forceinline__ void lp_two(const BkParams &P, uint32_t *shist, LpSum
 // dealt out to the lanes one each: child q of a node follows from the node's
 // sets and the ext members before q alone.  Children with at most two
 // candidates are settled at once, the others pushed.  (Each lane going through
-// the children of its own node left half of the lanes idle: R-MAT 18 searched
-// at 23.6 warp instructions a node; see with the children dealt out
-// the lane search takes 88 of the 168 ms a warp searches on R-MAT 18, whose
-// search fell from 218 to 196 ms.)
+// the children of its own node left half of the lanes idle; with the children
+// dealt out the search of R-MAT 18 fell from 218 to 196 ms, 88 of the 168 ms
+// that a warp was then busy in here.)
 //
 // Room: up to 512 nodes on the stack 32 are taken, and each pushes fewer than
 // 32; up to 1024, 8; above, one at a time, whose whole subtree then holds at

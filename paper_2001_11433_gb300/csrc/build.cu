@@ -18,7 +18,7 @@
 // up in a hash table of C in shared memory.  One lane per list with binary
 // searches, inside the search kernel at 16 warps an SM and one warp a hub,
 // kept every warp busy for 23.6 ms on the 1.7M-vertex graph, and one hub's
-// warp for 73 ms under the degeneracy rank; this kernel: 11.1 ms, hubs included.
+// warp for 73 ms under the degeneracy rank; this kernel: 10.6 ms, hubs included.
 #include "bk.cuh"
 
 namespace mce {

@@ -564,8 +564,9 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
         }
         P.split = o->split;
         // measured on GB300 with the lane search: 4,096 keeps every rank of the
-        // Chung-Lu graph balanced (12,288 costs the learned rank 18 %), while
-        // the R-MAT 18 benchmark set is fastest at 12,288, which it asks for
+        // Chung-Lu graph balanced (28.6 ms under the degree rank, 30.3 at
+        // 16,384), while R-MAT 18 is fastest with longer runs (182 ms, 165 at
+        // 16,384; its benchmark asks for 12,288)
         P.split_nodes = o->split ? (o->split_nodes ? o->split_nodes : 4096u) : 0u;
         P.sm_limit = o->sm_limit;
         P.lp_hold_waiting = o->lane_hold_waiting;
