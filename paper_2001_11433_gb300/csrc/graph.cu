@@ -5,8 +5,8 @@
 //                   normalised as in Section 6.1): drop self loops, symmetrise,
 //                   radix sort, deduplicate, row offsets by scan.
 //   vertex_key      Section 4.2 keys: degree, core number ("degeneracy" of a
-//                   vertex: in the k-core but not the (k+1)-core) by parallel
-//                   peeling, triangle count by oriented intersection.
+//                   vertex: in the k-core but not the (k+1)-core) by rounds of
+//                   the h-index step, triangle count by oriented intersection.
 //   rank_from_key   rank(v) = position of (key(v), id(v)) in ascending order.
 //   build_up_lists  Γ+(v) = neighbours of higher rank (the cand set of v's
 //                   subproblem in Algorithm 5), sorted by id.
@@ -133,18 +133,19 @@ __global__ void k_degree_key(const int32_t *row_ptr, int32_t n, int64_t *key) {
 // whose hubs fall one step after the other take hundreds.  Peeling level by
 // level (three barriers per removal step, each removed hub's row walked by one
 // warp) took 42.1 ms on the 1.7M-vertex graph (750 rounds here) and 9.3 ms on
-// R-MAT 18; this kernel: 21 ms and 3.4 ms.
+// R-MAT 18; this kernel: 13.6 ms and 3.8 ms.
 //
 // stamp[v] = round in which v is to be visited.  Lists by degree: [0] 2..32
-// (8 lanes a vertex), [1] 33..1024 (a warp), [2] above (64 threads, with the
+// (8 lanes a vertex), [1] 33..384 (a warp), [2] above (256 threads, with the
 // neighbours that can still matter kept apart once the hub has fallen); degrees
 // 0 and 1 are their own core numbers.  more[k][r % 3] = round r visits list k.
-constexpr int kCoreThreads = 512;   // 128 registers: a warp holds a row of 1024 entries
+constexpr int kCoreThreads = 512;   // 128 registers: 16 loads of a thread in flight
 constexpr int kCoreWarps = kCoreThreads / 32;
-constexpr int kCoreSmall = 32, kCoreMid = 1024;
-// (64: on the 1.7M-vertex graph nearly all of the 1,100 hubs are visited in every
-// round, one a group; with 128 threads two in turn, 25 ms for the 21.)
-constexpr int kHubThreads = 64, kHubWarps = kHubThreads / 32, kHubGroups = kCoreThreads / kHubThreads;
+constexpr int kCoreSmall = 32, kCoreMid = 384;
+// Measured on GB300 (R-MAT 14, R-MAT 18, Chung-Lu 1.7M; ms): a warp up to 384
+// neighbours and 256 threads above 1.0, 3.8, 13.6; 64 threads 1.3, 3.7, 14.6; a
+// warp up to 1024 and 256 threads above 0.65, 4.8, 20.5; 64 threads 0.75, 6.5, 26.4
+constexpr int kHubThreads = 256, kHubWarps = kHubThreads / 32, kHubGroups = kCoreThreads / kHubThreads;
 constexpr int kHubBins = 4096;
 constexpr size_t kCoreSmem = (size_t)kHubGroups * kHubBins * sizeof(int32_t);
 
@@ -194,13 +195,30 @@ __global__ void k_core_init(CoreParams P) {
 // next round if v counted towards x and no longer does.  A neighbour that is
 // visited in this round may end anywhere up to x, so its bound is `now` alone.
 // Returns the bit of w's list (of both it can be in, if x tells only that), or 0.
-__device__ __forceinline__ uint32_t core_tell(const CoreParams &P, int32_t w, int32_t x, int32_t was, int32_t now,
-                                              int32_t round) {
-    if (x <= now) return 0u;
-    if (x > was && __ldcg(P.stamp + w) != round) return 0u;
-    P.stamp[w] = round + 1;
-    if (x > kCoreSmall) return 6u;   // its degree is at least x
-    return 1u << core_class(P.row_ptr[w + 1] - P.row_ptr[w]);
+// N neighbours at a time (w = -1: none), their loads in flight together: told
+// one after the other, the notes of a lane took most of a visit.
+template <int N>
+__device__ __forceinline__ uint32_t core_tell(const CoreParams &P, const int32_t *w, const int32_t *x, int32_t was,
+                                                  int32_t now, int32_t round) {
+    bool tell[N];
+    int32_t d[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        int32_t st = round;
+        if (w[q] >= 0 && x[q] > was) st = __ldcg(P.stamp + w[q]);
+        tell[q] = w[q] >= 0 && x[q] > now && st == round;
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        d[q] = 0;
+        if (tell[q]) P.stamp[w[q]] = round + 1;
+        if (tell[q] && x[q] <= kCoreSmall) d[q] = P.row_ptr[w[q] + 1] - P.row_ptr[w[q]];
+    }
+    uint32_t told = 0u;
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+        if (tell[q]) told |= x[q] > kCoreSmall ? 6u : 1u << core_class(d[q]);
+    return told;
 }
 
 // largest h in [lo, hi) with cnt + (entries of bin[h - lo ..]) >= h, or 0, one warp
@@ -280,10 +298,13 @@ __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, in
     if (t == 0) P.val[v] = h;
     uint32_t told = 0u;
     if (from && h >= from) {   // neighbours above h are all among the kept ones
-#pragma unroll 16
-        for (int32_t e = t; e < n_kept; e += kHubThreads) {
-            const int32_t w = __ldcg(kept + e);
-            told |= core_tell(P, w, __ldcg(P.val + w), c, h, round);
+        for (int32_t b0 = t; b0 < n_kept; b0 += 8 * kHubThreads) {
+            int32_t w[8], x[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) w[q] = b0 + q * kHubThreads < n_kept ? __ldcg(kept + b0 + q * kHubThreads) : -1;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = w[q] >= 0 ? __ldcg(P.val + w[q]) : 0;
+            told |= core_tell<8>(P, w, x, c, h, round);
         }
         return told;
     }
@@ -295,19 +316,24 @@ __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, in
     }
     hub_sync(bar);
     int32_t *out = P.kept + m.at;
-    for (int32_t b0 = warp * 32; b0 < d; b0 += kHubThreads) {
-        const int32_t e = b0 + lane;
-        int32_t w = 0, x = 0;
-        if (e < d) {
-            w = P.col[e0 + e];
-            x = __ldcg(P.val + w);
-            told |= core_tell(P, w, x, c, h, round);
+    for (int32_t b0 = warp * 32; b0 < d; b0 += 4 * kHubThreads) {
+        int32_t w[4], x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int32_t e = b0 + q * kHubThreads + lane;
+            w[q] = e < d ? P.col[e0 + e] : -1;
         }
-        const uint32_t b = __ballot_sync(0xffffffffu, x >= keep);
-        int32_t at = 0;
-        if (lane == 0 && b) at = atomicAdd(&m.kept, __popc(b));
-        at = __shfl_sync(0xffffffffu, at, 0);
-        if (x >= keep) out[at + __popc(b & lanemask_lt())] = w;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = w[q] >= 0 ? __ldcg(P.val + w[q]) : 0;
+        told |= core_tell<4>(P, w, x, c, h, round);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t b = __ballot_sync(0xffffffffu, x[q] >= keep);
+            int32_t at = 0;
+            if (lane == 0 && b) at = atomicAdd(&m.kept, __popc(b));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (x[q] >= keep) out[at + __popc(b & lanemask_lt())] = w[q];
+        }
     }
     hub_sync(bar);
     if (t == 0) {
@@ -322,8 +348,7 @@ __device__ uint32_t core_hub(const CoreParams &P, HubShared &m, int32_t *bin, in
 // read once, all of a lane's entries in flight, and held while the value is
 // searched and the neighbours are told.  (Dependent passes over the row with
 // bins in shared memory made this visit 14 to 30 us long, and in each round
-// all other warps waited for one: the rounds of the 1.7M-vertex graph took 34 ms
-// and now take 25.)  Returns the list bits told.
+// all other warps waited for one.)  Returns the list bits told.
 template <int EACH>
 __device__ __forceinline__ uint32_t core_mid(const CoreParams &P, int32_t v, int32_t e0, int32_t d, int32_t c,
                                              int32_t round, int lane) {
@@ -349,8 +374,7 @@ __device__ __forceinline__ uint32_t core_mid(const CoreParams &P, int32_t v, int
     if (lane == 0) P.val[v] = lo;
     uint32_t told = 0u;
 #pragma unroll
-    for (int q = 0; q < EACH; ++q)
-        if (w[q] >= 0) told |= core_tell(P, w[q], x[q], c, lo, round);
+    for (int q = 0; q < EACH; q += 4) told |= core_tell<4>(P, w + q, x + q, c, lo, round);
     return told;
 }
 
@@ -386,7 +410,10 @@ __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
                 }
             }
         }
-        // ---- degrees 33..1024: a warp each, items dealt out warp by warp
+        // the others see this round's values of the hubs: without this barrier
+        // R-MAT 18 takes three times as many rounds
+        __syncthreads();
+        // ---- degrees 33..384: a warp each, items dealt out warp by warp
         if (visit & 2u)
             for (int64_t i0 = gwarp; i0 < n_mid; i0 += nwarp * 32) {
                 const int64_t i = i0 + (int64_t)lane * nwarp;
@@ -396,8 +423,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
                     const int32_t v = __shfl_sync(0xffffffffu, mine, __ffs(m) - 1);
                     const int32_t e0 = P.row_ptr[v], d = P.row_ptr[v + 1] - e0, c = __ldcg(P.val + v);
                     if (d <= 128) told |= core_mid<4>(P, v, e0, d, c, round, lane);
-                    else if (d <= 384) told |= core_mid<12>(P, v, e0, d, c, round, lane);
-                    else told |= core_mid<32>(P, v, e0, d, c, round, lane);
+                    else told |= core_mid<12>(P, v, e0, d, c, round, lane);
                 }
             }
         // ---- degrees 2..32: 8 lanes each, four vertices of a warp at a time
@@ -443,9 +469,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
                     if (v >= 0 && cnt < c) {
                         const int32_t h = lo > 1 ? lo : 1;
                         if ((lane & 7) == 0) P.val[v] = h;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            if (w[q] >= 0) told |= core_tell(P, w[q], x[q], c, h, round);
+                        told |= core_tell<4>(P, w, x, c, h, round);
                     }
                 }
             }

@@ -143,7 +143,7 @@ def core_graph(shape):
 @pytest.mark.parametrize("shape", ["path", "tree", "cliques", "deg32", "deg33", "deg128", "deg129", "deg384", "deg385", "deg1024",
                                    "deg1025", "core"])
 def test_core_numbers_by_degree_class(gpu_lib, shape):
-    """Lanes, warps and blocks a vertex (degrees up to 32, up to 1024, above)."""
+    """Lanes, warps and blocks a vertex (degrees up to 32, up to 384, above)."""
     mce = gpu_lib
     n, u, v = core_graph(shape)
     og = O.Graph(n, np.asarray(u, np.int32), np.asarray(v, np.int32))
