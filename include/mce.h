@@ -79,7 +79,9 @@ typedef struct {
     int32_t rank_kind;            /* MCE_RANK_* */
     const int32_t *user_rank;     /* device int32[n], a permutation of [0, n) (MCE_RANK_USER) */
     const mce_model *model;       /* MCE_RANK_LEARNED */
-    uint64_t node_budget;         /* stop after this many search-tree nodes; 0 = unlimited */
+    uint64_t node_budget;         /* stop after this many nodes of the searched trees (MCE_EBUDGET); 0 =
+                                     unlimited.  Counts are exact: the call completes iff the trees
+                                     have no more */
     uint64_t hash_seed;           /* seed of h(v) */
     void *stream;                 /* cudaStream_t */
     /* Optional clique list (device, caller-owned).  Clique i starts at

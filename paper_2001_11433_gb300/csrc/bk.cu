@@ -714,12 +714,20 @@ constexpr uint64_t BK_SPLIT_NS = 50000;
 // right away made searches of a millisecond up to 4 % slower.
 constexpr uint64_t BK_WAIT_NS = 128000;
 
-// Budget, abort and splitting checks, made every 64 nodes with the current
-// frame written back to memory.  Returns 0 = go on, 1 = stop the launch,
-// 2 = drop this task (its graph or subproblem is over budget).
+// `nodes` more tree nodes against the launch's budget; the launch stops once
+// they pass it.  One lane.  Returns false then.
+__device__ __forceinline__ bool charge_nodes(const BkParams &P, unsigned long long nodes) {
+    if (atomicAdd(&P.ctl[CTL_NODES], nodes) + nodes <= P.node_budget) return true;
+    atomicOr(&P.ctl[CTL_ABORT], 1ULL);
+    return false;
+}
+
+// Budget, abort and splitting checks, made every acc.tick units of node_weight
+// with the current frame written back to memory.
 // Lane 0 reads the control words and credits node counts; the result is
-// broadcast: returns 1 = stop the launch, 2 = drop this task, 0 = go on with
-// `hungry` = the number of hand-overs wanted (0 = none).
+// broadcast: returns 1 = stop the launch, 2 = drop this task (its graph or
+// subproblem is over budget), 0 = go on with `hungry` = the number of
+// hand-overs wanted (0 = none).
 __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int32_t root, uint64_t t_start,
                     unsigned long long &hungry_out) {
     hist_guard(P, acc, shist, lane);
@@ -729,18 +737,12 @@ __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int3
         const uint64_t now = globaltimer_ns();
         if (now - t_start > P.max_run_ns) atomicOr(&P.ctl[CTL_ABORT], 2ULL);
         ab = *(volatile unsigned long long *)&P.ctl[CTL_ABORT];
-        if (P.node_budget) {
-            const unsigned long long tot = atomicAdd(&P.ctl[CTL_NODES], 64ULL) + 64ULL;
-            if (tot > P.node_budget) {
-                atomicOr(&P.ctl[CTL_ABORT], 1ULL);
-                ab |= 1ULL;
-            }
-        }
-        // exact node counts per subproblem and per graph: the task's nodes
+        // exact node counts per launch, subproblem and graph: the task's nodes
         // since the last report (the rest is credited when the task ends), so
         // "over budget" holds exactly when the whole tree exceeds the budget
         const unsigned long long delta = acc.t_nodes - cold().t_rep;
         cold().t_rep = acc.t_nodes;
+        if (P.node_budget && !charge_nodes(P, delta)) ab |= 1ULL;
         if (P.sub_nodes) {
             const unsigned long long tot = atomicAdd(&P.sub_nodes[root], delta) + delta;
             if (tot > P.sub_budget) ab |= 16ULL;
@@ -873,8 +875,9 @@ __device__ void donate_mem(const BkParams &P, Ws &s, const Task &T, int lane, in
     __syncwarp();
 }
 
-// Checks made every 64 nodes with the current frame written back to memory.
-// Returns 0 = go on, 1 = stop the launch, 2 = drop this task.
+// The checks of poll, with the current frame written back to memory, and the
+// hand-overs they ask for.  Returns 0 = go on, 1 = stop the launch, 2 = drop
+// this task.
 __device__ int periodic(const BkParams &P, Ws &s, const Task &T, Acc &acc, uint32_t *shist, int lane, int d,
                         int32_t root, uint64_t t_start) {
     unsigned long long hungry = 0;
@@ -2417,6 +2420,7 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
             c.count += acc.t_count;
             c.hash += acc.t_hash;
             c.nodes += acc.t_nodes;
+            if (P.node_budget && acc.t_nodes > c.t_rep) charge_nodes(P, acc.t_nodes - c.t_rep);
             if (P.sub_nodes && acc.t_nodes > c.t_rep) atomicAdd(&P.sub_nodes[T.root], acc.t_nodes - c.t_rep);
             if (P.graph_nodes && acc.t_nodes > c.t_rep)
                 atomicAdd(&P.graph_nodes[P.graph_of[P.mode == BK_MCE ? T.root : P.eu[T.root]]], acc.t_nodes - c.t_rep);

@@ -389,6 +389,30 @@ def test_node_budget(gpu_lib):
     assert r.status == mce.MCE_EBUDGET and not r.complete
 
 
+@pytest.mark.parametrize("leaves", [0, 700])
+@pytest.mark.parametrize("small", [False, True])
+def test_node_budget_counts_nodes(gpu_lib, leaves, small):
+    """Wide nodes (up to 500 candidates; with the leaves a root of 1,200 in memory
+    frames) and small ones count as one node each: trees of at most the budget's
+    nodes complete, larger ones do not."""
+    mce = gpu_lib
+    i, j = np.triu_indices(500, 1)
+    keep = (i >= 16) | (i % 2 == 1) | (j != i + 1)         # K_500 without eight disjoint edges
+    n = 501 + leaves
+    u = np.concatenate([i[keep] + 1, np.zeros(n - 1)])     # and vertex 0, ranked lowest, joined to all
+    v = np.concatenate([j[keep] + 1, np.arange(1, n)])
+    g = gpu_graph(mce, n, u, v)
+    kw = dict(rank="user", user_rank=_t(np.arange(n)), warp_small_search=small)
+    ref = mce.enumerate_cliques(g, **kw)
+    assert ref.count == 256 + leaves
+    nodes = ref.tree_nodes - leaves                        # the leaves' own subproblems need no search
+    r = mce.enumerate_cliques(g, node_budget=nodes, **kw)
+    assert (r.status, r.complete) == (mce.MCE_OK, 1)
+    assert (r.count, r.hash, r.tree_nodes) == (ref.count, ref.hash, ref.tree_nodes)
+    r = mce.enumerate_cliques(g, node_budget=nodes // 2, allow=(mce.MCE_EBUDGET,), **kw)
+    assert r.status == mce.MCE_EBUDGET and not r.complete
+
+
 def test_list_overflow_keeps_summary(gpu_lib):
     mce = gpu_lib
     w = graphgen.er_2000()
