@@ -715,11 +715,9 @@ constexpr uint64_t BK_SPLIT_NS = 50000;
 constexpr uint64_t BK_WAIT_NS = 128000;
 
 // `nodes` more tree nodes against the launch's budget; the launch stops once
-// they pass it.  One lane.  Returns false then.
-__device__ __forceinline__ bool charge_nodes(const BkParams &P, unsigned long long nodes) {
-    if (atomicAdd(&P.ctl[CTL_NODES], nodes) + nodes <= P.node_budget) return true;
-    atomicOr(&P.ctl[CTL_ABORT], 1ULL);
-    return false;
+// they pass it.  One lane.
+__device__ __forceinline__ void charge_nodes(const BkParams &P, unsigned long long nodes) {
+    if (atomicAdd(&P.ctl[CTL_NODES], nodes) + nodes > P.node_budget) atomicOr(&P.ctl[CTL_ABORT], 1ULL);
 }
 
 // Budget, abort and splitting checks, made every acc.tick units of node_weight
@@ -736,13 +734,13 @@ __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int3
     if (lane == 0) {
         const uint64_t now = globaltimer_ns();
         if (now - t_start > P.max_run_ns) atomicOr(&P.ctl[CTL_ABORT], 2ULL);
-        ab = *(volatile unsigned long long *)&P.ctl[CTL_ABORT];
         // exact node counts per launch, subproblem and graph: the task's nodes
         // since the last report (the rest is credited when the task ends), so
         // "over budget" holds exactly when the whole tree exceeds the budget
         const unsigned long long delta = acc.t_nodes - cold().t_rep;
         cold().t_rep = acc.t_nodes;
-        if (P.node_budget && !charge_nodes(P, delta)) ab |= 1ULL;
+        if (P.node_budget) charge_nodes(P, delta);
+        ab = *(volatile unsigned long long *)&P.ctl[CTL_ABORT];
         if (P.sub_nodes) {
             const unsigned long long tot = atomicAdd(&P.sub_nodes[root], delta) + delta;
             if (tot > P.sub_budget) ab |= 16ULL;
