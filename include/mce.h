@@ -137,9 +137,9 @@ typedef struct {
      * too and equals Algorithm 1's count on the whole graph.  rank_kind,
      * user_rank and subset are ignored. */
     int32_t whole_graph;
-    /* Streaming multiprocessors that take search work (0 = all), for scaling
-     * measurements: the whole grid is launched and only blocks on SMs with an
-     * id below sm_limit search.  The result does not depend on it. */
+    /* Streaming multiprocessors that build subproblems and search them (0 =
+     * all), for scaling measurements: the whole grid is launched and only blocks
+     * on SMs with an id below sm_limit work.  The result does not depend on it. */
     int32_t sm_limit;
     /* Per-warp shared-memory words of the lane-parallel small search (0 =
      * automatic: what the block's shared memory leaves, at most 2048; values

@@ -23,10 +23,12 @@ __global__ void k_check_disjoint(const int32_t *row_ptr, const int32_t *col, con
             if (graph_of[col[e]] != graph_of[x]) atomicOr(bad, 1);
 }
 
-// next_build (may be null): back to 0 for the plan's next run
+// build_ctl (may be null): the words that a run of the plan counts in, back to 0
+// for its next run
 __global__ void k_graph_status(const unsigned long long *nodes, int32_t k, uint64_t budget, int32_t *status,
-                               int32_t *any, unsigned long long *next_build) {
-    if (next_build && blockIdx.x == 0 && threadIdx.x == 0) *next_build = 0ULL;
+                               int32_t *any, unsigned long long *build_ctl) {
+    if (build_ctl && blockIdx.x == 0 && threadIdx.x >= BUILD_NEXT && threadIdx.x < BUILD_WORDS)
+        build_ctl[threadIdx.x] = 0ULL;
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < k; g += (int64_t)gridDim.x * blockDim.x) {
         const bool over = budget && nodes[g] > budget;
         status[g] = over ? MCE_EBUDGET : MCE_OK;
@@ -173,7 +175,7 @@ mce_status plan_issue(mce_batched *b, cudaStream_t s) {
         MCE_CUDA(cudaMemsetAsync(P.ctl, 0, CTL_WORDS * 8, s));
     }
     MCE_LAUNCH(k_graph_status, grid_for(k, 256), 256, 0, s, b->gnodes.as<unsigned long long>(), k, P.graph_budget,
-               b->status.as<int32_t>(), b->any.as<int32_t>(), P.build_ctl ? P.build_ctl + BUILD_NEXT : nullptr);
+               b->status.as<int32_t>(), b->any.as<int32_t>(), P.build_ctl);
     return MCE_OK;
 }
 

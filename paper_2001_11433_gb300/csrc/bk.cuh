@@ -27,7 +27,9 @@ enum BuildWord {
     BUILD_TOP = 0,     // words of the build cache in use
     BUILD_BIG = 1,     // subproblems built by a block
     BUILD_NEXT = 2,    // next of them
-    BUILD_WORDS = 4
+    BUILD_CLAIM = 3,   // with sm_limit: next entry of the order for the builds by a warp
+    BUILD_LEFT = 4,    // with sm_limit: blocks that have left
+    BUILD_WORDS = 5
 };
 
 // Output block (uint64 words); the size histogram follows at OUT_HIST.
@@ -111,7 +113,7 @@ struct BkParams {
     int32_t lp_words;         // per-warp shared words of the lane-parallel small search (0 = off)
     uint32_t *lp_tasks;       // per warp: a stack of lp_task_cap node records (BK_LP_TASK_WORDS each)
     int32_t lp_task_cap;
-    int32_t sm_limit;         // blocks on SMs with %smid >= sm_limit do no work (0 = all SMs work)
+    int32_t sm_limit;         // blocks on SMs with %smid >= sm_limit neither build nor search (0 = all SMs work)
     const uint8_t *heavy;     // per vertex: 1 = predicted heavy, splits every heavy_split_nodes (or null)
     uint32_t heavy_split_nodes;
     uint32_t lp_hold_waiting; // waiting warps from which small subtrees stay with the whole warp (0 = never)
@@ -185,8 +187,9 @@ __host__ __device__ inline int64_t bk_ws_words(int64_t w, int64_t c, int32_t mod
 // Builds of every scheduled subproblem into the cache (which P has), before
 // launch_bk on the same stream; build_prepare once outside any capture.
 // launch_build_layout fills cache_off and build_big from the order (build_ctl
-// zero before it); launch_build_rows builds (BUILD_NEXT zero before it), and
-// sets the task ring and the control block to their start values.
+// zero before it); launch_build_rows builds (BUILD_NEXT and the words behind it
+// zero before it), and sets the task ring and the control block to their start
+// values.
 mce_status build_prepare();
 mce_status launch_build_layout(const BkParams &p, cudaStream_t s);
 mce_status launch_build_rows(const BkParams &p, cudaStream_t s);

@@ -68,6 +68,8 @@ struct BuildParams {
     const int32_t *big;                 // vertices for block builds, heavy ones first
     const unsigned long long *n_big;
     unsigned long long *next;           // next entry of big
+    int32_t sm_limit;                   // as BkParams
+    unsigned long long *claim, *left;   // BUILD_CLAIM, BUILD_LEFT
     // ring and control words of the search, set to their start values here
     unsigned long long *qseq, *ctl;
     int64_t qcap;
@@ -443,7 +445,9 @@ __device__ void build_by_block(const BuildParams &P, BlockSmem &m, const Parts &
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(kThreads, 2) k_build_rows(BuildParams P) {
+// LIMITED: with sm_limit (an instance of its own: with the claims in the other
+// one a run of 1,024 graphs took 1.2 % longer)
+template <bool LIMITED> __global__ void __launch_bounds__(kThreads, 2) k_build_rows(BuildParams P) {
     extern __shared__ __align__(16) unsigned char build_smem[];
     BuildSmem &m = *reinterpret_cast<BuildSmem *>(build_smem);
     __shared__ int32_t red[kWarps];
@@ -452,6 +456,18 @@ __global__ void __launch_bounds__(kThreads, 2) k_build_rows(BuildParams P) {
     const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     for (int64_t i = tid; i < P.qcap; i += (int64_t)gridDim.x * kThreads) P.qseq[i] = (unsigned long long)i;
     if (tid < CTL_WORDS) P.ctl[tid] = tid == CTL_PENDING ? (unsigned long long)P.n_sub : 0ULL;
+    // sm_limit (scaling measurements): only the blocks placed on the first SMs
+    // build, as in the search.  A block elsewhere leaves, unless all others have
+    // left: then nobody else is there to take what remains.
+    if (LIMITED) {
+        uint32_t smid;
+        asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+        if (threadIdx.x == 0) claim = (int32_t)smid < P.sm_limit || atomicAdd(P.left, 1ULL) + 1 == gridDim.x;
+        __syncthreads();
+        const bool stays = claim != 0;
+        __syncthreads();
+        if (!stays) return;
+    }
     const int32_t n_big = (int32_t)*P.n_big;
     for (;;) {
         if (threadIdx.x == 0) claim = (int32_t)atomicAdd(P.next, 1ULL);
@@ -464,14 +480,24 @@ __global__ void __launch_bounds__(kThreads, 2) k_build_rows(BuildParams P) {
                                         P.up_ptr[v + 1] - P.up_ptr[v]),
                        v, red);
     }
-    // ---- warp builds
+    // ---- warp builds, dealt out evenly; claimed one by one where blocks are missing
     const int64_t nwarp = (int64_t)gridDim.x * kWarps;
-    for (int64_t i = (int64_t)blockIdx.x + (int64_t)warp * gridDim.x; i < P.n_sub; i += nwarp) {
+    auto claimed = [&]() {
+        unsigned long long k = 0;
+        if (lane == 0) k = atomicAdd(P.claim, 1ULL);
+        return (int64_t)__shfl_sync(FULL, k, 0);
+    };
+    for (int64_t i = LIMITED ? claimed() : (int64_t)blockIdx.x + (int64_t)warp * gridDim.x; i < P.n_sub;
+         i = LIMITED ? claimed() : i + nwarp) {
         const int32_t v = P.order[i];
         const int32_t w = P.row_ptr[v + 1] - P.row_ptr[v];
         const long long off = P.cache_off[v];
         if (w >= kWarpW || off < 0) continue;
         build_by_warp(P, m.w[warp], parts_of(P.cache + off, w, P.up_ptr[v + 1] - P.up_ptr[v]), v, lane);
+    }
+    if (LIMITED) {
+        __syncthreads();
+        if (threadIdx.x == 0) atomicAdd(P.left, 1ULL);
     }
 }
 
@@ -527,7 +553,8 @@ mce_status build_prepare() {
     // above the 48 KB default: opted into once, outside any stream capture
     static std::atomic<bool> done{false};
     if (done.load()) return MCE_OK;
-    MCE_CUDA(cudaFuncSetAttribute(k_build_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BuildSmem)));
+    for (auto k : {k_build_rows<false>, k_build_rows<true>})
+        MCE_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BuildSmem)));
     done.store(true);
     return MCE_OK;
 }
@@ -552,11 +579,17 @@ mce_status launch_build_rows(const BkParams &P, cudaStream_t s) {
     B.big = P.build_big;
     B.n_big = P.build_ctl + BUILD_BIG;
     B.next = P.build_ctl + BUILD_NEXT;
+    B.sm_limit = P.sm_limit;
+    B.claim = P.build_ctl + BUILD_CLAIM;
+    B.left = P.build_ctl + BUILD_LEFT;
     B.qseq = P.qseq;
     B.qcap = P.qcap;
     B.ctl = P.ctl;
     const int64_t blocks = ((int64_t)P.n_sub + kWarps - 1) / kWarps, most = (int64_t)num_sms() * 2;
-    MCE_LAUNCH(k_build_rows, (unsigned)(blocks < most ? blocks : most), kThreads, sizeof(BuildSmem), s, B);
+    if (P.sm_limit > 0)   // a full grid, so that the first SMs get their blocks
+        MCE_LAUNCH(k_build_rows<true>, (unsigned)most, kThreads, sizeof(BuildSmem), s, B);
+    else
+        MCE_LAUNCH(k_build_rows<false>, (unsigned)(blocks < most ? blocks : most), kThreads, sizeof(BuildSmem), s, B);
     return MCE_OK;
 }
 

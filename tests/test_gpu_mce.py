@@ -658,6 +658,30 @@ def test_sm_limit_keeps_results(gpu_lib, sms):
     assert b.stats[6] <= sms * 4 * 8       # warps that took part: at most those of sms SMs
 
 
+def bipartite(half, degree):
+    """Random bipartite graph: subproblems that cost their build and little search."""
+    rng = np.random.default_rng(half)
+    u = np.repeat(np.arange(half, dtype=np.int32), degree)
+    v = rng.integers(half, 2 * half, half * degree).astype(np.int32)
+    return 2 * half, u, v
+
+
+def test_sm_limit_covers_the_builds(gpu_lib):
+    """On 8 of 152 SMs a call takes nineteen times as long when all of its work is
+    restricted to them; more than half of that is asked for."""
+    import torch
+    mce = gpu_lib
+    n, u, v = bipartite(20000, 600)
+    g = gpu_graph(mce, n, u, v)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ms, res = {}, {}
+    for lim in (0, 8):
+        runs = [mce.enumerate_cliques(g, rank="degree", sm_limit=lim) for _ in range(3)]
+        ms[lim], res[lim] = min(r.ms_search for r in runs), runs[0]
+    assert (res[0].count, res[0].hash, res[0].tree_nodes) == (res[8].count, res[8].hash, res[8].tree_nodes)
+    assert ms[8] > 0.5 * sms / 8 * ms[0], ms
+
+
 def test_hold_policy_keeps_results(gpu_lib):
     """With small subtrees kept by the whole warp while any warp waits (the
     hold policy, off by default), and with hand-overs forced often, every
