@@ -106,7 +106,8 @@ typedef struct {
                                      thread; 3 and 4 trade registers for warps) */
     int32_t shared_words;         /* per-warp shared-memory workspace words (0 = none, the default:
                                      the global workspaces then get the whole L1) */
-    uint32_t time_limit_ms;       /* stop the search after this long (MCE_ETIMEOUT); 0 = 600 s */
+    uint32_t time_limit_ms;       /* stop building and searching subproblems after this long
+                                     (MCE_ETIMEOUT); 0 = 600 s */
     /* Optional restriction to the subproblems of some vertices (device
      * int32[subset_len], distinct ids); NULL = every vertex. */
     const int32_t *subset;

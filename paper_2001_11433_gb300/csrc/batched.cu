@@ -23,12 +23,8 @@ __global__ void k_check_disjoint(const int32_t *row_ptr, const int32_t *col, con
             if (graph_of[col[e]] != graph_of[x]) atomicOr(bad, 1);
 }
 
-// build_ctl (may be null): the words that a run of the plan counts in, back to 0
-// for its next run
 __global__ void k_graph_status(const unsigned long long *nodes, int32_t k, uint64_t budget, int32_t *status,
-                               int32_t *any, unsigned long long *build_ctl) {
-    if (build_ctl && blockIdx.x == 0 && threadIdx.x >= BUILD_NEXT && threadIdx.x < BUILD_WORDS)
-        build_ctl[threadIdx.x] = 0ULL;
+                               int32_t *any) {
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < k; g += (int64_t)gridDim.x * blockDim.x) {
         const bool over = budget && nodes[g] > budget;
         status[g] = over ? MCE_EBUDGET : MCE_OK;
@@ -88,7 +84,7 @@ extern "C" mce_status mce_enumerate_batched(const mce_graph *g, const int32_t *g
     if (st != MCE_OK && st != MCE_EOVERFLOW) return st;
     MCE_CUDA(cudaMemsetAsync(bad.p, 0, 4, s));
     MCE_LAUNCH(k_graph_status, grid_for(k, 256), 256, 0, s, gnodes.as<unsigned long long>(), k, opts->node_budget,
-               status, bad.as<int32_t>(), (unsigned long long *)nullptr);
+               status, bad.as<int32_t>());
     MCE_CUDA(cudaMemcpyAsync(&hbad, bad.p, 4, cudaMemcpyDeviceToHost, s));
     MCE_CUDA(cudaStreamSynchronize(s));
     if (hbad) total->complete = 0;
@@ -143,11 +139,9 @@ mce_status plan_shape(mce_batched *b, cudaStream_t s) {
     MCE_TRY(b->bb.arena.alloc((size_t)P.qcap * P.slot_words * 4, s));
     MCE_TRY(b->bb.qseq.alloc((size_t)P.qcap * 8, s));
     MCE_TRY(b->bb.taskbuf.alloc((size_t)nwarps * P.slot_words * 4, s));
-    MCE_TRY(b->bb.ctl.alloc(CTL_WORDS * 8, s));
     P.arena = b->bb.arena.as<uint32_t>();
     P.qseq = b->bb.qseq.as<unsigned long long>();
     P.taskbuf = b->bb.taskbuf.as<uint32_t>();
-    P.ctl = b->bb.ctl.as<unsigned long long>();
     if (b->exec) {
         cudaGraphExecDestroy(b->exec);
         b->exec = nullptr;
@@ -169,13 +163,14 @@ mce_status plan_issue(mce_batched *b, cudaStream_t s) {
     MCE_CUDA(cudaMemsetAsync(b->gnodes.p, 0, (size_t)k * 8, s));
     MCE_CUDA(cudaMemsetAsync(b->any.p, 0, 4, s));
     if (P.n_sub > 0) {
+        MCE_CUDA(cudaMemsetAsync(P.ctl + CTL_ABORT, 0, (CTL_WORDS - CTL_ABORT + BUILD_RUN_WORDS) * 8, s));
         MCE_TRY(launch_build_rows(P, s));
         MCE_TRY(launch_bk(P, b->ls.warps_per_block, b->ls.blocks_per_sm, s));
     } else {
         MCE_CUDA(cudaMemsetAsync(P.ctl, 0, CTL_WORDS * 8, s));
     }
     MCE_LAUNCH(k_graph_status, grid_for(k, 256), 256, 0, s, b->gnodes.as<unsigned long long>(), k, P.graph_budget,
-               b->status.as<int32_t>(), b->any.as<int32_t>(), P.build_ctl);
+               b->status.as<int32_t>(), b->any.as<int32_t>());
     return MCE_OK;
 }
 
@@ -288,6 +283,8 @@ mce_status mce_batched_create(const mce_graph *g, const int32_t *graph_ptr, int3
     P.split_nodes = opts->split ? (opts->split_nodes ? opts->split_nodes : 4096u) : 0u;
     P.max_run_ns = (uint64_t)(opts->time_limit_ms ? opts->time_limit_ms : 600000u) * 1000000ULL;
     P.timeout_ns = 60ULL * 1000000000ULL;
+    MCE_TRY(b->bb.ctl.alloc((CTL_WORDS + BUILD_WORDS) * 8, s));
+    P.ctl = b->bb.ctl.as<unsigned long long>();
     if (cw > 0) {
         MCE_TRY(b->cache.alloc((size_t)cw * 4 + 512, s));
         MCE_TRY(b->coff.alloc((size_t)n * 8, s));
@@ -295,10 +292,9 @@ mce_status mce_batched_create(const mce_graph *g, const int32_t *graph_ptr, int3
         P.cache_words = cw;
         P.cache_off = b->coff.as<long long>();
         MCE_TRY(b->bb.big.alloc((size_t)n_act * 4, s));
-        MCE_TRY(b->bb.build_ctl.alloc(BUILD_WORDS * 8, s));
-        MCE_CUDA(cudaMemsetAsync(b->bb.build_ctl.p, 0, BUILD_WORDS * 8, s));
         P.build_big = b->bb.big.as<int32_t>();
-        P.build_ctl = b->bb.build_ctl.as<unsigned long long>();
+        P.build_ctl = P.ctl + CTL_WORDS;
+        MCE_CUDA(cudaMemsetAsync(P.build_ctl, 0, BUILD_WORDS * 8, s));
         MCE_TRY(build_prepare());
         MCE_TRY(launch_build_layout(P, s));
     }

@@ -2321,7 +2321,7 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
     int node_tick = 0;
     bool hungry = false;
     uint64_t idle_since = 0;
-    const uint64_t t_start = globaltimer_ns();
+    const uint64_t t_start = P.build_ctl ? P.build_ctl[BUILD_T_START] : globaltimer_ns();
     for (;;) {
         // ---- acquire work: queued pieces first, then the next subproblem
         Task T;

@@ -16,20 +16,24 @@ enum CtlWord {
     CTL_PENDING = 3 * 16,    // subproblems + queued tasks not finished
     CTL_HUNGRY = 4 * 16,     // warps waiting for work
     CTL_NODES = 5 * 16,      // tree nodes, for the budget
-    CTL_ABORT = 6 * 16,      // 1 = budget, 2 = timeout, 4 = workspace too small, 8 = bad task
-    CTL_T_LAST = 7 * 16,     // globaltimer when the last subproblem was claimed
-    CTL_T_END = 8 * 16,      // latest globaltimer at which a warp left the launch
+    CTL_T_LAST = 6 * 16,     // globaltimer when the last subproblem was claimed
+    CTL_T_END = 7 * 16,      // latest globaltimer at which a warp left the launch
+    CTL_ABORT = 8 * 16,      // 1 = budget, 2 = timeout, 4 = workspace too small, 8 = bad task
     CTL_WORDS = 9 * 16
 };
 
-// Control words of the builds (uint64).
+// Control words of the builds (uint64), behind the control block.  CTL_ABORT and
+// the first BUILD_RUN_WORDS of them are zero before every launch_build_rows, all
+// of them before launch_build_layout.
 enum BuildWord {
-    BUILD_TOP = 0,     // words of the build cache in use
-    BUILD_BIG = 1,     // subproblems built by a block
-    BUILD_NEXT = 2,    // next of them
-    BUILD_CLAIM = 3,   // with sm_limit: next entry of the order for the builds by a warp
-    BUILD_LEFT = 4,    // with sm_limit: blocks that have left
-    BUILD_WORDS = 5
+    BUILD_NEXT = 0,    // next subproblem built by a block
+    BUILD_CLAIM = 1,   // with sm_limit: next entry of the order for the builds by a warp
+    BUILD_LEFT = 2,    // with sm_limit: blocks that have left
+    BUILD_T_START = 3, // globaltimer when the builds began: the time limit covers them
+    BUILD_RUN_WORDS = 4,
+    BUILD_TOP = 4,     // words of the build cache in use
+    BUILD_BIG = 5,     // subproblems built by a block
+    BUILD_WORDS = 6
 };
 
 // Output block (uint64 words); the size histogram follows at OUT_HIST.
@@ -94,7 +98,7 @@ struct BkParams {
     int64_t cache_words;
     long long *cache_off;
     int32_t *build_big;       // n_sub entries: the subproblems built by a block
-    unsigned long long *build_ctl;   // BUILD_* words
+    unsigned long long *build_ctl;   // BUILD_* words (null without a build cache)
     unsigned long long *ctl;
     // outputs
     unsigned long long *out;
@@ -109,7 +113,7 @@ struct BkParams {
     int32_t split;
     uint32_t split_nodes;     // a task hands over a piece after this many nodes (0 = only when warps wait)
     uint64_t timeout_ns;      // bound on any single wait
-    uint64_t max_run_ns;      // bound on a warp's time in one launch
+    uint64_t max_run_ns;      // bound on the time of the builds and the search
     int32_t lp_words;         // per-warp shared words of the lane-parallel small search (0 = off)
     uint32_t *lp_tasks;       // per warp: a stack of lp_task_cap node records (BK_LP_TASK_WORDS each)
     int32_t lp_task_cap;
@@ -186,10 +190,9 @@ __host__ __device__ inline int64_t bk_ws_words(int64_t w, int64_t c, int32_t mod
 
 // Builds of every scheduled subproblem into the cache (which P has), before
 // launch_bk on the same stream; build_prepare once outside any capture.
-// launch_build_layout fills cache_off and build_big from the order (build_ctl
-// zero before it); launch_build_rows builds (BUILD_NEXT and the words behind it
-// zero before it), and sets the task ring and the control block to their start
-// values.
+// launch_build_layout fills cache_off and build_big from the order;
+// launch_build_rows builds, and sets the task ring and the control block but
+// CTL_ABORT to their start values.
 mce_status build_prepare();
 mce_status launch_build_layout(const BkParams &p, cudaStream_t s);
 mce_status launch_build_rows(const BkParams &p, cudaStream_t s);

@@ -69,7 +69,8 @@ struct BuildParams {
     const unsigned long long *n_big;
     unsigned long long *next;           // next entry of big
     int32_t sm_limit;                   // as BkParams
-    unsigned long long *claim, *left;   // BUILD_CLAIM, BUILD_LEFT
+    unsigned long long *claim, *left, *t_start;   // BUILD_CLAIM, BUILD_LEFT, BUILD_T_START
+    uint64_t max_run_ns;
     // ring and control words of the search, set to their start values here
     unsigned long long *qseq, *ctl;
     int64_t qcap;
@@ -452,10 +453,19 @@ template <bool LIMITED> __global__ void __launch_bounds__(kThreads, 2) k_build_r
     BuildSmem &m = *reinterpret_cast<BuildSmem *>(build_smem);
     __shared__ int32_t red[kWarps];
     __shared__ int32_t claim;
+    const uint64_t t0 = globaltimer_ns();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     for (int64_t i = tid; i < P.qcap; i += (int64_t)gridDim.x * kThreads) P.qseq[i] = (unsigned long long)i;
-    if (tid < CTL_WORDS) P.ctl[tid] = tid == CTL_PENDING ? (unsigned long long)P.n_sub : 0ULL;
+    if (tid < CTL_WORDS && tid != CTL_ABORT) P.ctl[tid] = tid == CTL_PENDING ? (unsigned long long)P.n_sub : 0ULL;
+    if (tid == 0) *P.t_start = t0;
+    // one thread: the time limit has passed (looked at before each build); the
+    // search then finds the abort word set and leaves before it reads a build
+    auto late = [&]() {
+        if (globaltimer_ns() - t0 <= P.max_run_ns) return false;
+        atomicOr(&P.ctl[CTL_ABORT], 2ULL);
+        return true;
+    };
     // sm_limit (scaling measurements): only the blocks placed on the first SMs
     // build, as in the search.  A block elsewhere leaves, unless all others have
     // left: then nobody else is there to take what remains.
@@ -470,7 +480,7 @@ template <bool LIMITED> __global__ void __launch_bounds__(kThreads, 2) k_build_r
     }
     const int32_t n_big = (int32_t)*P.n_big;
     for (;;) {
-        if (threadIdx.x == 0) claim = (int32_t)atomicAdd(P.next, 1ULL);
+        if (threadIdx.x == 0) claim = late() ? n_big : (int32_t)atomicAdd(P.next, 1ULL);
         __syncthreads();
         const int32_t i = claim;
         __syncthreads();
@@ -493,6 +503,7 @@ template <bool LIMITED> __global__ void __launch_bounds__(kThreads, 2) k_build_r
         const int32_t w = P.row_ptr[v + 1] - P.row_ptr[v];
         const long long off = P.cache_off[v];
         if (w >= kWarpW || off < 0) continue;
+        if (__shfl_sync(FULL, lane == 0 && late(), 0)) break;
         build_by_warp(P, m.w[warp], parts_of(P.cache + off, w, P.up_ptr[v + 1] - P.up_ptr[v]), v, lane);
     }
     if (LIMITED) {
@@ -582,6 +593,8 @@ mce_status launch_build_rows(const BkParams &P, cudaStream_t s) {
     B.sm_limit = P.sm_limit;
     B.claim = P.build_ctl + BUILD_CLAIM;
     B.left = P.build_ctl + BUILD_LEFT;
+    B.t_start = P.build_ctl + BUILD_T_START;
+    B.max_run_ns = P.max_run_ns;
     B.qseq = P.qseq;
     B.qcap = P.qcap;
     B.ctl = P.ctl;

@@ -309,7 +309,7 @@ mce_status run_bk(BkParams &P, const LaunchShape &ls, int64_t req_max, int64_t c
     MCE_TRY(b.arena.alloc((size_t)P.qcap * P.slot_words * 4, s));
     MCE_TRY(b.qseq.alloc((size_t)P.qcap * 8, s));
     MCE_TRY(b.taskbuf.alloc((size_t)nwarps * P.slot_words * 4, s));
-    MCE_TRY(b.ctl.alloc(CTL_WORDS * sizeof(unsigned long long), s));
+    MCE_TRY(b.ctl.alloc((CTL_WORDS + BUILD_WORDS) * sizeof(unsigned long long), s));
     P.arena = b.arena.as<uint32_t>();
     P.qseq = b.qseq.as<unsigned long long>();
     P.taskbuf = b.taskbuf.as<uint32_t>();
@@ -318,10 +318,9 @@ mce_status run_bk(BkParams &P, const LaunchShape &ls, int64_t req_max, int64_t c
     if (P.max_run_ns == 0) P.max_run_ns = 600ULL * 1000000000ULL;
     if (P.cache) {
         MCE_TRY(b.big.alloc((size_t)P.n_sub * 4, s));
-        MCE_TRY(b.build_ctl.alloc(BUILD_WORDS * 8, s));
-        MCE_CUDA(cudaMemsetAsync(b.build_ctl.p, 0, BUILD_WORDS * 8, s));
         P.build_big = b.big.as<int32_t>();
-        P.build_ctl = b.build_ctl.as<unsigned long long>();
+        P.build_ctl = P.ctl + CTL_WORDS;
+        MCE_CUDA(cudaMemsetAsync(P.ctl + CTL_ABORT, 0, (CTL_WORDS - CTL_ABORT + BUILD_WORDS) * 8, s));
         MCE_TRY(launch_build_layout(P, s));
         MCE_TRY(launch_build_rows(P, s));   // and the ring and control words to their start
     } else {

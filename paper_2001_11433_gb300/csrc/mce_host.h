@@ -15,7 +15,7 @@ struct LaunchShape {
 
 LaunchShape launch_shape(const mce_opts *o);
 struct BkBuffers {
-    DevBuf gws, arena, qseq, taskbuf, ctl, lp_tasks, big, build_ctl;
+    DevBuf gws, arena, qseq, taskbuf, ctl, lp_tasks, big;
 };
 // task lists of the lane-parallel small search (static MCE only)
 mce_status alloc_lp_tasks(BkParams &P, int64_t nwarps, cudaStream_t s, BkBuffers &b);

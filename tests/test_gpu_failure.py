@@ -51,6 +51,26 @@ def test_time_limit_ends_search_with_timeout(gpu_lib):
     assert (r2.count, r2.hash, r2.tree_nodes) == (ref.count, ref.hash, ref.nodes)
 
 
+@pytest.mark.parametrize("degree", [100, 600])
+def test_time_limit_covers_the_builds(gpu_lib, degree):
+    """Random bipartite graphs, whose subproblems (100 vertices: built by warps;
+    600: by blocks) cost much building and little search: a limit that the
+    search alone would keep ends the call."""
+    mce = gpu_lib
+    half = (24 << 20) // degree
+    rng = np.random.default_rng(degree)
+    u = np.repeat(np.arange(half, dtype=np.int32), degree)
+    v = rng.integers(half, 2 * half, half * degree).astype(np.int32)
+    g = mce.Graph(2 * half, _t(u), _t(v))
+    runs = [mce.enumerate_cliques(g, rank="degree") for _ in range(3)]
+    ms = min(r.ms_search for r in runs)
+    assert ms >= 8.0
+    r = mce.enumerate_cliques(g, rank="degree", time_limit_ms=int(0.7 * ms), allow=(mce.MCE_ETIMEOUT,))
+    assert r.status == mce.MCE_ETIMEOUT and not r.complete
+    r = mce.enumerate_cliques(g, rank="degree", time_limit_ms=int(4 * ms) + 100)
+    assert (r.status, r.count, r.hash, r.tree_nodes) == (mce.MCE_OK, runs[0].count, runs[0].hash, runs[0].tree_nodes)
+
+
 def _snapshot(st, nmax=1 << 16, wmax=1 << 20):
     row, col = st.graph().csr()
     return sorted(tuple(sorted(c)) for c in st.cliques(nmax, wmax)), row.copy(), col.copy()
