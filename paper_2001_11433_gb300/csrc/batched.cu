@@ -245,16 +245,15 @@ mce_status mce_batched_create(const mce_graph *g, const int32_t *graph_ptr, int3
                            b->graph_of.as<int32_t>(), b->gcount0.as<unsigned long long>(),
                            b->ghash0.as<unsigned long long>(), s));
     MCE_TRY(exclusive_scan_i32(flag.as<int32_t>(), flag.as<int32_t>(), n, s));
-    int32_t n_act = 0;
-    unsigned long long reqc[4] = {0, 0, 0, 0};
-    MCE_CUDA(cudaMemcpyAsync(&n_act, flag.as<int32_t>() + n, 4, cudaMemcpyDeviceToHost, s));
-    MCE_CUDA(cudaMemcpyAsync(reqc, reqb.p, 32, cudaMemcpyDeviceToHost, s));
+    unsigned long long reqc[PREPASS_WORDS];
+    MCE_CUDA(cudaMemcpyAsync(reqc, reqb.p, sizeof(reqc), cudaMemcpyDeviceToHost, s));
     MCE_CUDA(cudaStreamSynchronize(s));
+    const int32_t n_act = (int32_t)reqc[4];
     MCE_TRY(b->order.alloc(((size_t)n_act + 1) * 4, s));
     if (n_act > 0) {
         MCE_TRY(tmp.alloc((size_t)n_act * 16, s));
-        MCE_TRY(launch_order(flag.as<int32_t>(), keys.as<uint64_t>(), n, n_act, g->id_bits, tmp.as<uint64_t>(),
-                             b->order.as<int32_t>(), s));
+        MCE_TRY(launch_order(flag.as<int32_t>(), keys.as<uint64_t>(), n, n_act, g->id_bits, bits_for(reqc[5]),
+                             tmp.as<uint64_t>(), b->order.as<int32_t>(), s));
     }
     b->cmax = (int64_t)reqc[1];
     const int64_t cw = (int64_t)reqc[2] < ((int64_t)1 << 30) ? (int64_t)reqc[2] : ((int64_t)1 << 30);

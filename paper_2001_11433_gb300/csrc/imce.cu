@@ -167,7 +167,7 @@ __global__ void k_edge_order_keys(const int32_t *row_ptr2, const int32_t *eu, co
         const int32_t c = min(du, dv);
         r = max(r, (unsigned long long)bk_ws_words(c, c, BK_IMCE));
         cm = max(cm, (unsigned long long)c);
-        keys[i] = ((uint64_t)heavy_first_key((uint64_t)(uint32_t)c) << IB) | (uint64_t)i;
+        keys[i] = ((uint64_t)((1u << 30) - 1 - (uint32_t)c) << IB) | (uint64_t)i;
     }
     for (int o = 16; o; o >>= 1) {
         r = max(r, __shfl_xor_sync(FULL, r, o));
@@ -1390,7 +1390,8 @@ mce_status batch_cliques(imce_state *S, const mce_graph *gp, Batch &bt, DevBuf &
     MCE_CUDA(cudaMemsetAsync(reqb.p, 0, 16, s));
     MCE_LAUNCH(k_edge_order_keys, grid_for(rho, 256), 256, 0, s, gp->row_ptr, bt.eu.as<int32_t>(), bt.ev.as<int32_t>(),
                rho, IBr, okeys.as<uint64_t>(), reqb.as<unsigned long long>());
-    MCE_TRY(radix_sort_u64(okeys.as<uint64_t>(), otmp.as<uint64_t>(), rho, IBr, IBr + 16, s));
+    // degrees are below n: the key bits above id_bits are ones
+    MCE_TRY(radix_sort_u64(okeys.as<uint64_t>(), otmp.as<uint64_t>(), rho, IBr, IBr + gp->id_bits, s));
     MCE_LAUNCH(k_keys_low, grid_for(rho, 256), 256, 0, s, okeys.as<uint64_t>(), rho, IBr, order.as<int32_t>());
     unsigned long long reqc[2] = {0, 0};
     MCE_CUDA(cudaMemcpyAsync(reqc, reqb.p, 16, cudaMemcpyDeviceToHost, s));

@@ -159,14 +159,6 @@ __device__ __forceinline__ uint64_t clique_hash_from_sum(uint64_t hsum, uint32_t
     return fmix64(hsum + (uint64_t)size * kGolden);
 }
 
-// Order keys of subproblems, heaviest first, in kOrderBits bits: the sign-free
-// exponent and 8 mantissa bits of the estimate, inverted.  Estimates within
-// 0.4 % of each other keep the order of their ids; the sort takes two passes.
-constexpr int32_t kOrderBits = 16;
-__device__ __forceinline__ uint32_t heavy_first_key(uint64_t est) {
-    return 0xffffu - (__float_as_uint((float)est) >> 15);
-}
-
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));

@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
                               unsigned long long *req_max, const int32_t *graph_of, unsigned long long *g_count,
                               unsigned long long *g_hash, int64_t *list_off, int32_t *list_vtx,
                               int64_t list_max_cliques, int64_t list_max_words, const uint8_t *in_subset) {
-    unsigned long long cnt = 0, hsh = 0, nodes = 0, req = 0, cmax = 0, shw = 0, prv = 0, act = 0;
+    unsigned long long cnt = 0, hsh = 0, nodes = 0, req = 0, cmax = 0, shw = 0, prv = 0, act = 0, emax = 0;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
         if (in_subset && !in_subset[v]) {
             flag[v] = 0;
@@ -77,12 +77,15 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
                 // descending predicted cost: invert the order-preserving float map
                 uint32_t b = __float_as_uint(cost[v]);
                 b ^= (b >> 31) ? 0xffffffffu : 0x80000000u;
-                k = ((uint64_t)((~b) >> 16) << idb) | (uint64_t)v;
+                k = ((uint64_t)(~b) << idb) | (uint64_t)v;
             } else {
                 // expected cost: the search grows with c^2 at least, the build
                 // with the neighbourhood (each of the w local vertices is scanned)
-                const uint64_t est = (uint64_t)c * (uint64_t)c + 64ULL * (uint64_t)w;
-                k = ((uint64_t)heavy_first_key(est) << idb) | (uint64_t)v;
+                const uint64_t cap = (1ULL << (63 - idb)) - 1;
+                uint64_t est = (uint64_t)c * (uint64_t)c + 64ULL * (uint64_t)w;
+                est = est < cap ? est : cap;
+                k = ((cap - est) << idb) | (uint64_t)v;   // above the largest estimate's bits: ones
+                emax = max(emax, (unsigned long long)est);
             }
             keys[v] = k;
             req = max(req, (unsigned long long)bk_ws_words(w, c, BK_MCE));
@@ -101,8 +104,9 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
         shw += __shfl_xor_sync(0xffffffffu, shw, o);
         prv = max(prv, __shfl_xor_sync(0xffffffffu, prv, o));
         act += __shfl_xor_sync(0xffffffffu, act, o);
+        emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
     }
-    __shared__ unsigned long long part[8][kPrepassThreads / 32];
+    __shared__ unsigned long long part[9][kPrepassThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) {
         part[0][warp] = cnt;
@@ -113,6 +117,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
         part[5][warp] = shw;
         part[6][warp] = prv;
         part[7][warp] = act;
+        part[8][warp] = emax;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -125,6 +130,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
             shw += part[5][k];
             prv = max(prv, part[6][k]);
             act += part[7][k];
+            emax = max(emax, part[8][k]);
         }
         if (cnt) {
             atomicAdd(&out[OUT_COUNT], cnt);
@@ -138,6 +144,7 @@ __global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *
         if (shw) atomicAdd(req_max + 2, shw);
         if (prv) atomicMax(req_max + 3, prv);
         if (act) atomicAdd(req_max + 4, act);
+        if (emax) atomicMax(req_max + 5, emax);
     }
 }
 
@@ -232,10 +239,10 @@ mce_status launch_prepass(const mce_graph *g, const int32_t *up_ptr, uint64_t se
 }
 
 mce_status launch_order(const int32_t *flag_scan, const uint64_t *keys, int32_t n, int32_t n_act, int32_t idb,
-                        uint64_t *tmp2, int32_t *order, cudaStream_t s) {
+                        int32_t key_bits, uint64_t *tmp2, int32_t *order, cudaStream_t s) {
     uint64_t *act = tmp2, *act_tmp = tmp2 + n_act;
     MCE_LAUNCH(k_gather_active, grid_for(n, 256), 256, 0, s, flag_scan, keys, n, act);
-    MCE_TRY(radix_sort_u64(act, act_tmp, n_act, idb, idb + kOrderBits, s));
+    MCE_TRY(radix_sort_u64(act, act_tmp, n_act, idb, idb + key_bits, s));
     MCE_LAUNCH(k_order_from_keys, grid_for(n_act, 256), 256, 0, s, act, n_act, idb, order);
     return MCE_OK;
 }
@@ -527,10 +534,8 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
     if (n_act > 0) {
         MCE_TRY(tmp.alloc((size_t)n_act * 8 * 2, s));
         MCE_TRY(order.alloc((size_t)n_act * 4, s));
-        uint64_t *act = tmp.as<uint64_t>(), *act_tmp = act + n_act;
-        MCE_LAUNCH(k_gather_active, grid_for(n, 256), 256, 0, s, flag.as<int32_t>(), keys.as<uint64_t>(), n, act);
-        MCE_TRY(radix_sort_u64(act, act_tmp, n_act, idb, idb + kOrderBits, s));
-        MCE_LAUNCH(k_order_from_keys, grid_for(n_act, 256), 256, 0, s, act, n_act, idb, order.as<int32_t>());
+        MCE_TRY(launch_order(flag.as<int32_t>(), keys.as<uint64_t>(), n, n_act, idb, costp ? 32 : bits_for(reqc[5]),
+                             tmp.as<uint64_t>(), order.as<int32_t>(), s));
         BkParams P{};
         P.mode = BK_MCE;
         P.row_ptr = g->row_ptr;

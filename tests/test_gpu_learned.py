@@ -182,6 +182,41 @@ def test_learned_rank_and_order_keep_the_clique_set(gpu_lib):
     assert np.array_equal(mce.rank(g, rank="learned", model=m).cpu().numpy(), O.rank_from_key(pred))
 
 
+@pytest.mark.parametrize("by_model", [False, True])
+def test_schedule_keeps_close_costs_in_order(gpu_lib, by_model):
+    """Subproblems run in decreasing cost, also where the costs are within 0.2 % of
+    each other: of 48 K_199 the later half has its lowest vertex joined to more
+    lower-ranked vertices and is listed first (each clique by its lowest vertex's
+    subproblem; one warp a block, no hand-overs)."""
+    import torch
+    mce = gpu_lib
+    k, s, extra = 48, 199, 10 if by_model else 1
+    i, j = np.triu_indices(s, 1)
+    base = s * np.arange(k)
+    hubs = np.repeat(base[k // 2:], extra)
+    n = s * k + len(hubs)
+    u = np.concatenate([(base[:, None] + i).ravel(), hubs])
+    v = np.concatenate([(base[:, None] + j).ravel(), s * k + np.arange(len(hubs))])
+    rank = np.concatenate([len(hubs) + np.arange(s * k), np.arange(len(hubs))])
+    g = mce.Graph(n, _t(u), _t(v))
+    kw = {}
+    if by_model:   # 100 + log(1 + degree)
+        p = np.zeros(8 + 1 + 1 + 1 + 1 + 1, np.float32)
+        p[[0, 9, 11, 12]] = 1.0, 1.0, 1.0, 100.0
+        kw["model"] = mce.Model(1, features="light")
+        kw["model"].set(p)
+        kw["order_by_model"] = True
+    off = torch.empty(n + k, dtype=torch.int64, device="cuda")
+    vtx = torch.empty(s * k + 4 * n, dtype=torch.int32, device="cuda")
+    r = mce.enumerate_cliques(g, rank="user", user_rank=_t(rank), list_buf=(off, vtx), warps_per_block=1, split=False,
+                              sm_limit=4, **kw)
+    assert r.count == k + len(hubs)
+    off, vtx = off[:r.list_cliques].cpu().numpy(), vtx.cpu().numpy()
+    large = [o for o in off if vtx[o] == s]
+    place = {int(vtx[o + 1:o + 1 + s].min()) // s: p for p, o in enumerate(large)}
+    assert np.mean([place[c] for c in range(k // 2, k)]) < np.mean([place[c] for c in range(k // 2)])
+
+
 def test_model_driven_splits_keep_results(gpu_lib):
     """Learned heavy-subtree splitting (a model's predicted tree sizes mark
     subproblems that hand over pieces every 64 nodes) changes the schedule
