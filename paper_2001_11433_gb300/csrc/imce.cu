@@ -1397,9 +1397,11 @@ mce_status batch_cliques(imce_state *S, const mce_graph *gp, Batch &bt, DevBuf &
     MCE_CUDA(cudaMemcpyAsync(reqc, reqb.p, 16, cudaMemcpyDeviceToHost, s));
     MCE_CUDA(cudaStreamSynchronize(s));
     MCE_TRY(nout.alloc(OUT_WORDS * 8, s));
-    // room for a few cliques an edge (1.8 on the streams measured): a search
-    // whose list does not fit is run again with the room it asked for
-    int64_t mc = ((int64_t)1 << 14) + 4 * (int64_t)rho, mw = ((int64_t)1 << 18) + 32 * (int64_t)rho;
+    // room for a few cliques an edge (1.8 on the streams measured) of up to 2^20
+    // edges (168 MB): a search whose list does not fit is run again with the room
+    // it asked for
+    const int64_t edges = rho < (1 << 20) ? rho : (1 << 20);
+    int64_t mc = ((int64_t)1 << 14) + 4 * edges, mw = ((int64_t)1 << 18) + 32 * edges;
     for (int attempt = 0;; ++attempt) {
         MCE_TRY(loff.alloc((size_t)mc * 8, s));
         MCE_TRY(lvtx.alloc((size_t)mw * 4, s));

@@ -1,4 +1,5 @@
 """GPU parity of incremental MCE (Section 5) against the CPU oracle."""
+import ctypes
 import itertools
 import json
 import os
@@ -195,3 +196,39 @@ def test_more_than_512_new_edges_in_one_clique(gpu_lib):
     n = 40
     d = _imce_vs_oracle(gpu_lib, n, [], [(i, j) for i in range(n) for j in range(i + 1, n)])
     assert (d.new_count, d.sub_count) == (1, 40)
+
+
+def pool_used_high(reset=False):
+    """High-water mark of the bytes in use of the device's default memory pool."""
+    drv = ctypes.CDLL("libcuda.so.1")
+    dev, pool, val = ctypes.c_int(), ctypes.c_void_p(), ctypes.c_uint64()
+    assert drv.cuDeviceGet(ctypes.byref(dev), 0) == 0
+    assert drv.cuDeviceGetDefaultMemPool(ctypes.byref(pool), dev) == 0
+    high = 8                                               # CU_MEMPOOL_ATTR_USED_MEM_HIGH
+    if reset:
+        assert drv.cuMemPoolSetAttribute(pool, high, ctypes.byref(val)) == 0   # to the present use
+    assert drv.cuMemPoolGetAttribute(pool, high, ctypes.byref(val)) == 0
+    return val.value
+
+
+def test_large_batch_reserves_lists_by_its_cliques(gpu_lib):
+    """Six million new edges of few cliques each: the lists take what the cliques
+    need, not a fixed room for every edge."""
+    import torch
+    mce = gpu_lib
+    n, k = 400_000, 6_000_000
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    u, v = (torch.randint(0, n, (k,), generator=gen, device="cuda").int() for _ in range(2))
+    base = mce.Graph(n, u[:2].contiguous(), v[:2].contiguous())
+    st = mce.Imce(base)
+    torch.cuda.synchronize()
+    before = pool_used_high(reset=True)
+    d = st.add_edges(u[2:].contiguous(), v[2:].contiguous())
+    used = pool_used_high() - before
+    assert d.new_count > 0.9 * d.applied and d.applied > 0.99 * k
+    ref = mce.enumerate_cliques(mce.Graph(n, u, v))
+    assert d.alive == ref.count
+    # the split buffers of 16 warps an SM, and 152 B an edge (lists by the cliques
+    # included, 20 B); a room of 160 B for every edge would make it 292
+    fixed = torch.cuda.get_device_properties(0).multi_processor_count * 16 * 2 * 4096 * 32
+    assert used < fixed + 220 * k, used
