@@ -559,10 +559,11 @@ __device__ __forceinline__ void count_node_wops(Acc &acc, int lane, int cn, int 
 
 // The block's size bins are 32 bits wide: shared memory adds 32 bits in one
 // instruction, and counts the lanes of a warp that add 1 to the same bin
-// together (64 bits are a compare-and-swap loop over those lanes).  A warp that has emitted 2^18 cliques
-// since it last did so empties the bins into the 64-bit ones in memory;
-// between two checks a warp emits at most 64 * 3^11 more, so eight warps stay
-// far below 2^32.
+// together (64 bits are a compare-and-swap loop over those lanes).  A warp that
+// has emitted 2^18 cliques since it last did so empties the bins into the 64-bit
+// ones in memory; between two checks a warp emits at most the leaves of one
+// lp_run (1.72 million, see LpSums) or of a few nodes, so eight warps stay far
+// below 2^32.
 __device__ __forceinline__ void hist_guard(const BkParams &P, const Acc &acc, uint32_t *shist, int lane) {
     const unsigned long long since = cold().since_hist + (acc.t_count - cold().t_hist);
     __syncwarp();
@@ -1378,9 +1379,14 @@ __device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, u
 
 __device__ __forceinline__ int lp_universe_words(int cn, int xn) { return 4 * cn + 2 * xn; }
 
-// Sums of one lane over one lp_run.  32 bits hold them: 64 universes of at
-// most 32 candidates have fewer than 2^24 nodes, each of fewer than 2^8 word
-// operations.
+// Sums of one lane over one lp_run.  32 bits hold even the sums of all lanes.  A
+// tree over n candidates has at most 3^(n/3) leaves and 2.5 * 3^(n/3) nodes (a
+// node with k children leaves at most n - k candidates to each); a universe of n
+// candidates takes at least 4 n words of an arena of BK_LP_MAX_WORDS, so the
+// most an lp_run can hold is 14 universes of 32: 1.72 million leaves and 4.3
+// million nodes.  A node costs at most 64 word operations and 4 a child, the
+// clique of a leaf its size, below MCE_HIST_CAP: 2.1e9 in all.  (With 64 bits
+// for wops searches took 1 to 1.8 % longer.)
 struct LpSums {
     unsigned long long hash;
     uint32_t wops, count, nodes, smax;
@@ -1650,7 +1656,7 @@ __device__ void lp_flush(const BkParams &P, Ws &s, Acc &acc, uint32_t *shist, in
     __syncwarp();
     uint32_t smax = r.smax;
     unsigned long long hsh = r.hash, wops = r.wops;
-    // counts below 2^24 a lane, 2^29 a warp
+    // counts and nodes of all lanes below 2^23
     const uint32_t cnt = __reduce_add_sync(FULL, r.count), nodes = __reduce_add_sync(FULL, r.nodes);
     smax = __reduce_max_sync(FULL, smax);
     for (int o = 16; o; o >>= 1) {

@@ -151,6 +151,7 @@ constexpr int BK_PIV_WORDS = 64 + 256 + 96;
 // Lane-parallel small search: per warp a table of up to BK_LP_MAX_ROOTS
 // relabelled small nodes (4 words each) and an arena for their universes.
 constexpr int BK_LP_MAX_ROOTS = 64;
+constexpr int BK_LP_MAX_WORDS = 2048;   // table and arena; bounds the sums of one lp_run (bk.cu, LpSums)
 constexpr int BK_LP_TABLE_WORDS = BK_LP_MAX_ROOTS * 4;
 // A node of a small subtree waiting for its pivot, two 16-byte halves: (arena
 // offset | cn << 16, cand, finc, xs), (hash sum, clique size, unused).

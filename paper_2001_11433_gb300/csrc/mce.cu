@@ -273,7 +273,7 @@ LaunchShape launch_shape(const mce_opts *o) {
     // searches 5-14 % faster at 8 KB than at 12 KB).
     if (!o || !o->warp_small_search) {
         int64_t lp = (per_block - 2048) / 4 / ls.warps_per_block - BK_PIV_WORDS - ls.smem_words;
-        if (lp > 2048) lp = 2048;
+        if (lp > BK_LP_MAX_WORDS) lp = BK_LP_MAX_WORDS;
         if (o && o->lane_search_words > 0 && o->lane_search_words < lp) lp = o->lane_search_words;
         lp &= ~int64_t(3);   // 16-byte aligned regions
         ls.lp_words = lp >= 512 ? (int32_t)lp : 0;
