@@ -2312,7 +2312,8 @@ __global__ void __launch_bounds__(256, MINB) k_bk(BkParams P) {
     for (int i = threadIdx.x; i < 256; i += blockDim.x) shist[i] = 0u;
     __syncthreads();
     uint32_t *ws_smem = smem + BK_HIST_WORDS + (int64_t)nw_block * BK_PIV_WORDS + (int64_t)wib * P.smem_words;
-    uint32_t *lp_smem = smem + BK_HIST_WORDS + (int64_t)nw_block * (BK_PIV_WORDS + P.smem_words) + (int64_t)wib * P.lp_words;
+    uint32_t *lp_smem = smem + BK_HIST_WORDS + (int64_t)nw_block * (BK_PIV_WORDS + P.smem_words) +
+                        (int64_t)wib * P.lp_words;
     const int64_t gwarp = (int64_t)blockIdx.x * nw_block + wib;
     uint32_t *ws_glob = P.gws + gwarp * P.gws_words;
     uint32_t *taskbuf = P.taskbuf + gwarp * P.slot_words;

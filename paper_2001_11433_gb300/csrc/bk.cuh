@@ -92,7 +92,7 @@ struct BkParams {
     int64_t qcap;
     uint32_t *taskbuf;
     // build cache: the read-only parts of the subproblems, built before the
-    // search (launch_build); cache_off[v] = offset, -1 = no room, the warps that
+    // search (launch_build_rows); cache_off[v] = offset, -1 = no room, the warps that
     // take it build it for themselves
     uint32_t *cache;
     int64_t cache_words;

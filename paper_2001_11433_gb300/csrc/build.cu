@@ -101,10 +101,11 @@ __device__ __forceinline__ Parts parts_of(uint32_t *base, int32_t w, int32_t c) 
 __device__ __forceinline__ uint32_t slot_of(int32_t y, int shift) { return ((uint32_t)y * 0x9E3779B1u) >> shift; }
 
 // The loops below run until a vote of the whole warp ends them and have no
-// other exit: with a loop that each lane left by its own return, lanes with a
-// long chain of slots came out of it apart from their warp, and the shuffles
-// after it gave them wrong owners (a row of a subproblem in some 10^5 lost its
-// bits, in some runs).
+// other exit.  With loops that each lane left by its own return, some runs lost
+// bits of a row (one subproblem in some 10^5; R-MAT 12 under one random rank: 8 %
+// of the runs); with these, 640 of 640 runs are right.  Why is open: lanes may
+// leave a loop one by one before a shuffle that names all of them, and reading
+// shows neither an unordered access nor a vote that some lanes miss.
 
 // table of 2^(32 - shift) slots, at most half full: j[u] = index of y[u], or
 // -1 (also for y[u] = -1); the whole warp
@@ -446,8 +447,7 @@ __device__ void build_by_block(const BuildParams &P, BlockSmem &m, const Parts &
     __syncthreads();
 }
 
-// LIMITED: with sm_limit (an instance of its own: with the claims in the other
-// one a run of 1,024 graphs took 1.2 % longer)
+// LIMITED: with sm_limit (an instance of its own, calls without it make no claims)
 template <bool LIMITED> __global__ void __launch_bounds__(kThreads, 2) k_build_rows(BuildParams P) {
     extern __shared__ __align__(16) unsigned char build_smem[];
     BuildSmem &m = *reinterpret_cast<BuildSmem *>(build_smem);

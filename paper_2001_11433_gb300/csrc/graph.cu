@@ -401,7 +401,8 @@ __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
                 if (t == 0) m.n_active = 0;
                 hub_sync(1 + g);
                 const int64_t i = i0 + (int64_t)t * ngrp;
-                if (i < n_big && __ldcg(P.stamp + P.list[2][i]) == round) m.active[atomicAdd(&m.n_active, 1)] = (int32_t)i;
+                if (i < n_big && __ldcg(P.stamp + P.list[2][i]) == round)
+                    m.active[atomicAdd(&m.n_active, 1)] = (int32_t)i;
                 hub_sync(1 + g);
                 const int na = m.n_active;
                 for (int a = 0; a < na; ++a) {

@@ -1009,6 +1009,7 @@ __global__ void __launch_bounds__(256) k_dmce_created(DelParams P) {
         }
         // every split maximal in G - H, recorded once; the members of one
         // split at a time go where the edges were
+        static_assert(kEpBits <= 2 * kSubMaxEdges, "a clique's members fit where its edges were");
         for (int t = 0; t < ns; ++t) {
             const SplitMembers mm{cv, s, ep, S + (int64_t)t * MW};
             uint64_t h = 0;

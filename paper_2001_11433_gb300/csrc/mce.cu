@@ -25,7 +25,8 @@ unsigned prepass_grid(int32_t n) {
     return need < most ? need : most;
 }
 
-__global__ void __launch_bounds__(kPrepassThreads) k_mce_prepass(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ up_ptr, int32_t n,
+__global__ void __launch_bounds__(kPrepassThreads)
+k_mce_prepass(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ up_ptr, int32_t n,
                               int32_t idb, uint64_t seed, const float *cost, unsigned long long *out,
                               unsigned long long *pv_count, unsigned long long *pv_hash,
                               unsigned long long *pv_nodes, int32_t *flag, uint64_t *keys,
@@ -231,7 +232,8 @@ mce_status launch_prepass(const mce_graph *g, const int32_t *up_ptr, uint64_t se
                           const int32_t *graph_of, unsigned long long *g_count, unsigned long long *g_hash,
                           cudaStream_t s) {
     if (g->n == 0) return MCE_OK;
-    MCE_LAUNCH(k_mce_prepass, prepass_grid(g->n), kPrepassThreads, 0, s, g->row_ptr, up_ptr, g->n, g->id_bits, seed, cost, out,
+    MCE_LAUNCH(k_mce_prepass, prepass_grid(g->n), kPrepassThreads, 0, s, g->row_ptr, up_ptr, g->n, g->id_bits, seed,
+               cost, out,
                (unsigned long long *)nullptr, (unsigned long long *)nullptr, (unsigned long long *)nullptr, flag, keys,
                reqc, graph_of, g_count, g_hash, (int64_t *)nullptr, (int32_t *)nullptr, (int64_t)0, (int64_t)0,
                (const uint8_t *)nullptr);
@@ -514,8 +516,8 @@ mce_status enumerate(const mce_graph *g, const mce_opts *o, mce_result *res, con
         MCE_CUDA(cudaMemsetAsync(o->pv_nodes, 0, (size_t)n * 8, s));
     }
     if (n > 0)
-        MCE_LAUNCH(k_mce_prepass, prepass_grid(n), kPrepassThreads, 0, s, g->row_ptr, up_ptr.as<int32_t>(), n, idb, o->hash_seed,
-                   costp, out.as<unsigned long long>(), (unsigned long long *)o->pv_count,
+        MCE_LAUNCH(k_mce_prepass, prepass_grid(n), kPrepassThreads, 0, s, g->row_ptr, up_ptr.as<int32_t>(), n, idb,
+                   o->hash_seed, costp, out.as<unsigned long long>(), (unsigned long long *)o->pv_count,
                    (unsigned long long *)o->pv_hash, (unsigned long long *)o->pv_nodes, flag.as<int32_t>(),
                    keys.as<uint64_t>(), req, graph_of, g_count, g_hash, o->list_off,
                    o->list_vtx, o->list_max_cliques, o->list_max_words, maskp);
