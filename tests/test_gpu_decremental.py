@@ -263,6 +263,20 @@ def test_more_than_256_endpoints_in_one_clique_is_refused(gpu_lib):
     assert np.array_equal(np.asarray(row0), np.asarray(row1)) and np.array_equal(np.asarray(col0), np.asarray(col1))
 
 
+def test_deletions_are_the_same_every_time(gpu_lib):
+    """The lanes of a warp leave their tests of a split one by one; a batch that goes
+    out and in again gives the same cliques each time."""
+    mce = gpu_lib
+    n = 3000
+    u, v = graphgen.er(n, 0.02, 21)
+    st = mce.Imce(mce.Graph(n, _t(u), _t(v)))
+    out, back = set(), set()
+    for _ in range(40):
+        out.add(str(_key(st.remove_edges(_t(u[:4000]), _t(v[:4000])))))
+        back.add(str(_key(st.add_edges(_t(u[:4000]), _t(v[:4000])))))
+    assert len(out) == 1 and len(back) == 1
+
+
 @pytest.mark.parametrize("n,p", [(12, 0.9), (40, 0.4)])
 def test_edges_out_and_in_again(gpu_lib, n, p):
     """Cliques that come back after their deletion are dead entries of the

@@ -140,8 +140,8 @@ def core_graph(shape):
     return n, u, v
 
 
-@pytest.mark.parametrize("shape", ["path", "tree", "cliques", "deg32", "deg33", "deg128", "deg129", "deg384", "deg385", "deg1024",
-                                   "deg1025", "core"])
+@pytest.mark.parametrize("shape", ["path", "tree", "cliques", "deg32", "deg33", "deg128", "deg129", "deg384", "deg385",
+                                   "deg1024", "deg1025", "core"])
 def test_core_numbers_by_degree_class(gpu_lib, shape):
     """Lanes, warps and blocks a vertex (degrees up to 32, up to 384, above)."""
     mce = gpu_lib
@@ -149,6 +149,18 @@ def test_core_numbers_by_degree_class(gpu_lib, shape):
     og = O.Graph(n, np.asarray(u, np.int32), np.asarray(v, np.int32))
     key = mce.vertex_key(gpu_graph(mce, n, u, v), "degen").cpu().numpy()
     assert np.array_equal(key, O.core_numbers(og).astype(np.int64))
+
+
+@pytest.mark.parametrize("few,many", [(3500, 10000), (300, 120000)])
+def test_core_numbers_of_hubs_over_several_windows(gpu_lib, few, many):
+    """Complete bipartite graphs: the few start at the largest value their edges
+    allow (above 8,192) and fall over windows without a value to that of all, `few`."""
+    import torch
+    mce = gpu_lib
+    u = torch.arange(few, dtype=torch.int32, device="cuda").repeat_interleave(many)
+    v = few + torch.arange(many, dtype=torch.int32, device="cuda").repeat(few)
+    key = mce.vertex_key(mce.Graph(few + many, u, v), "degen")
+    assert (key == few).all()
 
 
 # ---------------------------------------------------------------- enumeration: small exact cases
@@ -355,6 +367,21 @@ def test_builds_are_the_same_every_time(gpu_lib):
     for i in range(60):
         mce.enumerate_cliques(g, rank="user", user_rank=rank, per_vertex=tuple(pv if i else first))
         assert i == 0 or torch.equal(pv, first), i
+
+
+def test_lane_search_is_the_same_every_time(gpu_lib):
+    """The lanes share one stack of nodes; which of them takes a node may change
+    from run to run, no subproblem's count, hash or nodes may."""
+    import torch
+    mce = gpu_lib
+    n, u, v = rmat(13, seed=8)
+    g = gpu_graph(mce, n, u, v)
+    first, pv = (torch.empty((3, n), dtype=torch.int64, device="cuda") for _ in range(2))
+    ops = None
+    for i in range(40):
+        r = mce.enumerate_cliques(g, per_vertex=tuple(pv if i else first), split_nodes=256)
+        ops = r.word_ops if ops is None else ops
+        assert r.word_ops == ops and (i == 0 or torch.equal(pv, first)), i
 
 
 def test_user_rank_random_permutation(gpu_lib):
