@@ -726,7 +726,8 @@ __device__ __forceinline__ void charge_nodes(const BkParams &P, unsigned long lo
 // Lane 0 reads the control words and credits node counts; the result is
 // broadcast: returns 1 = stop the launch, 2 = drop this task (its graph or
 // subproblem is over budget), 0 = go on with `hungry` = the number of
-// hand-overs wanted (0 = none).
+// hand-overs wanted (0 = none).  WIDE: asked by the search of wide nodes.
+template <bool WIDE>
 __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int32_t root, uint64_t t_start,
                     unsigned long long &hungry_out) {
     hist_guard(P, acc, shist, lane);
@@ -766,10 +767,13 @@ __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int3
             // a task hands over again only after 2048 more nodes of its own
             // (fewer for a heavy one) or BK_SPLIT_NS: pieces cut too small cost
             // their receivers more than they hold (without the build cache a
-            // whole build each: there only the nodes count), but the nodes of a
-            // hub's subproblem can take a tenth of a millisecond each
+            // whole build each: there only the nodes count), but the wide nodes
+            // of a hub's subproblem can take a tenth of a millisecond each.  In the
+            // small search of the whole warp, whose frames are cheap, only the
+            // nodes count: with the time as well a clique list of the 1.7M-vertex
+            // graph took 250 ms, 93 without
             if (acc.t_nodes - cold().t_split < (heavy && every < 2048ULL ? every : 2048ULL) &&
-                (!P.cache || now - cold().t_split_ns < BK_SPLIT_NS))
+                (!WIDE || !P.cache || now - cold().t_split_ns < BK_SPLIT_NS))
                 hungry = 0;
             // a long-running task spreads its subtree before anybody waits, while
             // less than a piece a warp lies in the ring: pieces are taken before
@@ -880,7 +884,7 @@ __device__ void donate_mem(const BkParams &P, Ws &s, const Task &T, int lane, in
 __device__ int periodic(const BkParams &P, Ws &s, const Task &T, Acc &acc, uint32_t *shist, int lane, int d,
                         int32_t root, uint64_t t_start) {
     unsigned long long hungry = 0;
-    const int code = poll(P, acc, shist, lane, root, t_start, hungry);
+    const int code = poll<true>(P, acc, shist, lane, root, t_start, hungry);
     if (code || !hungry) return code;
     // up to four hand-overs per check when many warps wait
     int budget = hungry > (unsigned long long)acc.give ? acc.give : (int)hungry;
@@ -1241,7 +1245,7 @@ __device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, u
                 node_tick = 0;
                 flush();
                 unsigned long long hungry = 0;
-                const int code = poll(P, acc, shist, lane, root, t_start, hungry);
+                const int code = poll<false>(P, acc, shist, lane, root, t_start, hungry);
                 if (code) return code;
                 if (hungry) {
                     int budget = hungry > (unsigned long long)acc.give ? acc.give : (int)hungry;

@@ -709,6 +709,18 @@ def test_sm_limit_covers_the_builds(gpu_lib):
     assert ms[8] > 0.5 * sms / 8 * ms[0], ms
 
 
+@pytest.mark.parametrize("rank", ["degree", "degen"])
+def test_small_search_of_the_warp_hands_over_by_nodes(gpu_lib, rank):
+    """Clique lists and warp_small_search: a task hands over, up to eight pieces at
+    a time, after 2,048 nodes of its own.  On this graph that makes 650 to 1,100
+    nodes a piece; 210 to 250 when the time since the last hand-over was enough."""
+    mce = gpu_lib
+    n, u, v = rmat(13, seed=8)
+    g = gpu_graph(mce, n, u, v)
+    r = mce.enumerate_cliques(g, rank=rank, warp_small_search=True)
+    assert 0 < 400 * r.tasks_split < r.tree_nodes, (r.tasks_split, r.tree_nodes)
+
+
 def test_hold_policy_keeps_results(gpu_lib):
     """With small subtrees kept by the whole warp while any warp waits (the
     hold policy, off by default), and with hand-overs forced often, every
