@@ -71,11 +71,58 @@ __global__ void k_unique_flags(const uint64_t *__restrict__ keys, int64_t k, uin
     if (lane == 0) seg_cnt[seg] = cnt;
 }
 
+//
+// SPARSE (more than twice as many rows as keys): most rows are empty then, and a
+// warp filled the rows of a long gap alone (50 pairs on 3M vertices: ingest 0.49
+// ms, now 0.10; with a key a row, evenly spread, the searches cost 0.03 ms more
+// than short gaps filled by their warps).
+// The row offsets are found by all threads instead, kRowsEach rows each: a binary
+// search for the first key of the first row, from there on for the next rows',
+// and the marked keys before it.
+constexpr int kRowsEach = 8;
+
+// set bits before position p, from the scanned counts of segments of `len` bits
+__device__ __forceinline__ int32_t bits_before(const uint32_t *__restrict__ bits, const int32_t *__restrict__ seg_off,
+                                               int64_t len, int64_t nseg, int64_t p) {
+    const int64_t s = p / len < nseg ? p / len : nseg - 1;
+    int32_t c = seg_off[s];
+    int64_t w = s * len >> 5;
+    for (; w < p >> 5; ++w) c += __popc(bits[w]);
+    return p & 31 ? c + __popc(bits[w] & ((1u << (p & 31)) - 1u)) : c;
+}
+
+template <bool SPARSE>
 __global__ void k_unique_fill(const uint64_t *__restrict__ keys, int64_t k, uint64_t sentinel, int64_t len, int32_t B,
                               int32_t n, const uint32_t *__restrict__ bits, const int32_t *__restrict__ seg_off,
                               int32_t *col, int32_t *row_ptr) {
     const int lane = threadIdx.x & 31;
-    const int64_t seg = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, seg = tid >> 5;
+    if (SPARSE) {
+        const int64_t nseg = (k + len - 1) / len;
+        const int64_t stride = (int64_t)gridDim.x * blockDim.x * kRowsEach;
+        for (int64_t v0 = tid * kRowsEach; v0 <= n; v0 += stride) {
+            int64_t lo = 0, hi = k;   // the row's first key is at lo..hi
+            int32_t at = 0;
+            for (int64_t v = v0; v < v0 + kRowsEach && v <= n; ++v) {
+                const uint64_t first = (uint64_t)v << B;
+                bool moved = v == v0;
+                if (!moved) {
+                    hi = lo;
+                    for (int64_t step = 1; hi < k && keys[hi] < first; step <<= 1) {
+                        lo = hi + 1;
+                        hi = hi + step < k ? hi + step : k;
+                        moved = true;
+                    }
+                }
+                while (lo < hi) {
+                    const int64_t mid = (lo + hi) >> 1;
+                    if (keys[mid] < first) lo = mid + 1; else hi = mid;
+                }
+                if (moved) at = bits_before(bits, seg_off, len, nseg, lo);
+                row_ptr[v] = at;
+            }
+        }
+    }
     const int64_t e0 = seg * len, e1 = e0 + len < k ? e0 + len : k;
     if (e0 >= k) return;
     const uint64_t mask = (1ULL << B) - 1;
@@ -89,6 +136,8 @@ __global__ void k_unique_fill(const uint64_t *__restrict__ keys, int64_t k, uint
         const uint32_t b = bits[c0 >> 5];
         const int32_t at = out + __popc(b & lanemask_lt());
         if ((b >> lane) & 1u) col[at] = (int32_t)(key & mask);
+        out += __popc(b);
+        if (SPARSE) continue;
         // a sentinel counts as row n: the rows behind the last key end here
         const int32_t r = key == sentinel ? n : (int32_t)(key >> B);
         int32_t prev = __shfl_up_sync(0xffffffffu, r, 1);
@@ -103,11 +152,10 @@ __global__ void k_unique_fill(const uint64_t *__restrict__ keys, int64_t k, uint
             const int32_t val = __shfl_sync(0xffffffffu, at, src);
             for (int32_t q = q0 + 1 + lane; q <= q1; q += 32) row_ptr[q] = val;
         }
-        out += __popc(b);
         row = __shfl_sync(0xffffffffu, r, 31);
     }
     // the graph's last key is no sentinel: the rows behind it
-    if (e1 == k && keys[k - 1] != sentinel) {
+    if (!SPARSE && e1 == k && keys[k - 1] != sentinel) {
         const int32_t r = (int32_t)(keys[k - 1] >> B);
         for (int32_t q = r + 1 + lane; q <= n; q += 32) row_ptr[q] = out;
     }
@@ -564,6 +612,9 @@ __global__ void k_scatter_rank(const uint64_t *sorted, int32_t n, int32_t idb, i
 // Bound: L2 (one gather of rank per entry).  A warp per row spent 1.02 ms on
 // the 22M entries of the 1.7M-vertex graph, waiting for the hubs' rows; the
 // two kernels and the scan between them take 0.19 ms.
+// SPARSE (more rows than entries): up_ptr by k_up_fill alone, one row a thread
+// (the warp of a segment would fill long gaps of empty rows by itself: 50 edges
+// on 3M vertices: their triangle counts took 5.4 ms, now 0.29).
 
 // warp: largest r in [0, n) with row_ptr[r] <= e (row_ptr[0] = 0 <= e)
 __device__ __forceinline__ int32_t warp_row_of(const int32_t *row_ptr, int32_t n, int32_t e, int lane) {
@@ -578,6 +629,7 @@ __device__ __forceinline__ int32_t warp_row_of(const int32_t *row_ptr, int32_t n
     return lo;
 }
 
+template <bool SPARSE>
 __global__ void k_up_flags(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
                            const int32_t *__restrict__ rank, int32_t n, int32_t nnz, int32_t len, uint32_t *bits,
                            int32_t *seg_cnt, int32_t *up_ptr) {
@@ -616,26 +668,29 @@ __global__ void k_up_flags(const int32_t *__restrict__ row_ptr, const int32_t *_
         const bool up = valid && rank[w] > rank[r];
         const uint32_t b = __ballot_sync(0xffffffffu, up);
         if (lane == 0) bits[c0 >> 5] = b;
-        int32_t prev = __shfl_up_sync(0xffffffffu, r, 1);
-        if (lane == 0) prev = before;
-        const int32_t at = cnt + __popc(b & lanemask_lt());
-        const bool far = valid && r - prev > 32;   // a long run of empty rows: filled by the whole warp
-        if (valid && !far)
-            for (int32_t q = r; q > prev; --q) up_ptr[q] = at;
-        for (uint32_t m = __ballot_sync(0xffffffffu, far); m; m &= m - 1u) {
-            const int src = __ffs(m) - 1;
-            const int32_t q1 = __shfl_sync(0xffffffffu, r, src), q0 = __shfl_sync(0xffffffffu, prev, src);
-            const int32_t val = __shfl_sync(0xffffffffu, at, src);
-            for (int32_t q = q0 + 1 + lane; q <= q1; q += 32) up_ptr[q] = val;
+        if (!SPARSE) {
+            int32_t prev = __shfl_up_sync(0xffffffffu, r, 1);
+            if (lane == 0) prev = before;
+            const int32_t at = cnt + __popc(b & lanemask_lt());
+            const bool far = valid && r - prev > 32;   // a long run of empty rows: filled by the whole warp
+            if (valid && !far)
+                for (int32_t q = r; q > prev; --q) up_ptr[q] = at;
+            for (uint32_t m = __ballot_sync(0xffffffffu, far); m; m &= m - 1u) {
+                const int src = __ffs(m) - 1;
+                const int32_t q1 = __shfl_sync(0xffffffffu, r, src), q0 = __shfl_sync(0xffffffffu, prev, src);
+                const int32_t val = __shfl_sync(0xffffffffu, at, src);
+                for (int32_t q = q0 + 1 + lane; q <= q1; q += 32) up_ptr[q] = val;
+            }
         }
         cnt += __popc(b);
         row = before = __shfl_sync(0xffffffffu, r, (uint32_t)e1 - c0 > 32u ? 31 : (int)((uint32_t)e1 - c0) - 1);
     }
-    if (e1 == nnz)
+    if (!SPARSE && e1 == nnz)
         for (int32_t q = row + 1 + lane; q <= n; q += 32) up_ptr[q] = cnt;
     if (lane == 0) seg_cnt[seg] = cnt;
 }
 
+template <bool SPARSE>
 __global__ void k_up_fill(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
                           const uint32_t *__restrict__ bits, const int32_t *__restrict__ seg_off, int32_t n,
                           int32_t nnz, int32_t len, int32_t nseg, int32_t *up_ptr, int32_t *up_col) {
@@ -654,6 +709,10 @@ __global__ void k_up_fill(const int32_t *__restrict__ row_ptr, const int32_t *__
     }
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = tid; v <= n; v += stride) {
+        if (SPARSE) {
+            up_ptr[v] = bits_before(bits, seg_off, len, nseg, row_ptr[v]);
+            continue;
+        }
         const int32_t sv = row_ptr[v] / len;
         up_ptr[v] += seg_off[sv < nseg ? sv : nseg - 1];
     }
@@ -719,6 +778,14 @@ mce_status check_csr(const mce_graph *g, cudaStream_t s) {
     return MCE_OK;
 }
 
+// blocks of 256 threads for work on the rows by `threads` threads beside `blocks`
+// for the segments
+static unsigned blocks_for_rows(int64_t threads, unsigned blocks) {
+    const unsigned rows = grid_for(threads, 256), most = (unsigned)num_sms() * 8;
+    const unsigned want = rows < most ? rows : most;
+    return blocks > want ? blocks : want;
+}
+
 mce_status build_csr(const int32_t *u, const int32_t *v, int64_t m, int32_t n, cudaStream_t s, mce_graph *g) {
     g->n = n;
     g->id_bits = bits_for(n > 0 ? (uint64_t)(n - 1) : 0);
@@ -764,8 +831,12 @@ mce_status build_csr(const int32_t *u, const int32_t *v, int64_t m, int32_t n, c
     }
     g->nnz = nnz;
     MCE_TRY(dev_alloc((void **)&g->col, ((size_t)nnz + 4) * sizeof(int32_t), s, "cudaMallocAsync"));
-    MCE_LAUNCH(k_unique_fill, blocks, 256, 0, s, keys.as<uint64_t>(), k, sentinel, len, B, n, bits.as<uint32_t>(),
-               seg.as<int32_t>(), g->col, g->row_ptr);
+    if (n > 2 * k)
+        MCE_LAUNCH(k_unique_fill<true>, blocks_for_rows(n / kRowsEach + 1, blocks), 256, 0, s, keys.as<uint64_t>(), k,
+                   sentinel, len, B, n, bits.as<uint32_t>(), seg.as<int32_t>(), g->col, g->row_ptr);
+    else
+        MCE_LAUNCH(k_unique_fill<false>, blocks, 256, 0, s, keys.as<uint64_t>(), k, sentinel, len, B, n,
+                   bits.as<uint32_t>(), seg.as<int32_t>(), g->col, g->row_ptr);
     return MCE_OK;
 }
 
@@ -907,11 +978,15 @@ mce_status build_up_lists(const mce_graph *g, const int32_t *rank, cudaStream_t 
     MCE_TRY(bits.alloc((size_t)(nnz / 32 + 1) * sizeof(uint32_t), s));
     MCE_TRY(seg.alloc((size_t)(nseg + 1) * sizeof(int32_t), s));
     const unsigned blocks = (unsigned)((nseg + 7) / 8);
-    MCE_LAUNCH(k_up_flags, blocks, 256, 0, s, g->row_ptr, g->col, rank, n, (int32_t)nnz, (int32_t)len,
-               bits.as<uint32_t>(), seg.as<int32_t>(), up_ptr.as<int32_t>());
+    const bool sparse = n > nnz;
+    const auto flags = sparse ? k_up_flags<true> : k_up_flags<false>;
+    const auto fill = sparse ? k_up_fill<true> : k_up_fill<false>;
+    MCE_LAUNCH(flags, blocks, 256, 0, s, g->row_ptr, g->col, rank, n,
+               (int32_t)nnz, (int32_t)len, bits.as<uint32_t>(), seg.as<int32_t>(), up_ptr.as<int32_t>());
     MCE_TRY(exclusive_scan_i32(seg.as<int32_t>(), seg.as<int32_t>(), nseg, s));
-    MCE_LAUNCH(k_up_fill, blocks, 256, 0, s, g->row_ptr, g->col, bits.as<uint32_t>(), seg.as<int32_t>(), n,
-               (int32_t)nnz, (int32_t)len, (int32_t)nseg, up_ptr.as<int32_t>(), up_col.as<int32_t>());
+    MCE_LAUNCH(fill, sparse ? blocks_for_rows((int64_t)n + 1, blocks) : blocks, 256, 0, s,
+               g->row_ptr, g->col, bits.as<uint32_t>(), seg.as<int32_t>(), n, (int32_t)nnz, (int32_t)len,
+               (int32_t)nseg, up_ptr.as<int32_t>(), up_col.as<int32_t>());
     return MCE_OK;
 }
 
