@@ -398,6 +398,8 @@ template <int HP> struct GradSmem {
     static constexpr int part = dT + HP * kRowStride;           // [2][rows]: halves of y
     static constexpr int dy = part + 2 * kGradRows;             // [rows]
     static constexpr int n = dy + kGradRows;
+    // resident blocks an SM: what the shared memory leaves room for
+    static constexpr int blocks = HP <= 16 ? 4 : HP <= 32 ? 2 : 1;
 };
 
 // acc (8 rows as 4 pairs, NC columns) += A^T B over k < K: A[k][row] from
@@ -435,7 +437,7 @@ __device__ __forceinline__ void grad_put(float *col, const f32x2 (&v)[4]) {
 // Forward + backward over rows idx[r0 .. r0 + cnt) (or r0.. when idx is null),
 // loss = (1/N) sum (y - t)^2, hidden width H padded with zero weights to HP.
 // Bound: FP32 multiply-adds (28,000 flops a row).  Persistent blocks, one an
-// SM, take tiles of 256 rows; each layer, forward and backward, is a register-
+// SM (two up to HP = 32, four up to 16), take tiles of 256 rows; each layer, forward and backward, is a register-
 // tiled product (8 rows x HP/8 columns a thread, 32 packed multiply-adds for
 // six 16-byte shared-memory loads at HP = 64), and every weight gradient is
 // summed over the block's rows in registers and added to memory once.  One
@@ -443,7 +445,7 @@ __device__ __forceinline__ void grad_put(float *col, const f32x2 (&v)[4]) {
 // took 6.47 ms for 200,000 rows at H = 64; a call with this kernel takes
 // 0.20 ms, 28 TFLOP/s.
 template <int HP>
-__global__ void __launch_bounds__(kGradRows, 1) k_mlp_grad(const float *__restrict__ wts, int H,
+__global__ void __launch_bounds__(kGradRows, GradSmem<HP>::blocks) k_mlp_grad(const float *__restrict__ wts, int H,
                                                            const float *__restrict__ feat,
                                                            const float *__restrict__ label,
                                                            const int32_t *__restrict__ idx, int64_t r0, int64_t cnt,
@@ -479,6 +481,9 @@ __global__ void __launch_bounds__(kGradRows, 1) k_mlp_grad(const float *__restri
     auto column = [&](int c) { return (c / V) * 8 * V + tc * V + c % V; };
     // W2 gradient entries (tj + 16 a, ti + 16 b)
     const int tj = (warp & 1) * 8 + (lane & 7), ti = (warp >> 1) * 4 + (lane >> 3);
+    // a warp whose columns, or W2 entries, are all padding has none to add up (for
+    // widths of 12 and less)
+    const bool cols = (warp >> 2) * 4 * V < H, entries = (warp & 1) * 8 < H && (warp >> 1) * 4 < H;
     f32x2 gW2[NJ][NJ], gW1[KT];
     float gb1[NC], gb2[NC], gw3[NC], gb3 = 0.f, gl = 0.f;
 #pragma unroll
@@ -505,7 +510,7 @@ __global__ void __launch_bounds__(kGradRows, 1) k_mlp_grad(const float *__restri
 #pragma unroll
             for (int p = 0; p < 4; ++p) acc[p][c] = pack2(b, b);
         }
-        grad_mm<NC, V, HP>(acc, sm + S::xT + tr * 4, sm + S::W1d + 2 * V * tc, kFeat);
+        if (cols) grad_mm<NC, V, HP>(acc, sm + S::xT + tr * 4, sm + S::W1d + 2 * V * tc, kFeat);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             f32x2 v[4];
@@ -521,7 +526,7 @@ __global__ void __launch_bounds__(kGradRows, 1) k_mlp_grad(const float *__restri
 #pragma unroll
             for (int p = 0; p < 4; ++p) acc[p][c] = pack2(b, b);
         }
-        grad_mm<NC, V, HP>(acc, sm + S::h1T + tr * 4, sm + S::W2Td + 2 * V * tc, HP);
+        if (cols) grad_mm<NC, V, HP>(acc, sm + S::h1T + tr * 4, sm + S::W2Td + 2 * V * tc, HP <= 16 ? H : HP);
         {
             float y[8];
 #pragma unroll
@@ -589,7 +594,7 @@ __global__ void __launch_bounds__(kGradRows, 1) k_mlp_grad(const float *__restri
         for (int c = 0; c < NC; ++c)
 #pragma unroll
             for (int p = 0; p < 4; ++p) acc[p][c] = 0ULL;
-        grad_mm<NC, V, HP>(acc, sm + S::dT + tr * 4, sm + S::W2d + 2 * V * tc, HP);
+        if (cols) grad_mm<NC, V, HP>(acc, sm + S::dT + tr * 4, sm + S::W2d + 2 * V * tc, HP <= 16 ? H : HP);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             const float *h = sm + S::h1T + column(c) * kRowStride + tr * 4;
@@ -609,7 +614,7 @@ __global__ void __launch_bounds__(kGradRows, 1) k_mlp_grad(const float *__restri
         }
         // ---- gradient of W2: sum over rows of dh2[j] h1[i], even and odd rows apart
 #pragma unroll 2
-        for (int r = 0; r < kGradRows; r += 4) {
+        for (int r = 0; r < (entries ? kGradRows : 0); r += 4) {
             ulonglong2 dj[NJ], hi[NJ];
 #pragma unroll
             for (int a = 0; a < NJ; ++a) {
@@ -775,7 +780,8 @@ static mce_status grad_launch_hp(const mce_model *m, const float *feat, const fl
     const size_t smem = (size_t)GradSmem<HP>::n * 4;
     MCE_CUDA(cudaFuncSetAttribute(k_mlp_grad<HP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int64_t tiles = (cnt + kGradRows - 1) / kGradRows;
-    const unsigned blocks = (unsigned)(tiles < num_sms() ? tiles : num_sms());
+    const int64_t most = (int64_t)num_sms() * GradSmem<HP>::blocks;
+    const unsigned blocks = (unsigned)(tiles < most ? tiles : most);
     MCE_LAUNCH(k_mlp_grad<HP>, blocks, kGradRows, smem, s, m->w, m->H, feat, label, idx, r0, cnt, inv_n, m->g, loss);
     return MCE_OK;
 }
