@@ -131,6 +131,13 @@ def core_graph(shape):
         w = 10.0 * (np.arange(n) + 1.0) ** -0.6
         hit = rng.random(len(i)) < np.minimum(w[i] * w[j], 1.0)
         return n, i[hit], j[hit]
+    if shape.startswith("dense"):             # 160 entries a vertex or more (peeled), some vertices of few
+        n = 700
+        i, j = np.triu_indices(n, 1)
+        hit = rng.random(len(i)) < 0.6 - 0.2 * (i < n // 2)
+        leaves = int(shape[5:])               # peeled up to a sixteenth of all vertices
+        return n + leaves, np.concatenate([i[hit], rng.integers(0, n, 3 * leaves)]), \
+            np.concatenate([j[hit], np.tile(n + np.arange(leaves), 3)])
     hubs = int(shape[3:])
     n = 3 * hubs + 50                         # three hubs of that degree over a sparse rest, two of them joined
     leaves = np.arange(3, n)
@@ -141,7 +148,7 @@ def core_graph(shape):
 
 
 @pytest.mark.parametrize("shape", ["path", "tree", "cliques", "deg32", "deg33", "deg128", "deg129", "deg384", "deg385",
-                                   "deg1024", "deg1025", "core"])
+                                   "deg1024", "deg1025", "core", "dense0", "dense46", "dense48", "dense200"])
 def test_core_numbers_by_degree_class(gpu_lib, shape):
     """Lanes, warps and blocks a vertex (degrees up to 32, up to 384, above)."""
     mce = gpu_lib
@@ -149,6 +156,24 @@ def test_core_numbers_by_degree_class(gpu_lib, shape):
     og = O.Graph(n, np.asarray(u, np.int32), np.asarray(v, np.int32))
     key = mce.vertex_key(gpu_graph(mce, n, u, v), "degen").cpu().numpy()
     assert np.array_equal(key, O.core_numbers(og).astype(np.int64))
+
+
+def test_core_numbers_of_a_dense_graph_by_peeling(gpu_lib):
+    """G(20000, 0.02): peeled in 1.7 ms; rounds over all of its vertices take 6.5."""
+    import torch
+    mce = gpu_lib
+    n = 20000
+    rng = np.random.default_rng(1)
+    g = gpu_graph(mce, n, rng.integers(0, n, 200 * n), rng.integers(0, n, 200 * n))
+    ms = []
+    for _ in range(6):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        mce.vertex_key(g, "degen")
+        b.record()
+        torch.cuda.synchronize()
+        ms.append(a.elapsed_time(b))
+    assert min(ms) < 4.0, ms
 
 
 @pytest.mark.parametrize("few,many", [(3500, 10000), (300, 120000)])
