@@ -706,6 +706,14 @@ __device__ __forceinline__ int node_weight(int cn, int fn) { return 1 + ((cn + f
 // GB300: 50 us; the 1.7M-vertex graph under the degeneracy rank searched
 // in 36 ms instead of 51 ms (one subproblem alone kept its warp busy for 42 ms).
 constexpr uint64_t BK_SPLIT_NS = 50000;
+// The same in the small search of the whole warp (clique lists,
+// warp_small_search), and then children of wide nodes alone: pieces cut from its
+// small frames every 50 us held 200 nodes (measured on GB300, 50 us and all
+// frames / by the nodes alone / 300 us and wide nodes: clique list of the
+// 1.7M-vertex graph 255 / 85 / 85 ms, R-MAT 14 840 / 84 / 54, 200,000 vertices
+// in pieces of 2^20 words 88 / 123 / 105; with 200 us R-MAT 14 took 57 or 111).
+constexpr uint64_t BK_SPLIT_SMALL_NS = 6 * BK_SPLIT_NS;
+constexpr unsigned long long BK_WIDE_ONLY = 1ULL << 62;   // flag in the hand-overs wanted
 // Longest pause between two looks of a waiting warp at the ring and the
 // counters.  Each look is a handful of loads and an atomic of words that the
 // busy warps need for their hand-overs: with 2,000 warps looking every 16 us
@@ -726,7 +734,8 @@ __device__ __forceinline__ void charge_nodes(const BkParams &P, unsigned long lo
 // Lane 0 reads the control words and credits node counts; the result is
 // broadcast: returns 1 = stop the launch, 2 = drop this task (its graph or
 // subproblem is over budget), 0 = go on with `hungry` = the number of
-// hand-overs wanted (0 = none).  WIDE: asked by the search of wide nodes.
+// hand-overs wanted (0 = none; with BK_WIDE_ONLY of wide nodes' children).
+// WIDE: asked by the search of wide nodes.
 template <bool WIDE>
 __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int32_t root, uint64_t t_start,
                     unsigned long long &hungry_out) {
@@ -768,13 +777,11 @@ __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int3
             // (fewer for a heavy one) or BK_SPLIT_NS: pieces cut too small cost
             // their receivers more than they hold (without the build cache a
             // whole build each: there only the nodes count), but the wide nodes
-            // of a hub's subproblem can take a tenth of a millisecond each.  In the
-            // small search of the whole warp, whose frames are cheap, only the
-            // nodes count: with the time as well a clique list of the 1.7M-vertex
-            // graph took 250 ms, 93 without
-            if (acc.t_nodes - cold().t_split < (heavy && every < 2048ULL ? every : 2048ULL) &&
-                (!WIDE || !P.cache || now - cold().t_split_ns < BK_SPLIT_NS))
-                hungry = 0;
+            // of a hub's subproblem can take a tenth of a millisecond each
+            if (acc.t_nodes - cold().t_split < (heavy && every < 2048ULL ? every : 2048ULL)) {
+                if (!P.cache || now - cold().t_split_ns < (WIDE ? BK_SPLIT_NS : BK_SPLIT_SMALL_NS)) hungry = 0;
+                else if (!WIDE && hungry) hungry |= BK_WIDE_ONLY;
+            }
             // a long-running task spreads its subtree before anybody waits, while
             // less than a piece a warp lies in the ring: pieces are taken before
             // the next subproblems, and up to half a ring of them kept heavy
@@ -1248,10 +1255,12 @@ __device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, u
                 const int code = poll<false>(P, acc, shist, lane, root, t_start, hungry);
                 if (code) return code;
                 if (hungry) {
+                    const bool wide_only = (hungry & BK_WIDE_ONLY) != 0ULL;
+                    hungry &= ~BK_WIDE_ONLY;
                     int budget = hungry > (unsigned long long)acc.give ? acc.give : (int)hungry;
                     // memory frames above the small root first, then small frames
                     if (d > 0) donate_mem(P, s, T, lane, d - 1, d, root, budget);
-                    for (int fd = 0; fd <= ds && budget > 0; ++fd) {
+                    for (int fd = 0; fd <= ds && budget > 0 && !wide_only; ++fd) {
                         const uint32_t *fr = stk + fd * SMALL_FRAME;
                         const uint32_t fe = fd < ds ? fr[2] : ext;
                         if (__popc(fe) < (fd < ds ? 1 : 2)) continue;

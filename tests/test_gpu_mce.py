@@ -759,9 +759,10 @@ def test_sm_limit_covers_the_builds(gpu_lib):
 
 @pytest.mark.parametrize("rank", ["degree", "degen"])
 def test_small_search_of_the_warp_hands_over_by_nodes(gpu_lib, rank):
-    """Clique lists and warp_small_search: a task hands over, up to eight pieces at
-    a time, after 2,048 nodes of its own.  On this graph that makes 650 to 1,100
-    nodes a piece; 210 to 250 when the time since the last hand-over was enough."""
+    """Clique lists and warp_small_search: a task hands over children of small nodes,
+    up to eight pieces at a time, after 2,048 nodes of its own.  On this graph that
+    makes 650 to 1,100 nodes a piece; 210 to 250 when 50 us since the last hand-over
+    were enough."""
     mce = gpu_lib
     n, u, v = rmat(13, seed=8)
     g = gpu_graph(mce, n, u, v)
