@@ -527,11 +527,11 @@ def test_subset_and_subproblem_budget(gpu_lib):
     assert r2.tree_nodes == o2.nodes and r2.incomplete == 0
 
 
-@pytest.mark.parametrize("hub_degree", [1500, 2100, 5000])
+@pytest.mark.parametrize("hub_degree", [130, 511, 512, 513, 1500, 2100, 5000])
 def test_wide_candidate_sets(gpu_lib, hub_degree):
     """A rank that puts a hub lowest gives its subproblem every neighbour as a
-    candidate (more than 1024 here, so frames in memory); the result must
-    not depend on the rank."""
+    candidate (frames in memory for more than 1024; a block's warps share the
+    lists of up to 511 evenly); the result must not depend on the rank."""
     mce = gpu_lib
     rng = np.random.default_rng(hub_degree)
     n = hub_degree + 1
