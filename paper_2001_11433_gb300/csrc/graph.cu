@@ -211,14 +211,14 @@ struct CoreParams {
 };
 
 // Graphs of kPeelDegree or more entries a vertex, nearly all of them of more
-// than kCoreSmall neighbours, are peeled: there the rounds visit every vertex
-// several times, and peeling has few steps.  The degrees are known on the device
-// alone (k_core_init), so both kernels are launched and one returns.  Measured on
-// GB300 (rounds / peeling, ms): G(n, p) with n = 20,000 of degree 64 0.65 / 0.77,
-// 128 1.08 / 0.99, 200 1.5 / 1.2, 400 6.5 / 1.7, 1,500 9.7 / 4.3, n = 100,000 of
-// degree 400 34 / 4.5; R-MAT with as many edges, but vertices of few neighbours:
-// scale 14, 128 edges a vertex 2.0 / 4.9.
-constexpr int64_t kPeelDegree = 160;
+// than kCoreSmall neighbours, are peeled: there the rounds visit every vertex, a
+// hub, several times, and peeling has few steps.  The degrees are known on the
+// device alone (k_core_init), so both kernels are launched and one returns.
+// Measured on GB300 (rounds / peeling, ms): G(n, p) with n = 20,000 of degree 200
+// 1.6 / 1.2, 350 1.2 / 1.6, 400 5.9 / 1.6, 1,500 9.7 / 4.3, n = 100,000 of degree
+// 400 35 / 4.7; bipartite of degree 300 2.1 / 4.0, 600 4.6 / 3.0; R-MAT, which has
+// many vertices of few neighbours, scale 14, 128 edges a vertex 2.0 / 4.9.
+constexpr int64_t kPeelDegree = kCoreMid;
 __device__ __forceinline__ bool core_peeled(int32_t dense, const int32_t *n_small, int32_t n) {
     return dense && (int64_t)*n_small * 16 < n;
 }

@@ -131,8 +131,8 @@ def core_graph(shape):
         w = 10.0 * (np.arange(n) + 1.0) ** -0.6
         hit = rng.random(len(i)) < np.minimum(w[i] * w[j], 1.0)
         return n, i[hit], j[hit]
-    if shape.startswith("dense"):             # 160 entries a vertex or more (peeled), some vertices of few
-        n = 700
+    if shape.startswith("dense"):             # 384 entries a vertex or more (peeled), some vertices of few
+        n = 1100
         i, j = np.triu_indices(n, 1)
         hit = rng.random(len(i)) < 0.6 - 0.2 * (i < n // 2)
         leaves = int(shape[5:])               # peeled up to a sixteenth of all vertices
@@ -148,7 +148,7 @@ def core_graph(shape):
 
 
 @pytest.mark.parametrize("shape", ["path", "tree", "cliques", "deg32", "deg33", "deg128", "deg129", "deg384", "deg385",
-                                   "deg1024", "deg1025", "core", "dense0", "dense46", "dense48", "dense200"])
+                                   "deg1024", "deg1025", "core", "dense0", "dense73", "dense74", "dense200"])
 def test_core_numbers_by_degree_class(gpu_lib, shape):
     """Lanes, warps and blocks a vertex (degrees up to 32, up to 384, above)."""
     mce = gpu_lib
