@@ -153,10 +153,10 @@ LANE_HOLD_WAITING = 0
 # kernel sources they were taken with (profiles/k_bk_rmat18.md): DRAM bytes
 # (read + write) and warp instructions of one-pass captures of the whole
 # timed launch.
-K_BK_COUNTERS = {"dram_bytes": 984_233_216 + 899_319_296, "dram_tree_nodes": 4_057_750_785,
-                 "warp_inst": 95_832_110_570, "inst_tree_nodes": 4_057_750_785,
-                 "sha256": {"bk.cu": "32f53fb462e3b1fa3e9eac500a151b753cb0bbe334b7459c72b48e01db8c831d",
-                            "bk.cuh": "46878bf93e68a8fac1a9fd948adb51137c5b9eebc0eb2775d789126daf185cab"}}
+K_BK_COUNTERS = {"dram_bytes": 331_649_280 + 93_594_624, "dram_tree_nodes": 4_057_750_785,
+                 "warp_inst": 86_823_854_309, "inst_tree_nodes": 4_057_750_785,
+                 "sha256": {"bk.cu": "c42a59058b413e2d7b19e9a601031988695f5ef53012c7a7b304deb5d93e63c4",
+                            "bk.cuh": "12b116721fad7fcc6a7aafd4e47495bc79797d1712c0766674c3ca7dafe8ef93"}}
 
 
 def _same_sources(digests) -> bool:
@@ -178,8 +178,8 @@ def k_bk_traffic(tree_nodes: int):
 def issue_roofline(tree_nodes: int, kernel_s: float, sms: int, sm_mhz: float):
     """Issue-rate roofline of the search kernel: warp instructions per tree
     node (from the one-pass ncu capture of the whole launch) times the tree
-    nodes per second, against 4 schedulers x SMs x clock (one warp
-    instruction per scheduler per clock)."""
+    nodes per second of builds and search, against 4 schedulers x SMs x clock
+    (one warp instruction per scheduler per clock)."""
     if not _same_sources(K_BK_COUNTERS["sha256"]) or kernel_s <= 0:
         return None
     per_node = K_BK_COUNTERS["warp_inst"] / K_BK_COUNTERS["inst_tree_nodes"]
@@ -437,8 +437,8 @@ def run_ours(args):
                               "small_search": "warp" if args.warp_small_search else "lane-parallel",
                               "lane_search_words": args.lane_search_words,
                               "lane_hold_waiting": args.lane_hold_waiting}},
-        "phases_ms": {"rank": res.ms_rank, "enumerate": res.ms_enum, "search_kernel": float(np.mean(search_ms))},
-        "roofline": {"bound": "alu", "kernel": "k_bk (persistent search)", "achieved": achieved, "peak": peak_ops,
+        "phases_ms": {"rank": res.ms_rank, "enumerate": res.ms_enum, "builds_and_search": float(np.mean(search_ms))},
+        "roofline": {"bound": "alu", "kernel": "k_build_rows and k_bk (builds and persistent search)", "achieved": achieved, "peak": peak_ops,
                      "unit": "word-ops/s", "frac": achieved / peak_ops if peak_ops else None,
                      "traffic": k_bk_traffic(res.tree_nodes), "traffic_unit": "DRAM bytes per launch",
                      "peak_source": f"{POPC_PER_CLK_PER_SM} POPC/clk/SM x {props.multi_processor_count} SMs x "
@@ -788,14 +788,17 @@ def train_learned_model(mce):
 def balance_stats(r):
     """Makespan and per-warp busy-time imbalance of one search launch, from
     the kernel's own counters (stats: build ns, search ns, idle ns, builds,
-    pieces, largest busy ns of one warp, warps, endgame ns)."""
+    pieces, largest busy ns of one warp, warps, endgame ns).  build_frac: the
+    share of the builds ahead of the search, which is what the warps' time in
+    the search leaves of the time of both."""
     st = r.stats
     warps = max(st[6], 1)
     mean_busy = (st[0] + st[1]) / warps
+    launch_ms = (st[0] + st[1] + st[2]) / warps / 1e6
     return {"search_ms": r.ms_search, "max_warp_busy_ms": st[5] / 1e6, "mean_warp_busy_ms": mean_busy / 1e6,
             "imbalance": st[5] / mean_busy if mean_busy else None, "idle_frac": st[2] / max(st[0] + st[1] + st[2], 1),
             "endgame_ms": st[7] / 1e6, "pieces": st[4], "builds": st[3],
-            "build_frac": st[0] / max(st[0] + st[1], 1)}
+            "build_frac": max(0.0, 1.0 - launch_ms / r.ms_search) if r.ms_search else 0.0}
 
 
 def measure_ranks(mce, steps=3, warmup=1, kinds=("degree", "degen", "triangle", "learned", "learned_split")):

@@ -180,7 +180,7 @@ __global__ void k_degree_key(const int32_t *row_ptr, int32_t n, int64_t *key) {
 // the latency of a round (one hub's visit and the barrier), of which graphs
 // whose hubs fall one step after the other take hundreds.  Peeling level by
 // level (three barriers per removal step, each removed hub's row walked by one
-// warp) took 42.1 ms on the 1.7M-vertex graph (750 rounds here) and 9.3 ms on
+// warp) took 42.1 ms on the 1.7M-vertex graph (340 rounds here) and 9.3 ms on
 // R-MAT 18; this kernel: 13.6 ms and 3.8 ms.
 //
 // stamp[v] = round in which v is to be visited.  Lists by degree: [0] 2..32

@@ -128,8 +128,9 @@ __device__ __forceinline__ float feature(const FeatParams &P, int64_t v, int32_t
 }
 
 // Eight lanes a vertex, one feature a lane at the end; vertices of more than
-// kFeatHub neighbours are left to k_features_hubs, a block each.  Bound: L2
-// (two gathers a neighbour).  A warp per vertex left most lanes of short rows
+// kFeatHub neighbours are left to k_features_hubs, a block each.  Bound:
+// instructions (57 % of their throughput at 400,000 vertices) and the latency of
+// two gathers a neighbour through L1 and L2.  A warp per vertex left most lanes of short rows
 // idle and took 0.99 ms on the 1.7M-vertex graph, waiting for the hubs; both
 // kernels together take 0.31 ms.
 constexpr int kFeatHub = 512;
@@ -271,8 +272,8 @@ __device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], u
 
 // BF16 inference (BF16 weights, biases and activations, FP32 sums), hidden
 // width H padded with zero weights to HP, a warp per 16 rows at a time.
-// Bound: HBM (36 B a row), with the instructions around the products close
-// behind.  Both layers run on warp-level matrix instructions because their
+// Bound: latency (12 warps an SM, as the weights fill their registers; at
+// 400,000 rows a quarter of the issue slots, 0.5 TB/s).  Both layers run on warp-level matrix instructions because their
 // accumulator fragments, rounded to BF16, are the next layer's operand
 // fragments as they stand: the activations never leave registers, where a
 // TMEM accumulator would be read back and staged again for an 8-deep and a
@@ -436,11 +437,13 @@ __device__ __forceinline__ void grad_put(float *col, const f32x2 (&v)[4]) {
 
 // Forward + backward over rows idx[r0 .. r0 + cnt) (or r0.. when idx is null),
 // loss = (1/N) sum (y - t)^2, hidden width H padded with zero weights to HP.
-// Bound: FP32 multiply-adds (28,000 flops a row).  Persistent blocks, one an
-// SM (two up to HP = 32, four up to 16), take tiles of 256 rows; each layer, forward and backward, is a register-
-// tiled product (8 rows x HP/8 columns a thread, 32 packed multiply-adds for
-// six 16-byte shared-memory loads at HP = 64), and every weight gradient is
-// summed over the block's rows in registers and added to memory once.  One
+// Bound: shared-memory reads (71 % of their throughput at 200,000 rows, H = 64)
+// for FP32 multiply-adds (28,000 flops a row; 45 % of the instruction slots).
+// Persistent blocks, one an SM (two up to HP = 32, four up to 16), take tiles of
+// 256 rows; each layer, forward and backward, is a register-tiled product (8 rows
+// x HP/8 columns a thread, 32 packed multiply-adds for six 16-byte shared-memory
+// loads at HP = 64), and every weight gradient is summed over the block's rows in
+// registers and added to memory once.  One
 // thread per row with serial dot products (columns of one row in one bank)
 // took 6.47 ms for 200,000 rows at H = 64; a call with this kernel takes
 // 0.20 ms, 28 TFLOP/s.
