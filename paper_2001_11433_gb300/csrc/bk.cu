@@ -810,7 +810,7 @@ __device__ int poll(const BkParams &P, Acc &acc, uint32_t *shist, int lane, int3
     if (ab & 3ULL) return 1;
     if (ab & 16ULL) return 2;
     if (hungry && lane == 0) {
-        cold().t_split = acc.t_nodes;
+        if (!(hungry & BK_WIDE_ONLY)) cold().t_split = acc.t_nodes;   // else once a piece has been cut
         cold().t_split_ns = globaltimer_ns();
     }
     return 0;
@@ -1257,9 +1257,11 @@ __device__ int search_small(const BkParams &P, Ws &s, const Task &T, Acc &acc, u
                 if (hungry) {
                     const bool wide_only = (hungry & BK_WIDE_ONLY) != 0ULL;
                     hungry &= ~BK_WIDE_ONLY;
-                    int budget = hungry > (unsigned long long)acc.give ? acc.give : (int)hungry;
+                    const int most = hungry > (unsigned long long)acc.give ? acc.give : (int)hungry;
+                    int budget = most;
                     // memory frames above the small root first, then small frames
                     if (d > 0) donate_mem(P, s, T, lane, d - 1, d, root, budget);
+                    if (wide_only && budget < most && lane == 0) cold().t_split = acc.t_nodes;
                     for (int fd = 0; fd <= ds && budget > 0 && !wide_only; ++fd) {
                         const uint32_t *fr = stk + fd * SMALL_FRAME;
                         const uint32_t fe = fd < ds ? fr[2] : ext;

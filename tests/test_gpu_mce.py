@@ -770,6 +770,19 @@ def test_small_search_of_the_warp_hands_over_by_nodes(gpu_lib, rank):
     assert 0 < 400 * r.tasks_split < r.tree_nodes, (r.tasks_split, r.tree_nodes)
 
 
+@pytest.mark.parametrize("size,k", [(3, 12), (2, 18)])
+def test_small_search_without_wide_nodes_still_hands_over(gpu_lib, size, k):
+    """Complete multipartite graphs of up to 36 vertices: one tree of half a million
+    cliques in small frames alone, which has to reach more than a few warps."""
+    mce = gpu_lib
+    n = size * k
+    i, j = np.triu_indices(n, 1)
+    keep = i // size != j // size
+    r = mce.enumerate_cliques(gpu_graph(mce, n, i[keep], j[keep]), warp_small_search=True)
+    assert r.count == size ** k
+    assert r.tasks_split >= 100, r.tasks_split
+
+
 def test_hold_policy_keeps_results(gpu_lib):
     """With small subtrees kept by the whole warp while any warp waits (the
     hold policy, off by default), and with hand-overs forced often, every
