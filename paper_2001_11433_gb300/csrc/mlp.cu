@@ -94,7 +94,6 @@ struct FeatParams {
     const int64_t *core, *tri;   // MCE_FEATURES_FULL
     const int32_t *up_ptr;       //
     int32_t n;
-    int32_t *hubs, *n_hubs;
     float *feat;
 };
 
@@ -128,17 +127,53 @@ __device__ __forceinline__ float feature(const FeatParams &P, int64_t v, int32_t
 }
 
 // Eight lanes a vertex, one feature a lane at the end; vertices of more than
-// kFeatHub neighbours are left to k_features_hubs, a block each.  Bound:
-// instructions (57 % of their throughput at 400,000 vertices) and the latency of
-// two gathers a neighbour through L1 and L2.  A warp per vertex left most lanes of short rows
-// idle and took 0.99 ms on the 1.7M-vertex graph, waiting for the hubs; both
-// kernels together take 0.31 ms.
+// kFeatHub neighbours by a block each, before the others: block b of an odd number
+// looks for them among b, b + blocks, b + 2 blocks, ..., so that hubs with close
+// ids, or ids a power of two apart as in R-MAT graphs, are spread over the blocks.
+// Bound: instructions (57 % of their throughput at 400,000 vertices) and the
+// latency of two gathers a neighbour through L1 and L2.  A warp per vertex left
+// most lanes of short rows idle and took 0.99 ms on the 1.7M-vertex graph, waiting
+// for the hubs; a call with this takes 0.29 ms.  (A list of the hubs in memory for
+// a second kernel made that 0.36 ms, and a call on a few thousand vertices 9 us
+// longer.)
 constexpr int kFeatHub = 512;
+constexpr int kFeatThreads = 256, kFeatWarps = kFeatThreads / 32;
 
-template <bool LIGHT> __global__ void k_features(FeatParams P) {
-    const int lane = threadIdx.x & 31, k = lane & 7;
-    const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-    const int64_t stride = ((int64_t)gridDim.x * blockDim.x) >> 3;
+template <bool LIGHT> __global__ void __launch_bounds__(kFeatThreads) k_features(FeatParams P) {
+    __shared__ __align__(8) unsigned char raw[kFeatWarps * sizeof(NbrSums)];
+    __shared__ int32_t hubs[kFeatThreads], n_hubs;
+    NbrSums *part = reinterpret_cast<NbrSums *>(raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = lane & 7;
+    const int64_t looking = gridDim.x - ((gridDim.x & 1u) ? 0 : 1);
+    // the same number of rounds for every thread of the block
+    for (int64_t v0 = blockIdx.x < looking ? blockIdx.x : P.n; v0 < P.n; v0 += looking * kFeatThreads) {
+        if (threadIdx.x == 0) n_hubs = 0;
+        __syncthreads();
+        const int64_t mine = v0 + threadIdx.x * looking;
+        if (mine < P.n && P.row_ptr[mine + 1] - P.row_ptr[mine] > kFeatHub)
+            hubs[atomicAdd(&n_hubs, 1)] = (int32_t)mine;
+        __syncthreads();
+        const int nh = n_hubs;
+        for (int h = 0; h < nh; ++h) {
+            const int32_t v = hubs[h];
+            const int32_t e0 = P.row_ptr[v], d = P.row_ptr[v + 1] - e0;
+            NbrSums a;
+#pragma unroll 8
+            for (int32_t e = threadIdx.x; e < d; e += kFeatThreads) a.add<LIGHT>(P.row_ptr, P.col[e0 + e], v, d);
+            __syncwarp();
+            a.reduce<LIGHT>(16);
+            if (lane == 0) part[warp] = a;
+            __syncthreads();
+            if (warp == 0) {
+                a = lane < kFeatWarps ? part[lane] : NbrSums();
+                a.reduce<LIGHT>(kFeatWarps / 2);
+                if (lane < kFeat) P.feat[(int64_t)v * kFeat + lane] = feature<LIGHT>(P, v, d, a, lane);
+            }
+            __syncthreads();
+        }
+    }
+    const int64_t g0 = ((int64_t)blockIdx.x * kFeatThreads + threadIdx.x) >> 3;
+    const int64_t stride = ((int64_t)gridDim.x * kFeatThreads) >> 3;
     for (int64_t w0 = g0 - (lane >> 3); w0 < P.n; w0 += stride) {   // the same for the whole warp
         const int64_t v = w0 + (lane >> 3);
         int32_t e0 = 0, d = 0;
@@ -151,36 +186,10 @@ template <bool LIGHT> __global__ void k_features(FeatParams P) {
         if (!hub) {
 #pragma unroll 4
             for (int32_t e = k; e < d; e += 8) a.add<LIGHT>(P.row_ptr, P.col[e0 + e], (int32_t)v, d);
-        } else if (k == 0) {
-            P.hubs[atomicAdd(P.n_hubs, 1)] = (int32_t)v;
         }
         __syncwarp();
         a.reduce<LIGHT>(4);
         if (v < P.n && !hub) P.feat[v * kFeat + k] = feature<LIGHT>(P, v, d, a, k);
-    }
-}
-
-template <bool LIGHT> __global__ void __launch_bounds__(512) k_features_hubs(FeatParams P) {
-    __shared__ __align__(8) unsigned char raw[16 * sizeof(NbrSums)];
-    NbrSums *part = reinterpret_cast<NbrSums *>(raw);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int32_t n_hubs = *P.n_hubs;
-    for (int32_t i = blockIdx.x; i < n_hubs; i += gridDim.x) {
-        const int32_t v = P.hubs[i];
-        const int32_t e0 = P.row_ptr[v], d = P.row_ptr[v + 1] - e0;
-        NbrSums a;
-#pragma unroll 4
-        for (int32_t e = threadIdx.x; e < d; e += 512) a.add<LIGHT>(P.row_ptr, P.col[e0 + e], v, d);
-        __syncwarp();
-        a.reduce<LIGHT>(16);
-        if (lane == 0) part[warp] = a;
-        __syncthreads();
-        if (warp == 0) {
-            a = lane < 16 ? part[lane] : NbrSums();
-            a.reduce<LIGHT>(8);
-            if (lane < kFeat) P.feat[(int64_t)v * kFeat + lane] = feature<LIGHT>(P, v, d, a, lane);
-        }
-        __syncthreads();
     }
 }
 
@@ -727,16 +736,9 @@ mce_status features(const mce_graph *g, int32_t kind, cudaStream_t s, float *fea
     P.col = g->col;
     P.n = n;
     P.feat = feat;
-    const int64_t max_hubs = g->nnz / kFeatHub;
-    DevBuf hubs, core, tri, deg, drank, up_ptr, up_col;
-    MCE_TRY(hubs.alloc((size_t)(max_hubs + 1) * 4, s));
-    MCE_CUDA(cudaMemsetAsync(hubs.p, 0, 4, s));
-    P.n_hubs = hubs.as<int32_t>();
-    P.hubs = P.n_hubs + 1;
-    const unsigned hub_blocks = (unsigned)(max_hubs < 2 * num_sms() ? max_hubs : 2 * num_sms());
+    DevBuf core, tri, deg, drank, up_ptr, up_col;
     if (kind == MCE_FEATURES_LIGHT) {
-        MCE_LAUNCH(k_features<true>, grid_for((int64_t)n * 8, 256), 256, 0, s, P);
-        if (hub_blocks) MCE_LAUNCH(k_features_hubs<true>, hub_blocks, 512, 0, s, P);
+        MCE_LAUNCH(k_features<true>, grid_for((int64_t)n * 8, kFeatThreads), kFeatThreads, 0, s, P);
         return MCE_OK;
     }
     MCE_TRY(core.alloc((size_t)n * 8, s));
@@ -752,8 +754,7 @@ mce_status features(const mce_graph *g, int32_t kind, cudaStream_t s, float *fea
     P.core = core.as<int64_t>();
     P.tri = tri.as<int64_t>();
     P.up_ptr = up_ptr.as<int32_t>();
-    MCE_LAUNCH(k_features<false>, grid_for((int64_t)n * 8, 256), 256, 0, s, P);
-    if (hub_blocks) MCE_LAUNCH(k_features_hubs<false>, hub_blocks, 512, 0, s, P);
+    MCE_LAUNCH(k_features<false>, grid_for((int64_t)n * 8, kFeatThreads), kFeatThreads, 0, s, P);
     return MCE_OK;
 }
 

@@ -59,6 +59,20 @@ def test_light_features_match_reference(gpu_lib, case):
     assert np.allclose(F, R, rtol=1e-4, atol=2e-3)
 
 
+@pytest.mark.parametrize("n", [33, 600, 70000, 400001])
+def test_light_features_of_hubs(gpu_lib, n):
+    """Rows on both sides of 512 neighbours, hubs 4,096 ids apart, one block and many."""
+    mce = gpu_lib
+    rng = np.random.default_rng(n)
+    hubs = np.arange(0, n, 4096)[:12]
+    deg = np.minimum(n - 1, np.array([n - 1, 511, 512, 513, 514, 700, 1023, 1025, 2047, 5000, 8193, 20000])[:len(hubs)])
+    u = np.concatenate([np.repeat(hubs, deg), rng.integers(0, n, 2 * n)])
+    v = np.concatenate([rng.choice(n, d, replace=False) for d in deg] + [rng.integers(0, n, 2 * n)])
+    F = mce.features(mce.Graph(n, _t(u), _t(v)), kind="light").cpu().numpy()
+    R = mlp.features_light(O.Graph(n, u.astype(np.int32), v.astype(np.int32)))
+    assert np.allclose(F, R, rtol=1e-4, atol=2e-3)
+
+
 def test_loss_and_gradient_match_reference(gpu_lib):
     """FP32 GPU gradient within 1e-4 of the float64 reference (relative to the
     largest gradient component)."""
