@@ -207,21 +207,27 @@ struct CoreParams {
     // hub i of list[2]: neighbours with val >= keep_from[i] at kept[keep_at[i]
     // .. + keep_n[i]) (keep_from 0: none kept yet)
     int32_t *keep_from, *keep_at, *keep_n, *kept;
-    int32_t dense;            // the graph may be left to k_core_peel
+    int32_t dense, large;     // the graph may be left to k_core_peel (core_leave)
 };
 
-// Graphs of kPeelDegree or more entries a vertex, nearly all of them of more
-// than kCoreSmall neighbours, are peeled: there the rounds visit every vertex, a
-// hub, several times, and peeling has few steps.  The degrees are known on the
-// device alone (k_core_init), so both kernels are launched and one returns.
-// Measured on GB300 (rounds / peeling, ms): G(n, p) with n = 20,000 of degree 200
+// Graphs that k_core_rounds leaves to k_core_peel, which is launched behind it for
+// those that may be, and returns at once for the others (ctl[kCorePeeled]).
+// Dense ones, of kPeelDegree or more entries a vertex, nearly all of them of more
+
+// than kCoreSmall neighbours: there the rounds visit every vertex, a hub, several
+// times, and peeling has few steps; the degrees are known on the device alone
+// (k_core_init).  Measured on GB300 (rounds / peeling, ms): G(n, p) with n = 20,000 of degree 200
 // 1.6 / 1.2, 350 1.2 / 1.6, 400 5.9 / 1.6, 1,500 9.7 / 4.3, n = 100,000 of degree
 // 400 35 / 4.7; bipartite of degree 300 2.1 / 4.0, 600 4.6 / 3.0; R-MAT, which has
 // many vertices of few neighbours, scale 14, 128 edges a vertex 2.0 / 4.9.
+// Large ones, of kPeelVertices or more, after kPeelRounds rounds in a row that
+// visited vertices of up to kCoreSmall neighbours alone: chains that fall from
+// their ends for thousands of rounds, each of which looks at every stamp (grid of
+// 1,000 x 1,000 vertices 17.5 ms by rounds alone, path of a million 4,624; peeled
+// 7.9 and 2,649).
 constexpr int64_t kPeelDegree = kCoreMid;
-__device__ __forceinline__ bool core_peeled(int32_t dense, const int32_t *n_small, int32_t n) {
-    return dense && (int64_t)*n_small * 16 < n;
-}
+constexpr int32_t kPeelVertices = 1 << 18, kPeelRounds = 64;
+constexpr int kCorePeeled = 15;
 
 __device__ __forceinline__ int core_class(int32_t d) { return d <= kCoreSmall ? 0 : d <= kCoreMid ? 1 : 2; }
 
@@ -441,7 +447,11 @@ __device__ __forceinline__ uint32_t core_mid(const CoreParams &P, int32_t v, int
 }
 
 __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
-    if (core_peeled(P.dense, P.ctl, P.n)) return;
+    if (P.dense && (int64_t)P.ctl[0] * 16 < P.n) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) P.ctl[kCorePeeled] = 1;
+        return;
+    }
+    int32_t chains = 0;   // rounds in a row that visited the first list alone
     cg::grid_group grid = cg::this_grid();
     extern __shared__ int32_t core_bins[];   // kHubBins a group
     __shared__ HubShared hub[kHubGroups];
@@ -548,11 +558,16 @@ __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) visit |= __ldcg(P.ctl + 4 + 3 * k + (round + 1) % 3) ? 1u << k : 0u;
         if (!visit) break;
+        chains = visit == 1u ? chains + 1 : 0;
+        if (P.large && chains == kPeelRounds) {   // the same for all threads of the grid
+            if (blockIdx.x == 0 && threadIdx.x == 0) P.ctl[kCorePeeled] = 1;
+            break;
+        }
     }
 }
 
-// Core numbers by level-synchronous peeling on a cooperative grid, for dense
-// graphs (core_peeled).  Level k:
+// Core numbers by level-synchronous peeling on a cooperative grid, for the graphs
+// that k_core_rounds left (*left).  Level k:
 // every alive vertex whose remaining degree is <= k is removed with core
 // number k; removing a vertex decrements its alive neighbours, and those that
 // fall to <= k are removed at the same level (claimed once by CAS).
@@ -566,25 +581,20 @@ __global__ void __launch_bounds__(kCoreThreads, 1) k_core_rounds(CoreParams P) {
 // remaining degree (one slot per level parity).
 // Every read of a control word is followed by a grid barrier before any
 // thread may change that word, so all threads take the same branches.
-__global__ void k_peel_init(const int32_t *row_ptr, int32_t n, int32_t *d, int32_t *core, int32_t *alive,
-                            int32_t *ctl) {
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (int64_t v = tid; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        d[v] = row_ptr[v + 1] - row_ptr[v];
-        core[v] = -1;
-        alive[v] = (int32_t)v;
-    }
-    // all alive, no remaining degree seen yet
-    if (tid < 8) ctl[tid] = tid == 3 ? n : tid == 5 || tid == 6 ? 0x7fffffff : 0;
-}
-
 __global__ void k_core_peel(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col, int32_t n,
                             int32_t *d, int32_t *core, int32_t *fa, int32_t *fb, int32_t *la, int32_t *lb,
-                            int32_t *ctl, const int32_t *n_small) {
-    if (!core_peeled(1, n_small, n)) return;
+                            int32_t *ctl, const int32_t *left) {
+    if (!*left) return;
     cg::grid_group grid = cg::this_grid();
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nth = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t v = tid; v < n; v += nth) {
+        d[v] = row_ptr[v + 1] - row_ptr[v];
+        core[v] = -1;
+        la[v] = (int32_t)v;
+    }
+    // all alive, no remaining degree seen yet
+    if (tid < 8) ctl[tid] = tid == 3 ? n : tid == 5 || tid == 6 ? 0x7fffffff : 0;
     const int lane = threadIdx.x & 31;
     const int64_t wid = tid >> 5, nwarp = nth >> 5;
     int32_t *cur = fa, *nxt = fb, *alive = la, *alive2 = lb;
@@ -666,7 +676,7 @@ __global__ void k_core_peel(const int32_t *__restrict__ row_ptr, const int32_t *
 }
 
 __global__ void k_core_key(CoreParams P, const int32_t *peeled, int64_t *key) {
-    const int32_t *core = core_peeled(P.dense, P.ctl, P.n) ? peeled : P.val;
+    const int32_t *core = peeled && P.ctl[kCorePeeled] ? peeled : P.val;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < P.n; v += (int64_t)gridDim.x * blockDim.x)
         key[v] = core[v];
 }
@@ -970,12 +980,11 @@ mce_status build_csr(const int32_t *u, const int32_t *v, int64_t m, int32_t n, c
     return MCE_OK;
 }
 
-// core numbers of a dense graph into `core` (first n of it), if core_peeled says so
+// core numbers into `core` (first n of it) if k_core_rounds left the graph
 static mce_status core_by_peeling(const mce_graph *g, const CoreParams &P, DevBuf &core, cudaStream_t s) {
     int32_t n = g->n;
     MCE_TRY(core.alloc(((size_t)n * 6 + 8) * sizeof(int32_t), s));
     int32_t *c = core.as<int32_t>(), *d = c + n, *fa = d + n, *fb = fa + n, *la = fb + n, *lb = la + n, *ctl = lb + n;
-    MCE_LAUNCH(k_peel_init, grid_for(n, 256), 256, 0, s, g->row_ptr, n, d, c, la, ctl);
     int per_sm = 0;
     MCE_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_core_peel, 256, 0));
     if (per_sm < 1) {
@@ -984,9 +993,9 @@ static mce_status core_by_peeling(const mce_graph *g, const CoreParams &P, DevBu
     }
     // few blocks: the many grid barriers cost in proportion to the blocks
     const unsigned blocks = (unsigned)(num_sms() * (per_sm < 2 ? per_sm : 2));
-    const int32_t *rp = g->row_ptr, *cl = g->col, *small = P.ctl;
+    const int32_t *rp = g->row_ptr, *cl = g->col, *left = P.ctl + kCorePeeled;
     void *args[] = {(void *)&rp, (void *)&cl, (void *)&n,  (void *)&d,   (void *)&c,    (void *)&fa,
-                    (void *)&fb, (void *)&la, (void *)&lb, (void *)&ctl, (void *)&small};
+                    (void *)&fb, (void *)&la, (void *)&lb, (void *)&ctl, (void *)&left};
     g_launches.fetch_add(1, std::memory_order_relaxed);
     MCE_CUDA(cudaLaunchCooperativeKernel((const void *)k_core_peel, dim3(blocks), dim3(256), args, 0, s));
     return MCE_OK;
@@ -1017,8 +1026,8 @@ static mce_status core_numbers(const mce_graph *g, cudaStream_t s, int64_t *key)
     P.keep_n = P.keep_at + hubs;
     P.kept = kept.as<int32_t>();
     P.dense = g->nnz >= kPeelDegree * n;
+    P.large = n >= kPeelVertices;
     MCE_LAUNCH(k_core_init, grid_for(n, 256), 256, 0, s, P);
-    if (P.dense) MCE_TRY(core_by_peeling(g, P, peeled, s));
     static std::once_flag once;
     static cudaError_t granted;
     std::call_once(once, [] {
@@ -1039,6 +1048,7 @@ static mce_status core_numbers(const mce_graph *g, cudaStream_t s, int64_t *key)
     g_launches.fetch_add(1, std::memory_order_relaxed);
     MCE_CUDA(cudaLaunchCooperativeKernel((const void *)k_core_rounds, dim3(blocks), dim3(kCoreThreads), args, kCoreSmem,
                                          s));
+    if (P.dense || P.large) MCE_TRY(core_by_peeling(g, P, peeled, s));
     MCE_LAUNCH(k_core_key, grid_for(n, 256), 256, 0, s, P, peeled.as<int32_t>(), key);
     return MCE_OK;
 }

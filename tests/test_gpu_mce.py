@@ -158,6 +158,28 @@ def test_core_numbers_by_degree_class(gpu_lib, shape):
     assert np.array_equal(key, O.core_numbers(og).astype(np.int64))
 
 
+@pytest.mark.parametrize("shape", ["path", "grid", "clique"])
+def test_core_numbers_of_long_chains(gpu_lib, shape):
+    """Large graphs whose values fall from the ends of chains for thousands of rounds
+    are handed to the peeling: a path, a grid, a path that ends in K_40."""
+    mce = gpu_lib
+    if shape == "grid":
+        k = np.arange(520 * 520).reshape(520, 520)
+        n, u, v = k.size, np.concatenate([k[:, :-1].ravel(), k[:-1].ravel()]), \
+            np.concatenate([k[:, 1:].ravel(), k[1:].ravel()])
+        want = np.full(n, 2)
+    else:
+        n = 1 << 18
+        u, v = np.arange(n - 1), np.arange(1, n)
+        want = np.ones(n)
+        if shape == "clique":
+            i, j = np.triu_indices(40, 1)
+            u, v = np.concatenate([u, i]), np.concatenate([v, j])
+            want[:40] = 39
+    key = mce.vertex_key(gpu_graph(mce, n, u, v), "degen").cpu().numpy()
+    assert np.array_equal(key, want.astype(np.int64))
+
+
 def test_core_numbers_of_a_dense_graph_by_peeling(gpu_lib):
     """G(20000, 0.02): peeled in 1.7 ms; rounds over all of its vertices take 6.5."""
     import torch
