@@ -153,9 +153,9 @@ LANE_HOLD_WAITING = 0
 # kernel sources they were taken with (profiles/k_bk_rmat18.md): DRAM bytes
 # (read + write) and warp instructions of one-pass captures of the whole
 # timed launch.
-K_BK_COUNTERS = {"dram_bytes": 331_649_280 + 93_594_624, "dram_tree_nodes": 4_057_750_785,
-                 "warp_inst": 86_823_854_309, "inst_tree_nodes": 4_057_750_785,
-                 "sha256": {"bk.cu": "c42a59058b413e2d7b19e9a601031988695f5ef53012c7a7b304deb5d93e63c4",
+K_BK_COUNTERS = {"dram_bytes": 330_905_088 + 93_160_192, "dram_tree_nodes": 4_057_750_785,
+                 "warp_inst": 86_961_169_695, "inst_tree_nodes": 4_057_750_785,
+                 "sha256": {"bk.cu": "c45261b3ed23f78599b141e1149b211f4ab1e50c95856227def7547affffa2db",
                             "bk.cuh": "12b116721fad7fcc6a7aafd4e47495bc79797d1712c0766674c3ca7dafe8ef93"}}
 
 

@@ -710,8 +710,8 @@ constexpr uint64_t BK_SPLIT_NS = 50000;
 // warp_small_search), and then children of wide nodes alone: pieces cut from its
 // small frames every 50 us held 200 nodes (measured on GB300, 50 us and all
 // frames / by the nodes alone / 300 us and wide nodes: clique list of the
-// 1.7M-vertex graph 255 / 85 / 85 ms, R-MAT 14 840 / 84 / 54, 200,000 vertices
-// in pieces of 2^20 words 88 / 123 / 105; with 200 us R-MAT 14 took 57 or 111).
+// 1.7M-vertex graph 255 / 85 / 85 ms, R-MAT 14 840 / 84 / 70 to 97, R-MAT 13 74 /
+// 17 / 13, 200,000 vertices in pieces of 2^20 words 88 / 123 / 106).
 constexpr uint64_t BK_SPLIT_SMALL_NS = 6 * BK_SPLIT_NS;
 constexpr unsigned long long BK_WIDE_ONLY = 1ULL << 62;   // flag in the hand-overs wanted
 // Longest pause between two looks of a waiting warp at the ring and the

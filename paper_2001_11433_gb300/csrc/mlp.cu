@@ -130,7 +130,7 @@ __device__ __forceinline__ float feature(const FeatParams &P, int64_t v, int32_t
 // kFeatHub neighbours by a block each, before the others: block b of an odd number
 // looks for them among b, b + blocks, b + 2 blocks, ..., so that hubs with close
 // ids, or ids a power of two apart as in R-MAT graphs, are spread over the blocks.
-// Bound: instructions (57 % of their throughput at 400,000 vertices) and the
+// Bound: instructions (54 % of their throughput at 400,000 vertices) and the
 // latency of two gathers a neighbour through L1 and L2.  A warp per vertex left
 // most lanes of short rows idle and took 0.99 ms on the 1.7M-vertex graph, waiting
 // for the hubs; a call with this takes 0.29 ms.  (A list of the hubs in memory for
